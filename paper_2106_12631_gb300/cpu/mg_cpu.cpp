@@ -70,9 +70,11 @@ template <class T, int W> inline Lane<T, W> fmac(Lane<T, W> a, Lane<T, W> b, Lan
 }
 
 template <class R>
-struct SlotArray {  // the current / amputated-current slots of one block
+struct SlotArray {  // the current / amputated-current slots of one block, and the scalars beside them
   mg::W4<R>* p;
+  mg::cx<R>* sc = nullptr;
   mg::W4<R> operator[](int i) const { return p[i]; }
+  mg::cx<R> scalar(int i) const { return sc[i]; }
 };
 
 template <class P>
@@ -118,6 +120,54 @@ inline void xitem(const mg::HsItem& it, const mg::W4<R>* cur, mg::W4<R>* xb, con
   xb[it.out] = o;
 }
 
+// items of the ordered program (as the GPU's ord_item and ord_xitem)
+template <class P, class R>
+inline void ord_item(const mg::HsItem& it, mg::W4<R>* cur, mg::W4<R>* xb, mg::cx<R>* sc, const R* K,
+                     const mg::cx<R>* pr, const mg::Couplings<R>& cp) {
+  using namespace mg;
+  const R one(1.0);
+  switch (it.type) {
+    case 15: cur[it.out] = FFV1_2<R>(cur[it.in[0]], cur[it.in[1]], one, K + 4 * it.k0, cp.mt, pr[it.prop]); return;
+    case 16: cur[it.out] = FFV1_1<R>(cur[it.in[0]], cur[it.in[1]], one, K + 4 * it.k0, cp.mt, pr[it.prop]); return;
+    case 17: cur[it.out] = w4_rscale(ord_pair(cur[it.in[0]], cur[it.in[1]]), -pr[it.prop].im); return;
+    case 18:
+      cur[it.out] = w4_rscale(ord_v3(cur[it.in[0]], cur[it.in[1]], K + 4 * it.k0, K + 4 * it.k1), pr[it.prop].im);
+      return;
+    case 19:
+    case 20:
+    case 21: {
+      const HsItemExt& ext = P::hs_item_ext()[it.in3()];
+      W4<R>&o = xb[it.out], &o2 = xb[it.out + HS_WORD];
+      if (it.type == 21) {
+        ord_g3(cur[it.in[0]], cur[it.in[1]], cur[it.in[2]], cur[ext.in[0]], cur[ext.in[1]], cur[ext.in[2]], K, ext.k,
+               pr[it.prop].im, o, o2);
+      } else if (it.type == 19) {
+        const W4<R> c = row_slash(cur[it.in[2]], cur[ext.in[2]]);
+        const cx<R> s = mul_i(pr[it.prop]);
+        o = scale(row_kslash_m(w4_add(row_slash(cur[it.in[0]], cur[it.in[1]]), c), K + 4 * it.k0, cp.mt), s);
+        o2 = scale(row_kslash_m(w4_sub(row_slash(cur[ext.in[0]], cur[ext.in[1]]), c), K + 4 * it.k0, cp.mt), s);
+      } else {
+        const W4<R> c = slash_col(cur[ext.in[2]], cur[it.in[2]]);
+        o = w4_add(slash_col(cur[it.in[1]], cur[it.in[0]]), c);
+        o2 = w4_sub(slash_col(cur[ext.in[1]], cur[ext.in[0]]), c);
+      }
+      return;
+    }
+    case 22:
+      xb[it.out] = w4_lower(w4_sub(ord_pair(cur[it.in[0]], cur[it.in[1]]),
+                                   ord_v3(cur[it.in[2]], cur[it.in3()], K + 4 * it.k0, K + 4 * it.k1)));
+      return;
+    case 23: xb[it.out] = w4_lower(ord_pair(cur[it.in[0]], cur[it.in[1]])); return;
+    case 24: {
+      W4<R> o = ord_v3(cur[it.in[0]], cur[it.in[1]], K + 4 * it.k0, K + 4 * it.k1);
+      o.w[0] = -o.w[0];
+      xb[it.out] = o;
+      return;
+    }
+    default: sc[it.out] = vdot(cur[it.in[0]], cur[it.in[1]]);
+  }
+}
+
 template <class P, class T>
 struct Engine {
   static constexpr int W = MGC_LANES_BYTES / (int)sizeof(T);
@@ -128,6 +178,7 @@ struct Engine {
   // per-thread work buffers
   std::vector<mg::W4<L>> cur = std::vector<mg::W4<L>>(P::HS_NSLOT);
   std::vector<mg::W4<L>> xb = std::vector<mg::W4<L>>(P::HS_XCAP);
+  std::vector<C> sc = std::vector<C>(P::HS_NSC);
   std::vector<C> J;
   L K[P::NMOM * 4];
   C pr[P::NPROP];
@@ -185,14 +236,21 @@ struct Engine {
     }
     // current variants, level by level
     for (int l = 1; l < P::HS_NLEVEL; ++l)
-      for (int t = P::hs_level(l); t < P::hs_level(l + 1); ++t) item<P, L>(items[t], cur.data(), K, pr, cl);
+      for (int t = P::hs_level(l); t < P::hs_level(l + 1); ++t) {
+        if constexpr (P::HS_ORDERED) ord_item<P, L>(items[t], cur.data(), xb.data(), sc.data(), K, pr, cl);
+        else item<P, L>(items[t], cur.data(), K, pr, cl);
+      }
     // amputated currents chunk by chunk; contractions of every good helicity
     J.assign((size_t)ng * NC, C(L(0.0), L(0.0)));
     const uint8_t* vt = P::hs_variants();
     for (int c = 0; c < P::HS_NXCHUNK; ++c) {
-      for (int t = P::hs_xitem(c); t < P::hs_xitem(c + 1); ++t) xitem<P, L>(items[t], cur.data(), xb.data(), K, cl);
+      for (int t = P::hs_xitem(c); t < P::hs_xitem(c + 1); ++t) {
+        if constexpr (P::HS_ORDERED) ord_item<P, L>(items[t], cur.data(), xb.data(), sc.data(), K, pr, cl);
+        else xitem<P, L>(items[t], cur.data(), xb.data(), K, cl);
+      }
       for (int h = 0; h < ng; ++h)
-        P::template hs_contract<L>(c, SlotArray<L>{cur.data()}, SlotArray<L>{xb.data()}, vt + good[h], &J[(size_t)h * NC]);
+        P::template hs_contract<L>(c, SlotArray<L>{cur.data()}, SlotArray<L>{xb.data(), sc.data()}, vt + good[h],
+                                   &J[(size_t)h * NC]);
     }
     // colour sum per helicity (lane precision), helicity sum per event in FP64
     double sum[W] = {};
@@ -212,7 +270,9 @@ struct Engine {
       }
       for (int i = 0; i < W; ++i) sum[i] += (double)s.v[i] / (double)P::CDEN;
     }
-    for (int i = 0; i < n; ++i) me[e0 + i] = sum[i] * P::NORM;
+    double norm = P::NORM;  // with the coupling where the currents go without it
+    for (int k = 0; k < P::HS_GS_POWER / 2; ++k) norm *= pp.gs2;
+    for (int i = 0; i < n; ++i) me[e0 + i] = sum[i] * norm;
   }
 };
 
@@ -223,7 +283,7 @@ void run(int64_t nevt, const double* mom, const int32_t* mask, const mg_params& 
   int ng = 0;
   for (int h = 0; h < P::NHEL; ++h)
     if (mask[h] != 0) good[ng++] = h;
-  const mg::PhysParams pp{prm.mz, prm.wz, prm.mt, prm.wt};
+  const mg::PhysParams pp{prm.mz, prm.wz, prm.mt, prm.wt, 4.0 * M_PI * prm.alpha_s};
   mg::Couplings<double> cd;
   const double e = std::sqrt(4.0 * M_PI / prm.alpha_inv), gs = std::sqrt(4.0 * M_PI * prm.alpha_s);
   cd.gs = gs;

@@ -17,6 +17,9 @@ struct Proc2 {
   static constexpr int NDIAGRAMS = 3;
   static constexpr int NAMPS = 3;
   // helicity-shared program (tables above)
+  static constexpr bool HS_ORDERED = false;
+  static constexpr int HS_GS_POWER = 0;  // couplings are in the currents
+  static constexpr int HS_NSC = 0;
   static constexpr int HS_NSLOT = 20;   // current variant slots per event
   static constexpr int HS_XCAP = 12;    // amputated-current slots per event and chunk
   static constexpr int HS_NXCHUNK = 1;
@@ -185,6 +188,7 @@ struct Proc2 {
     constexpr int t[NCOLOR][NCOLOR] = {{16, -2}, {-2, 16}};
     return t[i][j];
   }
+  static constexpr bool COLOUR_BLOCKS = false;
   // Dual amplitudes J_s of one helicity combination (hel[k] = +-1), accumulated
   // through J.add/sub/addi/subi(s, amp) (J_s += amp, -amp, i amp, -i amp);
   // Lock::sync() marks points where a CTA may re-align its warps.

@@ -496,4 +496,114 @@ __device__ __forceinline__ void dot4_acc(cx<R>& J, const W4<R>& x, const W4<R>& 
   else { J.im = -tr; J.re = ti; }
 }
 
+// ---- ordered program (g g -> t t~ g g) ------------------------------------------
+// Colour-ordered off-shell currents with the couplings and the factors i taken
+// out: G = -(V3 + V4) / K^2, R = -(sum R G/)(K/ + m) / D, V = (u gamma v) / K^2
+// with prop = i / D (top) or -i / K^2 (gluon), whose imaginary part is -1 / K^2.
+// V3(1, 2) = (A1.A2)(K2 - K1) - (A1.(K1 + 2 K2)) A2 + (A2.(2 K1 + K2)) A1
+template <class R>
+__device__ __forceinline__ W4<R> ord_v3(const W4<R>& a1, const W4<R>& a2, const R* K1, const R* K2) {
+  R d12[4], d23[4], d31[4];
+#pragma unroll
+  for (int mu = 0; mu < 4; ++mu) {
+    d12[mu] = K2[mu] - K1[mu];
+    d23[mu] = -(K1[mu] + R(2) * K2[mu]);
+    d31[mu] = R(2) * K1[mu] + K2[mu];
+  }
+  const cx<R> a12 = vdot(a1, a2);
+  const cx<R> c1 = kdot(d23, a1);
+  const cx<R> c2 = kdot(d31, a2);
+  W4<R> o;
+#pragma unroll
+  for (int mu = 0; mu < 4; ++mu) o.w[mu] = cfma(a1.w[mu], c2, cfma(a2.w[mu], c1, d12[mu] * a12));
+  return o;
+}
+template <class R>
+__device__ __forceinline__ W4<R> w4_rscale(const W4<R>& a, R s) {
+  W4<R> o;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) o.w[k] = s * a.w[k];
+  return o;
+}
+// s x + o
+template <class R>
+__device__ __forceinline__ W4<R> w4_axpy(cx<R> s, const W4<R>& x, const W4<R>& o) {
+  W4<R> r;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) r.w[k] = cfma(s, x.w[k], o.w[k]);
+  return r;
+}
+// lower index, sign s
+template <class R>
+__device__ __forceinline__ W4<R> w4_lower(const W4<R>& a) {
+  W4<R> o = a;
+#pragma unroll
+  for (int k = 1; k < 4; ++k) o.w[k] = -a.w[k];
+  return o;
+}
+// row . gamma^mu . col, upper index
+template <class R>
+__device__ __forceinline__ W4<R> ord_pair(const W4<R>& f, const W4<R>& g) {
+  W4<R> j;
+  const cx<R> ap = cfma(f.w[1], g.w[3], f.w[0] * g.w[2]), am = cfma(-f.w[1], g.w[3], f.w[0] * g.w[2]);
+  const cx<R> xp = cfma(f.w[1], g.w[2], f.w[0] * g.w[3]), xm = cfma(f.w[1], g.w[2], -(f.w[0] * g.w[3]));
+  const cx<R> bp = cfma(f.w[3], g.w[1], f.w[2] * g.w[0]), bm = cfma(f.w[3], g.w[1], -(f.w[2] * g.w[0]));
+  const cx<R> yp = cfma(f.w[3], g.w[0], f.w[2] * g.w[1]), ym = cfma(-f.w[3], g.w[0], f.w[2] * g.w[1]);
+  j.w[0] = ap + bp;
+  j.w[1] = xp - yp;
+  j.w[2] = mul_i(xm + ym);
+  j.w[3] = am + bm;
+  return j;
+}
+// the two words of a three-gluon current: G(ijk) and G(ikj) (up to the common
+// factor): V3 of the pair currents and V4(A,B,C) = (B.C) A + (A.B) C - 2 (A.C) B
+template <class R>
+__device__ __forceinline__ void ord_g3(const W4<R>& A, const W4<R>& B, const W4<R>& C, const W4<R>& AB,
+                                       const W4<R>& AC, const W4<R>& BC, const R* K, const uint8_t* k, R s,
+                                       W4<R>& w1, W4<R>& w2) {
+  const cx<R> ab = vdot(A, B), ac = vdot(A, C), bc = vdot(B, C);
+  W4<R> t = ord_v3(A, BC, K + 4 * k[0], K + 4 * k[5]);
+  w1 = ord_v3(AB, C, K + 4 * k[3], K + 4 * k[2]);
+  w2 = ord_v3(AC, B, K + 4 * k[4], K + 4 * k[1]);
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    const cx<R> x = bc * A.w[m];
+    w1.w[m] = s * cfma(ab, C.w[m], cfma(R(-2) * ac, B.w[m], w1.w[m] + (t.w[m] + x)));
+    w2.w[m] = s * cfma(ac, B.w[m], cfma(R(-2) * ab, C.w[m], w2.w[m] - (t.w[m] - x)));
+  }
+}
+// sum_i X_i Y_i.  FP32: the components in register pairs (0, 1), (2, 3) as the
+// planar slots load them: 8 FFMA2 and 3 additions, no register moves
+template <class R>
+__device__ __forceinline__ cx<R> dot4p(const W4<R>& x, const W4<R>& y) {
+  if constexpr (sizeof(R) == 4) {
+    const float2 xr0 = make_float2(x.w[0].re, x.w[1].re), xr1 = make_float2(x.w[2].re, x.w[3].re);
+    const float2 xi0 = make_float2(x.w[0].im, x.w[1].im), xi1 = make_float2(x.w[2].im, x.w[3].im);
+    const float2 yr0 = make_float2(y.w[0].re, y.w[1].re), yr1 = make_float2(y.w[2].re, y.w[3].re);
+    const float2 yi0 = make_float2(y.w[0].im, y.w[1].im), yi1 = make_float2(y.w[2].im, y.w[3].im);
+    float2 p = __ffma2_rn(xr1, yr1, __fmul2_rn(xr0, yr0));
+    const float2 q = __ffma2_rn(xi1, yi1, __fmul2_rn(xi0, yi0));
+    float2 r = __ffma2_rn(xr1, yi1, __fmul2_rn(xr0, yi0));
+    r = __ffma2_rn(xi0, yr0, r);
+    r = __ffma2_rn(xi1, yr1, r);
+    p = __ffma2_rn(make_float2(-1.0f, -1.0f), q, p);
+    return cx<R>(p.x + p.y, r.x + r.y);
+  } else {
+    cx<R> a = x.w[0] * y.w[0];
+#pragma unroll
+    for (int k = 1; k < 4; ++k) a = cfma(x.w[k], y.w[k], a);
+    return a;
+  }
+}
+// four-gluon vertex from its three products of opposite branches: 3 a - (a + b + c)
+template <class R>
+__device__ __forceinline__ cx<R> vertex4(cx<R> a, cx<R> sum) {
+  if constexpr (sizeof(R) == 4) {
+    const float2 r = __ffma2_rn(make_float2(3.0f, 3.0f), make_float2(a.re, a.im), make_float2(-sum.re, -sum.im));
+    return cx<R>(r.x, r.y);
+  } else {
+    return rfma(R(3), a, -sum);
+  }
+}
+
 }  // namespace mg

@@ -70,7 +70,7 @@ mg::SigLaunch sig_launch(int64_t nevt, const double* mom, const int32_t* mask, d
   l.mask = mask;
   l.me = me;
   l.mask_out = mask_out;
-  l.pp = mg::PhysParams{p.mz, p.wz, p.mt, p.wt};
+  l.pp = mg::PhysParams{p.mz, p.wz, p.mt, p.wt, 4.0 * M_PI * p.alpha_s};
   l.cd = couplings<double>(p);
   l.cf = couplings<float>(p);
   return l;
@@ -397,7 +397,7 @@ int mg_sigmakin_grad(int proc, int64_t nevt, double ecm, const double* rnd, int 
   l.gout = gout;
   l.grad = grad;
   l.me = me;
-  l.pp = mg::PhysParams{p.mz, p.wz, p.mt, p.wt};
+  l.pp = mg::PhysParams{p.mz, p.wz, p.mt, p.wt, 4.0 * M_PI * p.alpha_s};
   l.cd = couplings<double>(p);
   l.cf = couplings<float>(p);
   l.st = st;

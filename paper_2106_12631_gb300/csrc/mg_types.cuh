@@ -84,6 +84,37 @@ struct Slots {
   }
 };
 
+// The ordered program's slots: the real parts of a wavefunction's four
+// components, then the imaginary parts, so that the components come in
+// register pairs for the paired FP32 instructions (dot4p).  After the N slots
+// of a region, its scalars.
+template <class R, int N>
+struct PlanarSlots {
+  static constexpr int NPL = (int)(sizeof(W4<R>) / 16), PER = (int)(16 / sizeof(R));
+  uint4* p;
+  __device__ __forceinline__ W4<R> operator[](int i) const {
+    alignas(16) R v[8];
+#pragma unroll
+    for (int k = 0; k < NPL; ++k) *reinterpret_cast<uint4*>(v + k * PER) = p[i + k * N];
+    W4<R> w;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) w.w[c] = cx<R>(v[c], v[4 + c]);
+    return w;
+  }
+  __device__ __forceinline__ void set(int i, const W4<R>& w) const {
+    alignas(16) R v[8];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      v[c] = w.w[c].re;
+      v[4 + c] = w.w[c].im;
+    }
+#pragma unroll
+    for (int k = 0; k < NPL; ++k) p[i + k * N] = *reinterpret_cast<const uint4*>(v + k * PER);
+  }
+  __device__ __forceinline__ cx<R> scalar(int i) const { return reinterpret_cast<const cx<R>*>(p + N * NPL)[i]; }
+  __device__ __forceinline__ void set_scalar(int i, cx<R> x) const { reinterpret_cast<cx<R>*>(p + N * NPL)[i] = x; }
+};
+
 // Couplings and masses in the working precision.
 template <class R>
 struct Couplings {
@@ -106,18 +137,31 @@ struct Couplings {
 // external top mass; out/in: variant slots (a four-gluon term's three
 // operands X_0, X_1, W); k0/k1: momentum-table entries; prop: propagator
 // entry.  One aligned 16-byte word, read by one load.
+// Ordered program (types 15 on, see helas.cuh): 15 R(a), 16 C(a), 17 V, 18
+// G(ab), 19 R(ab) and R(ba), 20 C(ab) and C(ba), 21 G(ijk) and G(ikj), 22 vector
+// vertex B, 23 W, 24 P, 25 scalar product; a fourth operand, or the index of
+// the item's extension, in place of a and b (in3); an item with two words
+// writes the second one HS_WORD slots after the first.
+constexpr int HS_WORD = 8;
 struct alignas(16) HsItem {
   uint16_t out;
   uint16_t in[3];
   uint8_t type;
   int8_t a, b, c;
   uint8_t flag, k0, k1, prop;
+  __host__ __device__ int in3() const { return (uint8_t)a | (uint8_t)b << 8; }
 };
 static_assert(sizeof(HsItem) == 16, "item descriptor: one 16-byte word");
+// Further operand slots of an item with two words, and for three gluons the
+// momentum entries of i, j, k, ij, ik, jk.
+struct alignas(16) HsItemExt {
+  uint16_t in[3];
+  uint8_t k[6];
+};
 // Physics parameters in FP64 (propagator denominators are formed in FP64 in
-// both precision modes).
+// both precision modes); gs2 = g_s^2.
 struct PhysParams {
-  double mz, wz, mt, wt;
+  double mz, wz, mt, wt, gs2;
 };
 
 }  // namespace mg

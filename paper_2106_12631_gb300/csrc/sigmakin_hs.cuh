@@ -41,6 +41,11 @@ namespace mg {
 #define MG_HS_CTAS_SMALL 3  // the same below 24 colour flows (smaller variant sets per event)
 #endif
 
+// current slots and contraction operands in shared memory: the ordered
+// program's are planar
+template <class P, class R, int N>
+using HsSlots = std::conditional_t<P::HS_ORDERED, PlanarSlots<R, N>, Slots<R, N>>;
+
 // Many-colour processes in FP32: several 256-thread CTAs per SM (two of
 // 4 events x 64 helicities for gg -> t t~ g g, three of 8 x 32 for
 // gg -> t t~ g), so that one CTA's short barrier-bound phases overlap the
@@ -55,7 +60,8 @@ struct HsCfg {
   static constexpr int CTAS =
       P::NCOLOR >= 6 && sizeof(R) == 4 ? (P::NCOLOR >= 24 ? MG_HS_CTAS : MG_HS_CTAS_SMALL) : 1;
   static constexpr size_t CUR_BUDGET = 192 * 1024 / CTAS;
-  static constexpr size_t EV_BYTES = (size_t)(P::HS_NSLOT + P::HS_XBUFS * P::HS_XCAP) * sizeof(W4<R>);
+  static constexpr size_t EV_BYTES =
+      (size_t)(P::HS_NSLOT + P::HS_XBUFS * P::HS_XCAP) * sizeof(W4<R>) + (size_t)P::HS_NSC * sizeof(cx<R>);
   static constexpr int FIT = (int)(CUR_BUDGET / EV_BYTES);
   static constexpr int EVCAP = FIT < EVWANT ? (FIT > EVMIN ? FIT : EVMIN) : EVWANT;
   static constexpr int KP = ((P::NCOLOR + 15) / 16) * 16;
@@ -96,7 +102,8 @@ struct HsLayout {
   // the processes' slot counts, would otherwise map them to one group).
   static constexpr int EVPAD = EVCAP >= 8 ? 1 : 8 / EVCAP;
   static constexpr int CUR_EV = P::HS_NSLOT * Slots<R, 1>::NPL + EVPAD;
-  static constexpr int X_EV = P::HS_XCAP * Slots<R, 1>::NPL + EVPAD;
+  static constexpr int X_EV =
+      P::HS_XCAP * Slots<R, 1>::NPL + (int)(align_up((size_t)P::HS_NSC * sizeof(cx<R>), 128) / 16) + EVPAD;
   static constexpr size_t o_cur = o_U;
   static constexpr size_t o_x = o_U + 16 * size_t(EVCAP) * CUR_EV;
   static constexpr size_t o_A = o_U;
@@ -230,6 +237,17 @@ __device__ __forceinline__ void static_for(F&& f) {
   }
 }
 
+// (a.re b.re + c.re, a.im b.im + c.im): one paired instruction in FP32
+template <class R>
+__device__ __forceinline__ cx<R> pair_fma(cx<R> a, cx<R> b, cx<R> c) {
+  if constexpr (sizeof(R) == 4) {
+    const float2 r = __ffma2_rn(make_float2(a.re, a.im), make_float2(b.re, b.im), make_float2(c.re, c.im));
+    return cx<R>(r.x, r.y);
+  } else {
+    return cx<R>(fmac(a.re, b.re, c.re), fmac(a.im, b.im, c.im));
+  }
+}
+
 template <class P, class R>
 __device__ __forceinline__ R colour_sum_sym(const cx<R>* J) {
   static_assert(colour_matrix_symmetric<P>(), "colour matrix must be symmetric");
@@ -267,6 +285,53 @@ __device__ __forceinline__ R colour_sum_sym(const cx<R>* J) {
     sum = fmac(J[i].re, ur, fmac(J[i].im, ui, sum));
   });
   return sum / R(P::CDEN);
+}
+
+// Four-point Hadamard transform of every orbit of chains, in place, times s
+// (its own inverse for s = 1/4)
+template <class P, class R>
+__device__ __forceinline__ void colour_hadamard(cx<R>* J, R s) {
+  static_for<0, 6>([&](auto O) {
+    constexpr int o = decltype(O)::value;
+    cx<R>&a = J[P::colour_orbit(o, 0)], &b = J[P::colour_orbit(o, 1)], &c = J[P::colour_orbit(o, 2)],
+    &d = J[P::colour_orbit(o, 3)];
+    const cx<R> ab = a + b, cd = c + d, am = a - b, cm = c - d;
+    a = ab + cd;
+    b = ab - cd;
+    c = am + cm;
+    d = am - cm;
+    if (s != R(1)) {
+      a = s * a; b = s * b; c = s * c; d = s * d;
+    }
+  });
+}
+
+// |M_h|^2 on CUDA cores: the symmetric form of the whole matrix, or for 24
+// flows (where J is left transformed) of its four blocks: 129 paired FP32
+// instructions instead of 324
+template <class P, class R>
+__device__ __forceinline__ R colour_sum(cx<R>* J) {
+  if constexpr (!P::COLOUR_BLOCKS) {
+    return colour_sum_sym<P, R>(J);
+  } else {
+    colour_hadamard<P, R>(J, R(1));
+    cx<R> tot(R(0), R(0));  // re: sum of the products' real parts; im: of the imaginary parts
+    static_for<0, 24>([&](auto I) {
+      constexpr int x = decltype(I)::value / 6, i = decltype(I)::value % 6;
+      constexpr R mii = (R)P::colour_block(x, i, i);
+      const cx<R> y = J[P::colour_orbit(i, x)];
+      cx<R> u(mii * y.re, mii * y.im);
+      static_for<i + 1, 6>([&](auto Jc) {
+        constexpr int j = decltype(Jc)::value;
+        if constexpr (P::colour_block(x, i, j) != 0) {
+          constexpr R m = (R)(2 * P::colour_block(x, i, j));
+          u = pair_fma(cx<R>(m, m), J[P::colour_orbit(j, x)], u);
+        }
+      });
+      tot = pair_fma(y, u, tot);
+    });
+    return (tot.re + tot.im) / R(4 * P::CDEN);
+  }
 }
 
 // Propagator factor of one line from its FP64 momentum: the invariant
@@ -340,6 +405,109 @@ __device__ __forceinline__ cx<float> propagator_dfl(const float2* k, int kind, d
   const float inv = 1.0f / (r * r + di * di);
   const float ar = r * inv, ai = -di * inv;
   return kind == 1 ? cx<float>(-ai, ar) : cx<float>(ai, -ar);
+}
+
+// Products, sums, reciprocals and reciprocal square roots of double-floats (the
+// low parts not normalised), accurate to a few 2^-46.
+__device__ __forceinline__ dfl dfl_mul(dfl a, dfl b) {
+  const float p = a.hi * b.hi;
+  return {p, fmaf(a.lo, b.hi, fmaf(a.hi, b.lo, fmaf(a.hi, b.hi, -p)))};
+}
+__device__ __forceinline__ dfl dfl_add(dfl a, dfl b) {
+  const dfl s = two_sum(a.hi, b.hi);
+  return {s.hi, s.lo + (a.lo + b.lo)};
+}
+__device__ __forceinline__ float dfl_value(dfl a) { return a.hi + a.lo; }
+// one Newton step in FP32 on the FP32 value, its residual formed with FMAs; a
+// residual that is not small (the square of the value overflows) is dropped
+__device__ __forceinline__ float small_or_zero(float r) { return fabsf(r) < 1e-3f ? r : 0.0f; }
+__device__ __forceinline__ dfl dfl_rsqrt(dfl s) {
+  const float y = rsqrtf(s.hi), t = y * y, tl = fmaf(y, y, -t);
+  const float r = fmaf(s.hi, t, -1.0f) + fmaf(s.hi, tl, s.lo * t);
+  return {y, -0.5f * y * small_or_zero(r)};
+}
+__device__ __forceinline__ dfl dfl_rcp(dfl b) {
+  const float y = 1.0f / b.hi;
+  return {y, y * small_or_zero(-fmaf(b.hi, y, -1.0f) - b.lo * y)};
+}
+
+// External wavefunctions of the mixed mode, both helicities of a leg from its
+// double-float momentum (the formulas of ixxxxx, oxxxxx and vxxxxx): rounded
+// once, to FP32.  Near-collinear and soft events amplify the errors of the
+// spinors and polarisation vectors; in plain FP32 they were the mixed mode's
+// largest error there (2-norm of the error of g g -> t t~ g g over events inside
+// generator cuts 6.6e-7, rounded once 4.5e-7).  w[0]: helicity -1, w[1]: +1.
+__device__ __forceinline__ void ext_vector_dfl(const dfl* k, int nsv, W4<float>* w) {
+  const dfl kt2 = dfl_add(dfl_mul(k[1], k[1]), dfl_mul(k[2], k[2]));
+  const dfl kk2 = dfl_add(kt2, dfl_mul(k[3], k[3]));
+  const dfl r2 = {0.707106769f, 1.21016175e-8f};  // 1 / sqrt 2
+  float x1, x2, x3, y1, y2;  // (ct cp, ct sp, st), (sp, cp) over sqrt 2
+  if (kt2.hi > 0.0f) {
+    const dfl u = dfl_mul(dfl_rsqrt(kt2), r2), v = dfl_rsqrt(kk2);
+    const dfl cp = dfl_mul(k[1], u), sp = dfl_mul(k[2], u), ct = dfl_mul(k[3], v);
+    x1 = dfl_value(dfl_mul(ct, cp));
+    x2 = dfl_value(dfl_mul(ct, sp));
+    x3 = dfl_value(dfl_mul(dfl_mul(kt2, u), v));
+    y1 = dfl_value(sp);
+    y2 = dfl_value(cp);
+  } else {
+    x1 = k[3].hi >= 0.0f ? r2.hi : -r2.hi;
+    x2 = x3 = y1 = 0.0f;
+    y2 = r2.hi;
+  }
+  const float b = nsv > 0 ? -1.0f : 1.0f;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const float a = h == 0 ? 1.0f : -1.0f;
+    w[h].w[0] = cx<float>(0.0f, 0.0f);
+    w[h].w[1] = cx<float>(a * x1, -b * y1);
+    w[h].w[2] = cx<float>(a * x2, b * y2);
+    w[h].w[3] = cx<float>(-a * x3, 0.0f);
+  }
+}
+__device__ __forceinline__ void ext_fermion_dfl(const dfl* p, float m, int nsf, bool row, W4<float>* w) {
+  const dfl pt2 = dfl_add(dfl_mul(p[1], p[1]), dfl_mul(p[2], p[2]));
+  const dfl pp2 = dfl_add(pt2, dfl_mul(p[3], p[3]));
+  dfl pp = {0.0f, 0.0f};
+  if (pp2.hi > 0.0f) pp = dfl_mul(pp2, dfl_rsqrt(pp2));
+  const dfl ppz = p[3].hi >= 0.0f ? dfl_add(pp, p[3])
+                                  : dfl_mul(pt2, dfl_rcp(dfl_add(pp, dfl{-p[3].hi, -p[3].lo})));
+  // chi_+ = (a, b), chi_- = (-b^*, a), b = (bx, by)
+  dfl a = {0.0f, 0.0f}, bx = {1.0f, 0.0f}, by = {0.0f, 0.0f};  // exactly along -z
+  if (ppz.hi > 0.0f) {
+    const dfl n = dfl_mul(pp, ppz);
+    const dfl nrm = dfl_rsqrt(dfl{2.0f * n.hi, 2.0f * n.lo});
+    a = dfl_mul(ppz, nrm);
+    bx = dfl_mul(p[1], nrm);
+    by = dfl_mul(p[2], nrm);
+  }
+  const dfl e = dfl_add(p[0], pp), r = dfl_rsqrt(e);
+  const dfl wp = dfl_mul(e, r), wm = dfl_mul(r, dfl{m, 0.0f});
+  float q[2][3];  // omega_+ and omega_- times (a, bx, by)
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const dfl o = i == 0 ? wp : wm;
+    q[i][0] = dfl_value(dfl_mul(o, a));
+    q[i][1] = dfl_value(dfl_mul(o, bx));
+    q[i][2] = dfl_value(dfl_mul(o, by));
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    // u: chi_hel, omegas (-hel, hel); v: chi_-hel, omegas (-hel omega_hel, hel omega_-hel)
+    const bool plus = h == 1, chip = nsf > 0 ? plus : !plus;
+    const int lo = nsf > 0 ? (plus ? 1 : 0) : (plus ? 0 : 1);
+    const float slo = nsf > 0 ? 1.0f : (plus ? -1.0f : 1.0f), shi = nsf > 0 ? 1.0f : -slo;
+    cx<float> c[4];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const float* z = lo == i ? q[0] : q[1];
+      const float s = i == 0 ? slo : shi;
+      c[2 * i] = chip ? cx<float>(s * z[0], 0.0f) : cx<float>(-s * z[1], s * z[2]);
+      c[2 * i + 1] = chip ? cx<float>(s * z[1], s * z[2]) : cx<float>(s * z[0], 0.0f);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[h].w[i] = row ? conj(c[(i + 2) & 3]) : c[i];
+  }
 }
 
 // Phase 1 of the forward kernels, in three parts:
@@ -514,7 +682,10 @@ __device__ __forceinline__ void hs_tables(unsigned char* smem, const PhysParams&
   R* K = reinterpret_cast<R*>(smem + L::o_K);                // [EV][NMOM][4]
   cx<R>* pr = reinterpret_cast<cx<R>*>(smem + L::o_pr);      // [EV][NPROP]
   const int nev = grp.nev;
-  for (int t = grp.j; t < nev * (NM + NEXT); t += grp.tpg) {
+  // mixed mode: one thread per (event, leg), both helicities (consecutive items)
+  static_assert(NEXT == 2 * NPAR, "level 0: two helicities per leg");
+  constexpr int NE = DF ? NPAR : NEXT;
+  for (int t = grp.j; t < nev * (NM + NE); t += grp.tpg) {
     if (t < nev * NM) {
       const int el = t / NM, j = t - el * NM, e = grp.ev0 + el;
       const int4 d = md[j];
@@ -567,23 +738,37 @@ __device__ __forceinline__ void hs_tables(unsigned char* smem, const PhysParams&
         }
       }
     } else {
-      const int t2 = t - nev * NM, el = t2 / NEXT, e = grp.ev0 + el;
-      const HsItem it = P::hs_items()[t2 - el * NEXT];
-      R k[4];
+      const int t2 = t - nev * NM, el = t2 / NE, e = grp.ev0 + el, j = t2 - el * NE;
+      const HsSlots<P, R, P::HS_NSLOT> cur{curs + e * CUR_EV};
+      if constexpr (DF) {
+        const HsItem it = P::hs_items()[2 * j];
+        dfl k[4];
 #pragma unroll
-      for (int mu = 0; mu < 4; ++mu) {
-        if constexpr (DF) k[mu] = reinterpret_cast<const float2*>(smem + L::o_p)[(e * NPAR + it.a) * 4 + mu].x;
-        else k[mu] = reinterpret_cast<const double*>(smem + L::o_p)[(e * NPAR + it.a) * 4 + mu];
+        for (int mu = 0; mu < 4; ++mu) {
+          const float2 v = reinterpret_cast<const float2*>(smem + L::o_p)[(e * NPAR + it.a) * 4 + mu];
+          k[mu] = dfl{v.x, v.y};
+        }
+        W4<R> o[2];
+        if (it.type == 2) ext_vector_dfl(k, it.c, o);
+        else ext_fermion_dfl(k, it.flag ? cp.mt : 0.0f, it.c, it.type == 1, o);
+        cur.set(it.out, o[0]);
+        cur.set(P::hs_items()[2 * j + 1].out, o[1]);
+      } else {
+        const HsItem it = P::hs_items()[j];
+        const double* k = reinterpret_cast<const double*>(smem + L::o_p) + (e * NPAR + it.a) * 4;
+        W4<R> o;
+        if (it.type == 0) o = ixxxxx<R>(k, it.flag ? cp.mt : R(0), it.b, it.c);
+        else if (it.type == 1) o = oxxxxx<R>(k, it.flag ? cp.mt : R(0), it.b, it.c);
+        else o = vxxxxx<R>(k, it.b, it.c);
+        cur.set(it.out, o);
       }
-      W4<R> o;
-      if (it.type == 0) o = ixxxxx<R>(k, it.flag ? cp.mt : R(0), it.b, it.c);
-      else if (it.type == 1) o = oxxxxx<R>(k, it.flag ? cp.mt : R(0), it.b, it.c);
-      else o = vxxxxx<R>(k, it.b, it.c);
-      Slots<R, P::HS_NSLOT>{curs + e * CUR_EV}.set(it.out, o);
     }
   }
   grp.sync();
 }
+
+// a shared-memory word read where it is written here (not kept in a register)
+__device__ __forceinline__ int lds_again(const int* p) { return *reinterpret_cast<const volatile int*>(p); }
 
 // Item of work index t when the lanes take items item-major: consecutive
 // lanes take one item for each of the group's nev events, so that a warp holds
@@ -593,6 +778,57 @@ __device__ __forceinline__ void hs_tables(unsigned char* smem, const PhysParams&
 template <class L>
 __device__ __forceinline__ int hs_item_of(int t, int nev) {
   return nev == L::EVCAP ? t / L::EVCAP : t / nev;
+}
+
+// Items of the ordered program: a two-leg current ...
+template <class P, class R>
+__device__ __forceinline__ void ord_item(const HsItem& it, const HsSlots<P, R, P::HS_NSLOT>& cur, const R* K,
+                                         const cx<R>* pr, const Couplings<R>& cp) {
+  W4<R> o;
+  switch (it.type) {
+    case 15: o = FFV1_2<R>(cur[it.in[0]], cur[it.in[1]], R(1), K + 4 * it.k0, cp.mt, pr[it.prop]); break;
+    case 16: o = FFV1_1<R>(cur[it.in[0]], cur[it.in[1]], R(1), K + 4 * it.k0, cp.mt, pr[it.prop]); break;
+    case 17: o = w4_rscale(ord_pair(cur[it.in[0]], cur[it.in[1]]), -pr[it.prop].im); break;
+    default: o = w4_rscale(ord_v3(cur[it.in[0]], cur[it.in[1]], K + 4 * it.k0, K + 4 * it.k1), pr[it.prop].im);
+  }
+  cur.set(it.out, o);
+}
+// ... and an operand of the contractions
+template <class P, class R>
+__device__ __forceinline__ void ord_xitem(const HsItem& it, const HsSlots<P, R, P::HS_NSLOT>& cur,
+                                          const HsSlots<P, R, P::HS_XCAP>& xb, const R* K, const cx<R>* pr,
+                                          const Couplings<R>& cp) {
+  if (it.type == 25) {
+    xb.set_scalar(it.out, vdot(cur[it.in[0]], cur[it.in[1]]));
+    return;
+  }
+  W4<R> o, o2;
+  if (it.type <= 21) {  // two words
+    const HsItemExt ext = P::hs_item_ext()[it.in3()];
+    if (it.type == 21) {
+      ord_g3(cur[it.in[0]], cur[it.in[1]], cur[it.in[2]], cur[ext.in[0]], cur[ext.in[1]], cur[ext.in[2]], K, ext.k,
+             pr[it.prop].im, o, o2);
+    } else if (it.type == 19) {
+      const W4<R> c = row_slash(cur[it.in[2]], cur[ext.in[2]]);
+      const cx<R> s = mul_i(pr[it.prop]);
+      o = scale(row_kslash_m(w4_add(row_slash(cur[it.in[0]], cur[it.in[1]]), c), K + 4 * it.k0, cp.mt), s);
+      o2 = scale(row_kslash_m(w4_sub(row_slash(cur[ext.in[0]], cur[ext.in[1]]), c), K + 4 * it.k0, cp.mt), s);
+    } else {
+      const W4<R> c = slash_col(cur[ext.in[2]], cur[it.in[2]]);
+      o = w4_add(slash_col(cur[it.in[1]], cur[it.in[0]]), c);
+      o2 = w4_sub(slash_col(cur[ext.in[1]], cur[ext.in[0]]), c);
+    }
+    xb.set(it.out + HS_WORD, o2);
+  } else if (it.type == 22) {
+    const W4<R> g = ord_v3(cur[it.in[2]], cur[it.in3()], K + 4 * it.k0, K + 4 * it.k1);
+    o = w4_lower(w4_sub(ord_pair(cur[it.in[0]], cur[it.in[1]]), g));
+  } else if (it.type == 23) {
+    o = w4_lower(ord_pair(cur[it.in[0]], cur[it.in[1]]));
+  } else {
+    o = ord_v3(cur[it.in[0]], cur[it.in[1]], K + 4 * it.k0, K + 4 * it.k1);  // times -1, lower index
+    o.w[0] = -o.w[0];
+  }
+  xb.set(it.out, o);
 }
 
 // one current variant
@@ -709,13 +945,15 @@ __device__ __forceinline__ void hs_choices(const unsigned char* smem, const SigA
 // Record of one event's current variants and momentum table in global memory
 // (the kernel-split variant: the first kernel writes them, the second reads
 // them back into shared memory): HS_NSLOT slots of 16-byte planes, then the
-// momentum table K[NMOM][4] in the working precision.
+// momentum table K[NMOM][4] in the working precision and, where operands of the
+// contractions have propagators (ordered program), the propagator factors.
 template <class P, class R>
 struct HsRecord {
   static constexpr int CUR = P::HS_NSLOT * Slots<R, 1>::NPL;
   static_assert((P::NMOM * 4 * sizeof(R)) % 16 == 0, "momentum table in 16-byte words");
   static constexpr int KW = (int)(P::NMOM * 4 * sizeof(R) / 16);
-  static constexpr int WORDS = CUR + KW;
+  static constexpr int PW = P::HS_ORDERED ? (int)(align_up(P::NPROP * sizeof(cx<R>), 16) / 16) : 0;
+  static constexpr int WORDS = CUR + KW + PW;
 };
 
 // Where a group's momenta come from: the momentum buffer (mg_sigmakin), the
@@ -751,6 +989,15 @@ __device__ __noinline__ void rambo_event_fused(const double* __restrict__ rnd, i
 #pragma unroll
     for (int mu = 0; mu < 4; ++mu) out[(2 + f) * 4 + mu] = z.k[f][mu];
   wgt[i] = z.w;
+}
+
+// averaging factors, and the coupling where the currents go without it
+template <class P>
+__device__ __forceinline__ double hs_norm(const PhysParams& pp) {
+  double f = P::NORM;
+#pragma unroll
+  for (int k = 0; k < P::HS_GS_POWER / 2; ++k) f *= pp.gs2;
+  return f;
 }
 
 // The helicity-shared program for the events [first, last) of the batch.
@@ -796,6 +1043,13 @@ __device__ __forceinline__ void hs_sigmakin_body(const SigArgs& a, const Couplin
   // group per CTA for a grid of all groups, several for a persistent grid
   const int ngrp = (int)((last - first + ev - 1) / ev);
   if ((int)blockIdx.x >= ngrp) return;
+  // kept in shared memory and read where they are needed: registers that would
+  // stay live through the contractions otherwise
+  if (tid == 0) {
+    misc[2] = ngrp;
+    misc[6] = ng;
+    misc[7] = ev;
+  }
   if (ng == 0) {
     for (int g = blockIdx.x; g < ngrp; g += gridDim.x) {
       const int64_t e0 = first + (int64_t)g * ev;
@@ -819,6 +1073,7 @@ __device__ __forceinline__ void hs_sigmakin_body(const SigArgs& a, const Couplin
     tc::fence_before_sync();
   }
   const R* Kall = reinterpret_cast<const R*>(smem + L::o_K);
+  const cx<R>* prall = reinterpret_cast<const cx<R>*>(smem + L::o_pr);
   const HsItem* items = P::hs_items();
   if constexpr (SRC == kSrcMomenta) {
     // the first group's momenta; later groups' arrive by prefetch
@@ -840,8 +1095,9 @@ __device__ __forceinline__ void hs_sigmakin_body(const SigArgs& a, const Couplin
     tmem = static_cast<uint32_t>(misc[1]);
   }
 #pragma unroll 1
-  for (int g = blockIdx.x; g < ngrp; g += gridDim.x) {
+  for (int g = blockIdx.x; g < lds_again(misc + 2); g += gridDim.x) {
     // e0 and nev are formed again after the contractions (fewer live registers)
+    const int ev = lds_again(misc + 7);
     const int nev = (int)min((int64_t)ev, last - (first + (int64_t)g * ev));
     const HsGroup grp = hs_group<NT>(L::TC || !MG_HS_EVENT_SYNC, ng, ev, nev);
     if constexpr (FROM_RECORDS) {
@@ -853,7 +1109,16 @@ __device__ __forceinline__ void hs_sigmakin_body(const SigArgs& a, const Couplin
         const int e = t / RC::WORDS, w = t - e * RC::WORDS;
         const uint4 v = __ldcs(in + t);  // read once: streaming
         if (w < RC::CUR) curs[e * CUR_EV + w] = v;
-        else ks[e * (L::KEV * (int)sizeof(R) / 16) + (w - RC::CUR)] = v;
+        else if (w < RC::CUR + RC::KW) ks[e * (L::KEV * (int)sizeof(R) / 16) + (w - RC::CUR)] = v;
+        else {
+          const cx<R>* f = reinterpret_cast<const cx<R>*>(&v);
+          constexpr int PER = (int)(16 / sizeof(cx<R>));
+#pragma unroll
+          for (int k = 0; k < PER; ++k) {
+            const int j = (w - RC::CUR - RC::KW) * PER + k;
+            if (j < P::NPROP) reinterpret_cast<cx<R>*>(smem + L::o_pr)[e * P::NPROP + j] = f[k];
+          }
+        }
       }
       __syncthreads();
     } else {
@@ -861,7 +1126,7 @@ __device__ __forceinline__ void hs_sigmakin_body(const SigArgs& a, const Couplin
       // converted after the last current level (p is free once the tables are built)
       const int gn = g + gridDim.x;
       const int64_t e0n = first + (int64_t)gn * ev;
-      const int nevn = gn < ngrp ? (int)min((int64_t)ev, last - e0n) : 0;
+      const int nevn = gn < lds_again(misc + 2) ? (int)min((int64_t)ev, last - e0n) : 0;
       if constexpr (SRC == kSrcRambo) {
         // the next group's RAMBO on the last lanes, which the tables phase
         // leaves idle when it has fewer items than threads
@@ -874,7 +1139,6 @@ __device__ __forceinline__ void hs_sigmakin_body(const SigArgs& a, const Couplin
       }
       // 1. per-event tables (the momenta are in p)
       hs_tables<P, R, L, CUR_EV, L::KEV>(smem, a.pp, grp, curs, cp);
-      const cx<R>* prall = reinterpret_cast<const cx<R>*>(smem + L::o_pr);
       // 2. current variants, level by level (level 0, the external wavefunctions,
       //    came with phase 1); consecutive threads take one item for each event (hs_item_of)
 #pragma unroll
@@ -883,8 +1147,9 @@ __device__ __forceinline__ void hs_sigmakin_body(const SigArgs& a, const Couplin
         for (int t = grp.j; t < n; t += grp.tpg) {
           const int ii = hs_item_of<L>(t, grp.nev), e = grp.ev0 + t - ii * grp.nev;
           const HsItem it = items[i0 + ii];
-          hs_item<P, R>(it, Slots<R, P::HS_NSLOT>{curs + e * CUR_EV}, Kall + e * L::KEV, prall + e * P::NPROP,
-                        cp);
+          const HsSlots<P, R, P::HS_NSLOT> cur{curs + e * CUR_EV};
+          if constexpr (P::HS_ORDERED) ord_item<P, R>(it, cur, Kall + e * L::KEV, prall + e * P::NPROP, cp);
+          else hs_item<P, R>(it, cur, Kall + e * L::KEV, prall + e * P::NPROP, cp);
         }
         if (l == P::HS_NLEVEL - 1) {
           cp_async_wait_all();
@@ -895,48 +1160,41 @@ __device__ __forceinline__ void hs_sigmakin_body(const SigArgs& a, const Couplin
         }
       }
     }
-    // 3. amputated currents chunk by chunk into two alternating buffers: in
-    //    interval c every thread first builds its share of chunk c, then
-    //    contracts chunk c - 1 for its (event, helicity) (J in registers), so the
-    //    latency of the item work hides behind other warps' contractions
+    // 3. the operands of the contractions (amputated currents), then every
+    //    thread contracts for its (event, helicity), J in registers
+    {
+      const int i0 = P::hs_xitem(0), ni = P::hs_xitem(1) - i0, n = ni * grp.nev;
+      for (int t = grp.j; t < n; t += grp.tpg) {
+        const int ii = hs_item_of<L>(t, grp.nev), ex = grp.ev0 + t - ii * grp.nev;
+        const HsItem it = items[i0 + ii];
+        const HsSlots<P, R, P::HS_NSLOT> cur{curs + ex * CUR_EV};
+        const HsSlots<P, R, P::HS_XCAP> xs{xbufs + ex * X_EV};
+        if constexpr (P::HS_ORDERED) ord_xitem<P, R>(it, cur, xs, Kall + ex * L::KEV, prall + ex * P::NPROP, cp);
+        else hs_xitem<P, R>(it, cur, xs, Kall + ex * L::KEV, cp);
+      }
+    }
+    grp.sync();
+    const int ng = lds_again(misc + 6);
     const bool active = tid < nev * ng;
     const int e = active ? tid / ng : 0;
     const int ih = good[active ? tid - e * ng : 0];
-    constexpr int XBUF = L::EVCAP * X_EV;  // one chunk buffer, all events
     cx<R> J[NC];
 #pragma unroll
     for (int s = 0; s < NC; ++s) J[s] = cx<R>(R(0), R(0));
-#pragma unroll 1
-    for (int c = 0; c <= P::HS_NXCHUNK; ++c) {
-      if (c < P::HS_NXCHUNK) {
-        uint4* xb = xbufs + (P::HS_XBUFS == 2 ? (c & 1) * XBUF : 0);
-        const int i0 = P::hs_xitem(c), ni = P::hs_xitem(c + 1) - i0, n = ni * grp.nev;
-        for (int t = grp.j; t < n; t += grp.tpg) {
-          const int ii = hs_item_of<L>(t, grp.nev), ex = grp.ev0 + t - ii * grp.nev;
-          const HsItem it = items[i0 + ii];
-          hs_xitem<P, R>(it, Slots<R, P::HS_NSLOT>{curs + ex * CUR_EV}, Slots<R, P::HS_XCAP>{xb + ex * X_EV},
-                         Kall + ex * L::KEV, cp);
-        }
-      }
-      if (c > 0) {
-        const uint4* xb = xbufs + (P::HS_XBUFS == 2 ? ((c - 1) & 1) * XBUF : 0);
-        P::template hs_contract<R>(c - 1, Slots<R, P::HS_NSLOT>{curs + e * CUR_EV},
-                                   Slots<R, P::HS_XCAP>{const_cast<uint4*>(xb) + e * X_EV}, vtab + ih, J);
-      }
-      if (c < P::HS_NXCHUNK) grp.sync();
-    }
+    P::template hs_contract<R>(0, HsSlots<P, R, P::HS_NSLOT>{curs + e * CUR_EV},
+                               HsSlots<P, R, P::HS_XCAP>{xbufs + e * X_EV}, vtab + ih, J);
     // 4. colour sum and helicity sum
     double m2;
     if constexpr (L::TC) {
       __syncthreads();  // the A tiles overwrite the current variants
       m2 = (double)colour_sum_tc_regs<P, L>(smem, J, tmem, mbar);
     } else {
-      m2 = (double)colour_sum_sym<P, R>(J);
+      m2 = (double)colour_sum<P, R>(J);
     }
     sm2[tid] = active ? m2 : 0.0;
     if constexpr (L::TC) tc::fence_before_sync();
     grp.sync();
-    const int64_t e0 = first + (int64_t)g * ev;
+    const int64_t e0 = first + (int64_t)g * lds_again(misc + 7);
     // fixed-order FP64 helicity sum per event: eight lanes per event each add
     // every eighth helicity in order, then a butterfly over the eight lanes
     // (addition commutes, so every lane ends with the same bits); sm2 is next
@@ -952,7 +1210,7 @@ __device__ __forceinline__ void hs_sigmakin_body(const SigArgs& a, const Couplin
       sum += __shfl_xor_sync(0xffffffffu, sum, 1);
       sum += __shfl_xor_sync(0xffffffffu, sum, 2);
       sum += __shfl_xor_sync(0xffffffffu, sum, 4);
-      if (t < grp.nev * 8 && q == 0) a.me[e0 + eh] = sum * P::NORM;
+      if (t < grp.nev * 8 && q == 0) a.me[e0 + eh] = sum * hs_norm<P>(a.pp);
     }
     // 5. helicity and colour-flow choices (batched entry point), once every
     //    group of the CTA is done with the union region; the closing barrier
@@ -960,6 +1218,7 @@ __device__ __forceinline__ void hs_sigmakin_body(const SigArgs& a, const Couplin
     if (a.hel_out || a.col_out) {
       __syncthreads();
       if (a.col_out) {
+        if constexpr (!L::TC && P::COLOUR_BLOCKS) colour_hadamard<P, R>(J, R(0.25));  // back to the chains
         R* wj = reinterpret_cast<R*>(smem + L::o_U) + tid * HsChoice<P, R>::NCP;  // the union is dead here
 #pragma unroll
         for (int s = 0; s < NC; ++s) wj[s] = active ? J[s].re * J[s].re + J[s].im * J[s].im : R(0);

@@ -59,8 +59,9 @@ __global__ void __launch_bounds__(HsSplitA<P, R>::NT, HsSplitA<P, R>::CTAS)
     for (int t = tid; t < n; t += NT) {
       const int e = t / ni;
       const HsItem it = items[i0 + t - e * ni];
-      hs_item<P, R>(it, Slots<R, P::HS_NSLOT>{curs + e * RC::CUR}, Kall + e * P::NMOM * 4, prall + e * P::NPROP,
-                    cp);
+      const HsSlots<P, R, P::HS_NSLOT> cur{curs + e * RC::CUR};
+      if constexpr (P::HS_ORDERED) ord_item<P, R>(it, cur, Kall + e * P::NMOM * 4, prall + e * P::NPROP, cp);
+      else hs_item<P, R>(it, cur, Kall + e * P::NMOM * 4, prall + e * P::NPROP, cp);
     }
     __syncthreads();
   }
@@ -68,7 +69,18 @@ __global__ void __launch_bounds__(HsSplitA<P, R>::NT, HsSplitA<P, R>::CTAS)
   uint4* out = rec + (e0 - first) * RC::WORDS;
   for (int t = tid; t < nev * RC::WORDS; t += NT) {
     const int e = t / RC::WORDS, w = t - e * RC::WORDS;
-    out[t] = w < RC::CUR ? curs[e * RC::CUR + w] : ks[e * RC::KW + (w - RC::CUR)];
+    if (w < RC::CUR + RC::KW) {
+      out[t] = w < RC::CUR ? curs[e * RC::CUR + w] : ks[e * RC::KW + (w - RC::CUR)];
+    } else {
+      constexpr int PER = (int)(16 / sizeof(cx<R>));
+      alignas(16) cx<R> f[PER];
+#pragma unroll
+      for (int k = 0; k < PER; ++k) {
+        const int j = (w - RC::CUR - RC::KW) * PER + k;
+        f[k] = prall[e * P::NPROP + min(j, P::NPROP - 1)];
+      }
+      out[t] = *reinterpret_cast<const uint4*>(f);
+    }
   }
 }
 

@@ -388,6 +388,45 @@ def colour_sum_flops(cnum) -> int:
     return 4 * nz + 4 * cnum.shape[0] + 1
 
 
+# The colour matrix commutes with relabelling the gluons.  For four gluons the
+# relabellings by the Klein four-group split the 24 chains into six orbits of four,
+# and a four-point Hadamard transform of each orbit splits C into four 6 x 6 blocks
+# (one per character), most of whose entries vanish:
+#   J^dagger C J = 1/4 sum_x sum_{o,p} y_xo^* M_x[o][p] y_xp,
+#   y_xo = sum_k x(k) J[k o],  M_x[o][p] = sum_k x(k) C[o][k p]
+KLEIN = ((0, 1, 2, 3), (1, 0, 3, 2), (2, 3, 0, 1), (3, 2, 1, 0))
+KLEIN_CHARACTERS = ((1, 1, 1, 1), (1, 1, -1, -1), (1, -1, 1, -1), (1, -1, -1, 1))
+
+
+def colour_blocks(perms, cnum):
+    """(orbits [6][4] of chain indices, blocks [4][6][6]) of the four-gluon colour matrix."""
+    index = {p: i for i, p in enumerate(perms)}
+    orbits, seen = [], set()
+    for p in perms:
+        if p not in seen:
+            o = [tuple(e[g] for g in p) for e in KLEIN]
+            seen |= set(o)
+            orbits.append([index[w] for w in o])
+    blocks = [[[sum(x[k] * int(cnum[a[0], b[k]]) for k in range(4)) for b in orbits] for a in orbits]
+              for x in KLEIN_CHARACTERS]
+    H = np.zeros((24, 24), dtype=np.int64)  # rows (x, orbit), columns chains
+    for xi, x in enumerate(KLEIN_CHARACTERS):
+        for oi, o in enumerate(orbits):
+            for k in range(4):
+                H[6 * xi + oi, o[k]] = x[k]
+    B = np.zeros((24, 24), dtype=np.int64)
+    for xi in range(4):
+        B[6 * xi:6 * xi + 6, 6 * xi:6 * xi + 6] = blocks[xi]
+    assert np.array_equal(H.T @ B @ H, 4 * np.asarray(cnum))
+    return orbits, blocks
+
+
+def colour_blocks_flops(blocks) -> int:
+    """Hadamard transforms (8 complex adds per orbit), then as colour_sum_sym_flops."""
+    upper = sum(1 for M in blocks for i in range(6) for j in range(i + 1, 6) if M[i][j])
+    return 6 * 8 * 2 + 2 * 24 + 4 * upper + 4 * 24 + 1
+
+
 LOCK_EVERY = 8  # routine calls between CTA-wide lockstep points
 
 
@@ -723,6 +762,14 @@ def bf16_colour_image(cnum) -> np.ndarray:
     return img.view(np.uint32)
 
 
+ORDERED_PROCS = (4,)  # processes evaluated by the ordered program
+
+
+def program(proc: Process, em: "Emitter"):
+    """The helicity-shared program of a process."""
+    return (OrderedProgram if proc.spec.pid in ORDERED_PROCS else SharedProgram)(proc, em)
+
+
 def generate(pid: int) -> str:
     proc = Process(PROCS[pid])
     em = Emitter(proc)
@@ -743,7 +790,7 @@ def generate(pid: int) -> str:
     out.append("// colour-flow coefficients used: %s" % sorted(coefs, key=lambda z: (z.real, z.imag)))
     out.append("#pragma once")
     out.append("namespace mg {")
-    sp = SharedProgram(proc, em)
+    sp = program(proc, em)
     out.extend(sp.emit_tables(pid))
     img = bf16_colour_image(em.cnum)
     out.append("// colour-matrix numerators as the BF16 B operand of the tensor-core colour sum")
@@ -816,6 +863,21 @@ def generate(pid: int) -> str:
                % ", ".join("{" + ", ".join(str(int(x)) for x in row) + "}" for row in em.cnum))
     out.append("    return t[i][j];")
     out.append("  }")
+    out.append("  static constexpr bool COLOUR_BLOCKS = %s;" % ("true" if ncol == 24 else "false"))
+    if ncol == 24:
+        orbits, blocks = colour_blocks(em.perms, em.cnum)
+        out.append("  // chains of each orbit under the Klein four-group's relabellings, and the blocks of")
+        out.append("  // the colour matrix per character: J^dagger CNUM J = 1/4 sum_x y_x^dagger block_x y_x,")
+        out.append("  // y_x[o] = sum_k x(k) J[orbit(o, k)]")
+        out.append("  static __host__ __device__ constexpr int colour_orbit(int o, int k) {")
+        out.append("    constexpr int t[6][4] = {%s};" % ", ".join("{" + ", ".join(map(str, o)) + "}" for o in orbits))
+        out.append("    return t[o][k];")
+        out.append("  }")
+        out.append("  static __host__ __device__ constexpr int colour_block(int x, int i, int j) {")
+        out.append("    constexpr int t[4][6][6] = {%s};" % ", ".join(
+            "{" + ", ".join("{" + ", ".join(map(str, r)) + "}" for r in M) + "}" for M in blocks))
+        out.append("    return t[x][i][j];")
+        out.append("  }")
     out.append("  // Dual amplitudes J_s of one helicity combination (hel[k] = +-1), accumulated")
     out.append("  // through J.add/sub/addi/subi(s, amp) (J_s += amp, -amp, i amp, -i amp);")
     out.append("  // Lock::sync() marks points where a CTA may re-align its warps.")
@@ -845,10 +907,11 @@ def summary(pid: int) -> dict:
     for leg in range(proc.n):
         em.momentum_phys(leg)
     em.emit()
-    sp = SharedProgram(proc, em)
+    sp = program(proc, em)
     sp.emit_tables(pid)
     return dict(flops_amp=em.flops, flops_csum=colour_sum_flops(em.cnum),
-                flops_csum_sym=colour_sum_sym_flops(em.cnum), ncurrents=em.ncurrents,
+                flops_csum_sym=(colour_blocks_flops(colour_blocks(em.perms, em.cnum)[1]) if em.coef.shape[1] == 24
+                                else colour_sum_sym_flops(em.cnum)), ncurrents=em.ncurrents,
                 hs_flops_items=sp.flops_items, hs_flops_amp_hel=sp.flops_amps_hel, hs_ncur=len(sp.order),
                 hs_nslots=sp.nslots, hs_nx=len(sp.xoff), hs_xcap=sp.xcap, hs_nxchunk=len(sp.chunks),
                 ndiagrams=proc.ndiagrams, namps=len(proc.amps), ncolor=em.coef.shape[1],
@@ -1363,6 +1426,9 @@ class SharedProgram:
                     "  }"]
         return [
             "  // helicity-shared program (tables above)",
+            "  static constexpr bool HS_ORDERED = false;",
+            "  static constexpr int HS_GS_POWER = 0;  // couplings are in the currents",
+            "  static constexpr int HS_NSC = 0;",
             "  static constexpr int HS_NSLOT = %d;   // current variant slots per event" % self.nslots,
             "  static constexpr int HS_XCAP = %d;    // amputated-current slots per event and chunk" % self.xcap,
             "  static constexpr int HS_NXCHUNK = %d;" % len(self.chunks),
@@ -1568,3 +1634,360 @@ class SharedProgram:
             lines.append("      } break;")
         lines += ["      default: break;", "    }", "  }"]
         return lines
+
+
+# ---------------------------------------------------------------------------
+# Ordered program (g g -> t t~ g g): the colour-flow amplitudes J_s from off-shell
+# currents that are summed before they are contracted.
+# ---------------------------------------------------------------------------
+# J_s of the chain (T^{a_1} T^{a_2} T^{a_3} T^{a_4})_{top, antitop} is the colour-
+# ordered amplitude A(q, 1, 2, 3, 4, Q) (q top, Q antitop, all outgoing).  With the
+# colour-ordered off-shell currents (Berends and Giele, Nucl. Phys. B306 (1988) 759)
+#   R(w)  top line with the gluons w attached in this order, C(w) antitop line,
+#   G(w)  gluon line of the gluons w, V = gluon line of the pair (q, Q),
+# every planar diagram of six legs has either one line that splits the legs 3 | 3 or a
+# vertex whose branches have two legs each (or a four-gluon vertex with branches
+# 2, 2, 1, 1), so that
+#   A(1234) = R(12) . C(34)  +  B(1) . G(234)  +  B'(4) . G(123)
+#           + G(23) . (R(1) gamma C(4))  +  V . [G(12), G(34)]
+#           + {V, 1, 2, G(34)} + {V, 1, G(23), 4} + {V, G(12), 3, 4}
+# with B(1) = the vector vertex (R(1) gamma v) - V3(V, 1), B'(4) = (u gamma C(4)) -
+# V3(4, V), amputated.  Gluon lines are Lie elements: G(ab) = -G(ba), G(abc) = G(cba),
+# G(abc) + G(bca) + G(cab) = 0, so each set of gluons needs (n - 1)! of its words and
+# one contraction feeds several flows.  123 diagrams (159 amplitude terms) take 55
+# contractions per helicity.
+#
+# Real form: with the coupling and one factor i per vertex and propagator taken out
+# (a quark-gluon vertex i g, an ordered three-gluon vertex -i g, an ordered four-gluon
+# vertex -i g^2, propagators i / D and -i / K^2), the currents are
+#   G = -(V3 + V4) / K^2,   R = -(sum R G/) (K/ + m) / D,   V = (u gamma v) / K^2,
+# amputated quark-gluon vertices enter with +1, gluon vertices with -1, and
+# J = i g^4 A: |M|^2 = g^8 (the sum of the A's), applied to the result in FP64.
+
+
+class OrderedProgram:
+    # device item types (csrc/mg_types.cuh)
+    T_ROW1, T_COL1, T_PAIR, T_GG, T_ROW2, T_COL2, T_G3, T_VB, T_W, T_P, T_DOT = range(15, 26)
+    COST = {"row1": 164, "col1": 164, "pair": 64, "gg": 164, "row2": 404, "col2": 212, "g3": 716, "vb": 228,
+            "w": 56, "p": 156, "dot": 30}
+
+    def __init__(self, proc: Process, emitter: "Emitter"):
+        self.p, self.em, self.n = proc, emitter, proc.n
+        self.q, self.Q = 2, 3
+        self.gl = proc.gluon_legs()
+        assert len(self.gl) == 4 and proc.spec.root == self.Q
+        self.cur, self.x, self.sc = {}, {}, {}      # name -> (first slot or scalar, legs)
+        self.nslots = self.nx = self.nsc = 0
+        self.levels, self.xitems, self.ext = [[], []], [], []
+        self.kinds = []
+        self._program()
+
+    # ---- storage and momenta -------------------------------------------------
+    def _add(self, table, name, legs):
+        """Slots (or scalars) of every variant of `name`, over the legs in ascending order."""
+        legs = tuple(sorted(legs))
+        n = 1 << len(legs)
+        at = {id(self.cur): "nslots", id(self.x): "nx", id(self.sc): "nsc"}[id(table)]
+        table[name] = (getattr(self, at), legs)
+        setattr(self, at, getattr(self, at) + n)
+        return n
+
+    @staticmethod
+    def _sub(child, parent, v):
+        """Variant over `child` legs inside variant v over `parent` legs (ascending bits)."""
+        return sum(((v >> parent.index(l)) & 1) << k for k, l in enumerate(child))
+
+    def _at(self, table, name, parent, v):
+        first, legs = table[name]
+        return first + self._sub(legs, parent, v)
+
+    def _k(self, legs):
+        return self.em.momentum(tuple(sorted(legs)))
+
+    def _prop(self, legs, kind):
+        legs = frozenset(legs)
+        if self.Q in legs:  # the invariant from the side without the antitop
+            legs = frozenset(range(self.n)) - legs
+        return self.em.prop(legs, kind)
+
+    def _item(self, to, t, out, ins=(), k0=0, k1=0, prop=0, a=0, b=0, c=0, flag=0, kind=None, ext=None):
+        ins = list(ins) + [0] * (4 - len(ins))
+        if ext is not None:
+            ins[3] = len(self.ext)
+            self.ext.append(ext)
+        if ins[3]:  # a fourth operand, or the index of the extension, in place of the external parameters
+            assert not (a or b)
+            a, b = (w - 256 if w > 127 else w for w in (ins[3] & 255, ins[3] >> 8))
+        to.append((t, a, b, c, flag, out, ins[:3], k0, k1, prop))
+        if kind:
+            self.kinds.append(kind)
+
+    # ---- the program ---------------------------------------------------------------
+    def _program(self):
+        em, spec, q, Q, gl = self.em, self.p.spec, self.q, self.Q, self.gl
+        cur, x, sc = self.cur, self.x, self.sc
+        L0, L1 = self.levels
+        G = lambda *w: "G" + "".join("%d" % l for l in w)
+        # external wavefunctions
+        for l in range(self.n):
+            name = {q: "q", Q: "Q"}.get(l, G(l))
+            self._add(cur, name, (l,))
+            S = spec.legs[l]
+            t = 2 if S.kind == "g" else (0 if _is_col(S.kind) else 1)
+            c = (1 if S.incoming else -1) if S.kind == "g" else (1 if S.particle else -1)
+            for v in (0, 1):
+                self._item(L0, t, cur[name][0] + v, k0=em.momentum_phys(l), a=l, b=1 if v else -1, c=c,
+                           flag=1 if S.mass == "mt" else 0)
+        # two-leg currents
+        pairs = list(itertools.combinations(gl, 2))
+        for a, b in pairs:
+            legs = (a, b)
+            for v in range(self._add(cur, G(a, b), legs)):
+                self._item(L1, self.T_GG, cur[G(a, b)][0] + v,
+                           [self._at(cur, G(l), legs, v) for l in (a, b)], self._k((a,)), self._k((b,)),
+                           self._prop(legs, "g"), kind="gg")
+        for name, end, t in (("R", q, self.T_ROW1), ("C", Q, self.T_COL1)):
+            for g in gl:
+                legs = tuple(sorted((end, g)))
+                nm = "%s%d" % (name, g)
+                for v in range(self._add(cur, nm, legs)):
+                    self._item(L1, t, cur[nm][0] + v,
+                               [self._at(cur, "q" if end == q else "Q", legs, v), self._at(cur, G(g), legs, v)],
+                               self._k(legs), 0, self._prop(legs, "t"), kind="row1" if end == q else "col1")
+        vq = tuple(sorted((q, Q)))
+        for v in range(self._add(cur, "V", vq)):
+            self._item(L1, self.T_PAIR, cur["V"][0] + v, [self._at(cur, "q", vq, v), self._at(cur, "Q", vq, v)],
+                       prop=self._prop(vq, "g"), kind="pair")
+        # ---- what the contractions read besides the two-leg currents -----------------
+        X = self.xitems
+        words = list(itertools.permutations(gl, 2))
+        # three-gluon currents: words (i j k) and (i k j) of each set i < j < k
+        for tri in itertools.combinations(gl, 3):
+            i, j, k = tri
+            self._add(x, G(i, j, k), tri)
+            self._add(x, G(i, k, j), tri)
+            for v in range(8):
+                s = lambda *w: self._at(cur, G(*w), tri, v)
+                self._item(X, self.T_G3, x[G(i, j, k)][0] + v, [s(i), s(j), s(k)],
+                           ext=([s(i, j), s(i, k), s(j, k)],
+                                [self._k(w) for w in ((i,), (j,), (k,), (i, j), (i, k), (j, k))]),
+                           prop=self._prop(tri, "g"), kind="g3")
+        # vector vertices B(g) (first gluon) and B'(g) (last gluon)
+        kV = self._k(vq)
+        for first in (True, False):
+            for g in gl:
+                legs = tuple(sorted((q, Q, g)))
+                nm = ("B%d" if first else "D%d") % g
+                for v in range(self._add(x, nm, legs)):
+                    at = lambda n_: self._at(cur, n_, legs, v)
+                    f = [at("R%d" % g), at("Q")] if first else [at("q"), at("C%d" % g)]
+                    gv = [(at("V"), kV), (at(G(g)), self._k((g,)))]
+                    if not first:
+                        gv.reverse()
+                    # operands: row, column, then the two gluon lines in cyclic order
+                    self._item(X, self.T_VB, x[nm][0] + v, f + [gv[0][0], gv[1][0]], gv[0][1], gv[1][1], kind="vb")
+        # [G(ab), G(cd)]: the three pairings of the gluons, a the first of them
+        self.pairings = [((gl[0], b), tuple(g for g in gl[1:] if g != b)) for b in gl[1:]]
+        four = tuple(gl)
+        for ab, cd in self.pairings:
+            nm = "P" + G(*ab)
+            for v in range(self._add(x, nm, four)):
+                self._item(X, self.T_P, x[nm][0] + v, [self._at(cur, G(*ab), four, v), self._at(cur, G(*cd), four, v)],
+                           self._k(ab), self._k(cd), kind="p")
+        # R(ab) and R(ba), amputated C(ab) and C(ba): one item for both words (a < b), which share
+        # the term with G(ab) = -G(ba)
+        for nm, end, t in (("R", q, self.T_ROW2), ("C", Q, self.T_COL2)):
+            for a, b in pairs:
+                legs = tuple(sorted((end, a, b)))
+                self._add(x, "%s%d%d" % (nm, a, b), legs)
+                self._add(x, "%s%d%d" % (nm, b, a), legs)
+                # row: R(a) G(b), R(b) G(a); column: C(b) G(a), C(a) G(b)
+                f, g = (a, b) if end == q else (b, a)
+                for v in range(8):
+                    at = lambda n_: self._at(cur, n_, legs, v)
+                    self._item(X, t, x["%s%d%d" % (nm, a, b)][0] + v,
+                               [at("%s%d" % (nm, f)), at(G(g)), at("q" if end == q else "Q")],
+                               ext=([at("%s%d" % (nm, g)), at(G(f)), at(G(a, b))], [0] * 6),
+                               k0=self._k(legs) if end == q else 0, prop=self._prop(legs, "t") if end == q else 0,
+                               kind="row2" if end == q else "col2")
+        # R(a) gamma C(b)
+        for a, b in words:
+            legs = tuple(sorted((q, Q, a, b)))
+            nm = "W%d%d" % (a, b)
+            for v in range(self._add(x, nm, legs)):
+                at = lambda n_: self._at(cur, n_, legs, v)
+                self._item(X, self.T_W, x[nm][0] + v, [at("R%d" % a), at("C%d" % b)], kind="w")
+        # scalar products of gluon lines (four-gluon vertices)
+        def dot(m, n, legs):
+            nm = m + "." + n
+            for v in range(self._add(sc, nm, legs)):
+                self._item(X, self.T_DOT, sc[nm][0] + v, [self._at(cur, m, tuple(sorted(legs)), v),
+                                                         self._at(cur, n, tuple(sorted(legs)), v)], kind="dot")
+        for a, b in pairs:
+            dot(G(a), G(b), (a, b))
+        for g in gl:
+            dot("V", G(g), (q, Q, g))
+        for a, b in pairs:
+            dot("V", G(a, b), (q, Q, a, b))
+        for a, b in pairs:
+            for g in gl:
+                if g not in (a, b):
+                    dot(G(g), G(a, b), (g, a, b))
+        self.xcap = self.nx
+        self.chunks = [list(x)]
+        self.xoff = {nm: x[nm][0] for nm in x}
+        self.order = list(cur)
+        self.flops_items = (sum({0: FLOPS["ixxxxx"], 1: FLOPS["oxxxxx"], 2: FLOPS["vxxxxx"]}[t[0]] for t in L0)
+                            + sum(self.COST[k] for k in self.kinds))
+
+    # ---- emission -----------------------------------------------------------------------
+    def emit_tables(self, pid: int) -> list:
+        nh = 1 << self.n
+        items = self.levels[0] + self.levels[1] + self.xitems
+        level_start = [0, len(self.levels[0]), len(self.levels[0]) + len(self.levels[1])]
+        xitem_start = [level_start[-1], len(items)]
+        self.contract = self._contract_code()
+        self.tables = dict(nitems=len(items), level_start=level_start, xitem_start=xitem_start)
+        assert self.nslots < 65536 and self.xcap < 65536 and self.nsc < 65536
+        out = ["// ordered program: %d current slots, %d slots and %d scalars for the contractions; %d flops per"
+               " event (all helicities)" % (self.nslots, self.xcap, self.nsc, self.flops_items + nh * self.flops_amps_hel)]
+        out.append("static __device__ const HsItem kHsItems%d[%d] = {%s};" % (
+            pid, len(items), ", ".join("{%d, {%s}, %d, %d, %d, %d, %d, %d, %d, %d}" % (
+                o, ", ".join(map(str, ins)), t, a, b, c, flag, k0, k1, pr)
+                for (t, a, b, c, flag, o, ins, k0, k1, pr) in items)))
+        out.append("// items with two words: three further operand slots; three-gluon: momenta of i, j, k, ij, ik, jk")
+        out.append("static __device__ const HsItemExt kHsExt%d[%d] = {%s};" % (
+            pid, len(self.ext), ", ".join("{{%s}, {%s}}" % (", ".join(map(str, s)), ", ".join(map(str, k)))
+                                          for s, k in self.ext)))
+        out.append("static __constant__ int kHsXItem%d[2] = {%d, %d};  // item range of the contractions' operands"
+                   % (pid, xitem_start[0], xitem_start[1]))
+        var = []
+        for S in range(1 << self.n):
+            for ih in range(nh):
+                v = k = 0
+                for l in range(self.n):
+                    if S >> l & 1:
+                        v |= ((ih >> (self.n - 1 - l)) & 1) << k
+                        k += 1
+                var.append(v)
+        out.append("static __device__ __align__(16) const uint8_t kHsVar%d[%d] = {%s};  // [leg set][helicity]"
+                   % (pid, len(var), ", ".join(map(str, var))))
+        return out
+
+    def struct_lines(self, pid: int) -> list:
+        t = self.tables
+        lv = t["level_start"]
+        return [
+            "  // ordered program (tables above)",
+            "  static constexpr bool HS_ORDERED = true;",
+            "  static constexpr int HS_GS_POWER = %d;  // |M|^2 carries g_s to this power, applied to the sum" % (2 * len(self.gl)),
+            "  static constexpr int HS_NSLOT = %d;   // current variant slots per event" % self.nslots,
+            "  static constexpr int HS_XCAP = %d;    // slots per event of the contractions' further operands" % self.xcap,
+            "  static constexpr int HS_NSC = %d;     // scalar products per event" % self.nsc,
+            "  static constexpr int HS_NXCHUNK = 1;",
+            "  static constexpr int HS_XBUFS = 1;",
+            "  static constexpr int HS_NITEM = %d;" % t["nitems"],
+            "  static constexpr int HS_NLEVEL = %d;" % (len(lv) - 1),
+            "  // operations: items per event, contractions + flow sums per helicity",
+            "  static constexpr long HS_FLOPS_ITEMS = %d;" % self.flops_items,
+            "  static constexpr long HS_FLOPS_AMP_HEL = %d;" % self.flops_amps_hel,
+            "  static __host__ __device__ constexpr int hs_level(int i) {",
+            "    constexpr int t[%d] = {%s};" % (len(lv), ", ".join(map(str, lv))),
+            "    return t[i];",
+            "  }",
+            "  static __device__ __forceinline__ int hs_xitem(int c) { return kHsXItem%d[c]; }" % pid,
+            "  static __device__ __forceinline__ const uint8_t* hs_variants() { return kHsVar%d; }" % pid,
+            "  static __device__ __forceinline__ const HsItem* hs_items() { return kHsItems%d; }" % pid,
+            "  static __device__ __forceinline__ const HsItemExt* hs_item_ext() { return kHsExt%d; }" % pid,
+        ] + self.contract
+
+    def _contract_code(self) -> list:
+        nh = 1 << self.n
+        gl = self.gl
+        index = {tuple(gl[k] for k in p): i for i, p in enumerate(itertools.permutations(range(4)))}
+        G = lambda *w: "G" + "".join("%d" % l for l in w)
+        flops = 0
+        started = set()
+
+        def ref(table, nm):
+            first, legs = table[nm]
+            arr = {id(self.cur): "cur[%d + vt[%d]]", id(self.x): "xb[%d + vt[%d]]",
+                   id(self.sc): "xb.scalar(%d + vt[%d])"}[id(table)]
+            return arr % (first, sum(1 << l for l in legs) * nh)
+
+        def add(word, sign, a):
+            nonlocal flops
+            s = index[tuple(word)]
+            flops += 2
+            return "flow_add<%d>(J[%d], %s);" % (0 if sign > 0 else 1, s, a)
+
+        L = ["  // J_s of one helicity: operands cur[..] (currents), xb[..] and xb.scalar(..), variant of a leg",
+             "  // set S for this helicity = vt[S * NHEL]; J in the order of the colour chains",
+             "  template <class R, class CUR, class XB>",
+             "  static __device__ __forceinline__ void hs_contract(int, const CUR& cur, const XB& xb,"
+             " const uint8_t* __restrict__ vt, cx<R>* J) {"]
+        # R(ab) . C(cd): one per flow, the first term of its sum
+        for ab in itertools.combinations(gl, 2):
+            cd = tuple(g for g in gl if g not in ab)
+            L.append("    {")
+            for i, (c, d) in enumerate(itertools.permutations(cd)):
+                L.append("      const W4<R> C%d = %s;" % (i, ref(self.x, "C%d%d" % (c, d))))
+            for (a, b) in itertools.permutations(ab):
+                L.append("      { const W4<R> X = %s;" % ref(self.x, "R%d%d" % (a, b)))
+                for i, (c, d) in enumerate(itertools.permutations(cd)):
+                    L.append("        J[%d] = dot4p(X, C%d);" % (index[(a, b, c, d)], i))
+                    flops += 30
+                L.append("      }")
+            L.append("    }")
+        # B(i) . G(jkl) and B'(i) . G(jkl): with c1 = G(j k l), c2 = G(j l k), j < k < l:
+        # G(k j l) = -(c1 + c2), G(w reversed) = G(w)
+        for nm, last in (("B", False), ("D", True)):
+            for i in gl:
+                j, k, l = [g for g in gl if g != i]
+                wd = lambda *w: (list(w) + [i]) if last else ([i] + list(w))
+                L.append("    { const W4<R> X = %s;" % ref(self.x, "%s%d" % (nm, i)))
+                L.append("      const cx<R> a = dot4p(X, %s), b = dot4p(X, %s), c = a + b;"
+                         % (ref(self.x, G(j, k, l)), ref(self.x, G(j, l, k))))
+                flops += 62
+                L.append("      " + " ".join([add(wd(j, k, l), 1, "a"), add(wd(l, k, j), 1, "a"),
+                                              add(wd(j, l, k), 1, "b"), add(wd(k, l, j), 1, "b"),
+                                              add(wd(k, j, l), -1, "c"), add(wd(l, j, k), -1, "c")]))
+                L.append("    }")
+        # V parts and the four-gluon vertices with V; then G(bc) . W(x, y)
+        L.append("    HS_FENCE();")
+        L.append("    {")
+        for ab, cd in self.pairings:
+            nm = "P" + G(*ab)
+            for pair, other, sg in ((cd, ab, 1), (ab, cd, 0)):
+                b, c = pair
+                xx, yy = other
+                # s, t, u = (V.bc)(x.y), (V.x)(y.bc), (V.y)(x.bc); the vertex with branches V, bc, x, y has
+                # 2 (product of the opposite branches) - the other two products
+                L.append("      { const cx<R> s = %s * %s, t = %s * %s, u = %s * %s;" % (
+                    ref(self.sc, "V." + G(b, c)), ref(self.sc, G(xx) + "." + G(yy)),
+                    ref(self.sc, "V." + G(xx)), ref(self.sc, G(yy) + "." + G(b, c)),
+                    ref(self.sc, "V." + G(yy)), ref(self.sc, G(xx) + "." + G(b, c))))
+                L.append("        const cx<R> w = s + t + u;")
+                flops += 18 + 4
+                if sg:  # V . [G(xy), G(bc)] joins this pair's terms
+                    L.append("        const cx<R> p = dot4p(%s, %s);" % (ref(self.cur, "V"), ref(self.x, nm)))
+                    L.append("        const cx<R> ly = vertex4(u, w) + p, lx = vertex4(t, w) - p, lb = vertex4(s, w);")
+                    flops += 30 + 4 + 12
+                else:
+                    L.append("        const cx<R> ly = vertex4(u, w), lx = vertex4(t, w), lb = vertex4(s, w);")
+                    flops += 12
+                for w_, sgn, a in (((xx, yy, b, c), 1, "ly"), ((xx, yy, c, b), -1, "ly"), ((b, c, yy, xx), 1, "ly"),
+                                   ((c, b, yy, xx), -1, "ly"), ((yy, xx, b, c), 1, "lx"), ((yy, xx, c, b), -1, "lx"),
+                                   ((b, c, xx, yy), 1, "lx"), ((c, b, xx, yy), -1, "lx")):
+                    L.append("        " + add(w_, sgn, a))
+                L.append("        const W4<R> Y = %s;" % ref(self.cur, G(b, c)))
+                L.append("        { const cx<R> a = lb + dot4p(Y, %s);" % ref(self.x, "W%d%d" % (xx, yy)))
+                L.append("          " + add((xx, b, c, yy), 1, "a") + " " + add((xx, c, b, yy), -1, "a") + " }")
+                L.append("        { const cx<R> a = lb + dot4p(Y, %s);" % ref(self.x, "W%d%d" % (yy, xx)))
+                L.append("          " + add((yy, b, c, xx), 1, "a") + " " + add((yy, c, b, xx), -1, "a") + " }")
+                flops += 64
+                L.append("      }")
+                L.append("      HS_FENCE();")
+        L += ["    }", "  }"]
+        self.flops_amps_hel = flops
+        return L
