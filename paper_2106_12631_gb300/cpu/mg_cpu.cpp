@@ -129,7 +129,7 @@ inline void ord_item(const mg::HsItem& it, mg::W4<R>* cur, mg::W4<R>* xb, mg::cx
   switch (it.type) {
     case 15: cur[it.out] = FFV1_2<R>(cur[it.in[0]], cur[it.in[1]], one, K + 4 * it.k0, cp.mt, pr[it.prop]); return;
     case 16: cur[it.out] = FFV1_1<R>(cur[it.in[0]], cur[it.in[1]], one, K + 4 * it.k0, cp.mt, pr[it.prop]); return;
-    case 17: cur[it.out] = w4_rscale(ord_pair(cur[it.in[0]], cur[it.in[1]]), -pr[it.prop].im); return;
+    case 17: cur[it.out] = w4_rscale(vector_pair(cur[it.in[0]], cur[it.in[1]]), -pr[it.prop].im); return;
     case 18:
       cur[it.out] = w4_rscale(ord_v3(cur[it.in[0]], cur[it.in[1]], K + 4 * it.k0, K + 4 * it.k1), pr[it.prop].im);
       return;
@@ -154,10 +154,10 @@ inline void ord_item(const mg::HsItem& it, mg::W4<R>* cur, mg::W4<R>* xb, mg::cx
       return;
     }
     case 22:
-      xb[it.out] = w4_lower(w4_sub(ord_pair(cur[it.in[0]], cur[it.in[1]]),
+      xb[it.out] = w4_lower(w4_sub(vector_pair(cur[it.in[0]], cur[it.in[1]]),
                                    ord_v3(cur[it.in[2]], cur[it.in3()], K + 4 * it.k0, K + 4 * it.k1)));
       return;
-    case 23: xb[it.out] = w4_lower(ord_pair(cur[it.in[0]], cur[it.in[1]])); return;
+    case 23: xb[it.out] = w4_lower(vector_pair(cur[it.in[0]], cur[it.in[1]])); return;
     case 24: {
       W4<R> o = ord_v3(cur[it.in[0]], cur[it.in[1]], K + 4 * it.k0, K + 4 * it.k1);
       o.w[0] = -o.w[0];

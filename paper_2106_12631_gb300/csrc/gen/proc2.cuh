@@ -22,8 +22,8 @@ struct Proc2 {
   static constexpr int HS_NSC = 0;
   static constexpr int HS_NSLOT = 20;   // current variant slots per event
   static constexpr int HS_XCAP = 12;    // amputated-current slots per event and chunk
+  static constexpr int HS_NVT = 16;
   static constexpr int HS_NXCHUNK = 1;
-  static constexpr int HS_XBUFS = 1;   // chunk buffers
   static constexpr int HS_NITEM = 32;
   static constexpr int HS_NLEVEL = 2;
   static constexpr int HS_NAMP = 3;

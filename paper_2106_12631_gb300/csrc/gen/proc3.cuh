@@ -22,8 +22,8 @@ struct Proc3 {
   static constexpr int HS_NSC = 0;
   static constexpr int HS_NSLOT = 94;   // current variant slots per event
   static constexpr int HS_XCAP = 100;    // amputated-current slots per event and chunk
+  static constexpr int HS_NVT = 32;
   static constexpr int HS_NXCHUNK = 1;
-  static constexpr int HS_XBUFS = 1;   // chunk buffers
   static constexpr int HS_NITEM = 194;
   static constexpr int HS_NLEVEL = 3;
   static constexpr int HS_NAMP = 18;

@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(HsGradCfg<P, R>::NT) sigmakin_hs_grad_kernel(G
     return;
   }
   // 2. forward: tables, currents, amputated currents, contractions, colour sum
-  hs_tables<P, R, L>(smem, a.pp, HsGroup{0, NT, tid, 0, nev, 0}, curs, cp);
+  hs_tables<P, R, L>(smem, a.pp, nev, curs, cp);
   const HsItem* items = P::hs_items();
 #pragma unroll
   for (int l = 1; l < P::HS_NLEVEL; ++l) {

@@ -186,6 +186,21 @@ __device__ __forceinline__ W4<R> bilinear(const W4<R>& f, const W4<R>& g, R gl, 
   return j;
 }
 
+// row . gamma^mu . col, upper index
+template <class R>
+__device__ __forceinline__ W4<R> vector_pair(const W4<R>& f, const W4<R>& g) {
+  W4<R> j;
+  const cx<R> ap = cfma(f.w[1], g.w[3], f.w[0] * g.w[2]), am = cfma(-f.w[1], g.w[3], f.w[0] * g.w[2]);
+  const cx<R> xp = cfma(f.w[1], g.w[2], f.w[0] * g.w[3]), xm = cfma(f.w[1], g.w[2], -(f.w[0] * g.w[3]));
+  const cx<R> bp = cfma(f.w[3], g.w[1], f.w[2] * g.w[0]), bm = cfma(f.w[3], g.w[1], -(f.w[2] * g.w[0]));
+  const cx<R> yp = cfma(f.w[3], g.w[0], f.w[2] * g.w[1]), ym = cfma(-f.w[3], g.w[0], f.w[2] * g.w[1]);
+  j.w[0] = ap + bp;
+  j.w[1] = xp - yp;
+  j.w[2] = mul_i(xm + ym);
+  j.w[3] = am + bm;
+  return j;
+}
+
 // ---- amplitude routines -----------------------------------------------------
 // i g  row . V/ . col  (fermion-fermion-vector vertex, vector coupling)
 template <class R>
@@ -243,7 +258,7 @@ __device__ __forceinline__ W4<R> FFV1_1(const W4<R>& fi, const W4<R>& v, R g, co
 // off-shell vector from a fermion pair:  i g (row . gamma^mu . col) prop
 template <class R>
 __device__ __forceinline__ W4<R> FFV1P0_3(const W4<R>& fo, const W4<R>& fi, R g, cx<R> prop) {
-  return scale(bilinear(fo, fi, R(1), R(1)), mul_i(g * prop));
+  return scale(vector_pair(fo, fi), mul_i(g * prop));
 }
 // off-shell Z from a lepton pair: -i gz (row . gamma^mu (gl PL + gr PR) . col) prop
 template <class R>
@@ -319,7 +334,7 @@ __device__ __forceinline__ W4<R> FFV1_1A(const W4<R>& fi, const W4<R>& v, R g) {
 // i g (row . gamma_mu . col)
 template <class R>
 __device__ __forceinline__ W4<R> FFV1P0_3A(const W4<R>& fo, const W4<R>& fi, R g) {
-  const W4<R> j = bilinear(fo, fi, R(1), R(1));
+  const W4<R> j = vector_pair(fo, fi);
   W4<R> o;
   o.w[0] = mul_i(g * j.w[0]);
 #pragma unroll
@@ -540,20 +555,6 @@ __device__ __forceinline__ W4<R> w4_lower(const W4<R>& a) {
 #pragma unroll
   for (int k = 1; k < 4; ++k) o.w[k] = -a.w[k];
   return o;
-}
-// row . gamma^mu . col, upper index
-template <class R>
-__device__ __forceinline__ W4<R> ord_pair(const W4<R>& f, const W4<R>& g) {
-  W4<R> j;
-  const cx<R> ap = cfma(f.w[1], g.w[3], f.w[0] * g.w[2]), am = cfma(-f.w[1], g.w[3], f.w[0] * g.w[2]);
-  const cx<R> xp = cfma(f.w[1], g.w[2], f.w[0] * g.w[3]), xm = cfma(f.w[1], g.w[2], -(f.w[0] * g.w[3]));
-  const cx<R> bp = cfma(f.w[3], g.w[1], f.w[2] * g.w[0]), bm = cfma(f.w[3], g.w[1], -(f.w[2] * g.w[0]));
-  const cx<R> yp = cfma(f.w[3], g.w[0], f.w[2] * g.w[1]), ym = cfma(-f.w[3], g.w[0], f.w[2] * g.w[1]);
-  j.w[0] = ap + bp;
-  j.w[1] = xp - yp;
-  j.w[2] = mul_i(xm + ym);
-  j.w[3] = am + bm;
-  return j;
 }
 // the two words of a three-gluon current: G(ijk) and G(ikj) (up to the common
 // factor): V3 of the pair currents and V4(A,B,C) = (B.C) A + (A.B) C - 2 (A.C) B

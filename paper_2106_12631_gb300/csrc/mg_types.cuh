@@ -40,6 +40,46 @@ template <class R> __device__ __forceinline__ cx<R> rfma(R s, cx<R> a, cx<R> c) 
   return cx<R>(fmac(s, a.re, c.re), fmac(s, a.im, c.im));
 }
 
+// Two events side by side: the mixed mode's kernels evaluate a pair of events
+// per thread, so that every FP32 operation is one paired instruction (FFMA2,
+// FADD2, FMUL2: two results per issue slot; operand signs and a scalar repeated
+// in both halves cost nothing).  The arithmetic of each event is that of a
+// single float.
+struct alignas(8) f2 {
+  float x, y;
+  f2() = default;
+  __host__ __device__ constexpr f2(float a, float b) : x(a), y(b) {}
+  __host__ __device__ explicit constexpr f2(float a) : x(a), y(a) {}
+  __host__ __device__ explicit constexpr f2(double a) : x((float)a), y((float)a) {}
+  __host__ __device__ explicit constexpr f2(int a) : x((float)a), y((float)a) {}
+};
+__device__ __forceinline__ float2 f2_raw(f2 a) { return make_float2(a.x, a.y); }
+__device__ __forceinline__ f2 f2_of(float2 a) { return f2(a.x, a.y); }
+__device__ __forceinline__ f2 operator-(f2 a) { return f2(-a.x, -a.y); }
+__device__ __forceinline__ f2 operator+(f2 a, f2 b) { return f2_of(__fadd2_rn(f2_raw(a), f2_raw(b))); }
+__device__ __forceinline__ f2 operator-(f2 a, f2 b) { return f2_of(__fadd2_rn(f2_raw(a), f2_raw(-b))); }
+__device__ __forceinline__ f2 operator*(f2 a, f2 b) { return f2_of(__fmul2_rn(f2_raw(a), f2_raw(b))); }
+__device__ __forceinline__ f2& operator+=(f2& a, f2 b) { a = a + b; return a; }
+__device__ __forceinline__ f2& operator-=(f2& a, f2 b) { a = a - b; return a; }
+__device__ __forceinline__ f2 operator/(f2 a, f2 b) { return f2(a.x / b.x, a.y / b.y); }
+__device__ __forceinline__ f2 fmac(f2 a, f2 b, f2 c) { return f2_of(__ffma2_rn(f2_raw(a), f2_raw(b), f2_raw(c))); }
+__device__ __forceinline__ cx<f2> operator*(cx<f2> a, cx<f2> b) {
+  return cx<f2>(fmac(-a.im, b.im, a.re * b.re), fmac(a.im, b.re, a.re * b.im));
+}
+// scalar type and events of a lane type; value of one event
+template <class V>
+struct LaneOf {
+  using scalar = V;
+  static constexpr int EW = 1;
+};
+template <>
+struct LaneOf<f2> {
+  using scalar = float;
+  static constexpr int EW = 2;
+};
+template <class V> __host__ __device__ __forceinline__ V lane_value(V v, int) { return v; }
+__host__ __device__ __forceinline__ float lane_value(f2 v, int i) { return i == 0 ? v.x : v.y; }
+
 // Four complex components: a Dirac spinor (chiral basis, upper pair
 // left-handed; a row spinor for flowing-out fermions, a column spinor for
 // flowing-in ones) or a Lorentz vector with upper index.  The paper's
@@ -69,6 +109,14 @@ struct Slots {
     const uint4* s = reinterpret_cast<const uint4*>(&w);
 #pragma unroll
     for (int k = 0; k < NPL; ++k) p[i + k * N] = s[k];
+  }
+  // one event's values of a slot (lane of V)
+  template <class S>
+  __device__ __forceinline__ void set_lane(int i, int lane, const W4<S>& w) const {
+    constexpr int EW = LaneOf<R>::EW, PER = (int)(16 / sizeof(R));
+    const S* v = reinterpret_cast<const S*>(&w);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) reinterpret_cast<S*>(p + i + (k / PER) * N)[(k % PER) * EW + lane] = v[k];
   }
   // slot i += w, component by component with shared-memory atomics (adjoint
   // accumulation from many threads)
@@ -111,6 +159,15 @@ struct PlanarSlots {
 #pragma unroll
     for (int k = 0; k < NPL; ++k) p[i + k * N] = *reinterpret_cast<const uint4*>(v + k * PER);
   }
+  template <class S>
+  __device__ __forceinline__ void set_lane(int i, int lane, const W4<S>& w) const {
+    constexpr int EW = LaneOf<R>::EW;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const S v = c < 4 ? w.w[c & 3].re : w.w[c & 3].im;
+      reinterpret_cast<S*>(p + i + (c / PER) * N)[(c % PER) * EW + lane] = v;
+    }
+  }
   __device__ __forceinline__ cx<R> scalar(int i) const { return reinterpret_cast<const cx<R>*>(p + N * NPL)[i]; }
   __device__ __forceinline__ void set_scalar(int i, cx<R> x) const { reinterpret_cast<cx<R>*>(p + N * NPL)[i] = x; }
 };
@@ -126,6 +183,11 @@ struct Couplings {
   R gzr;   // Z right coupling, -Q sin^2 theta_W
   R mt;    // top mass
 };
+
+template <class V, class S>
+__device__ __forceinline__ Couplings<V> lane_couplings(const Couplings<S>& c) {
+  return {V(c.gs), V(c.gs2), V(c.ee), V(c.gz), V(c.gzl), V(c.gzr), V(c.mt)};
+}
 
 // Helicity-shared program tables (generated per process).
 // One variant of one off-shell current or amputated current: type (0 ixxxxx,

@@ -11,7 +11,7 @@
 //   * currents and amputated currents are item tables walked by short loops
 //     (lanes take one item for each of the CTA's events); the contractions of
 //     a chunk's amplitudes are generated straight-line code.
-// CTA of NT threads = EV events x ngood helicities.  Phases:
+// CTA of NT threads = units (pairs of events in the mixed mode) x ngood helicities.  Phases:
 //   1. per-event momenta, momentum sums and FP64 propagator factors (as SIGMAKIN);
 //   2. current variants, level by level (a level only reads earlier levels);
 //   3. per chunk of amputated currents: their variants (all threads), then one
@@ -28,17 +28,13 @@
 
 namespace mg {
 
+// threads per CTA of the mixed kernels of six and more colour flows, and their
+// CTAs per SM (six flows; more: one)
 #ifndef MG_HS_NT
 #define MG_HS_NT 256
 #endif
 #ifndef MG_HS_CTAS
-#define MG_HS_CTAS 2  // resident CTAs per SM the shared-memory budget is split for (24+ colour flows)
-#endif
-#ifndef MG_HS_EVENT_SYNC
-#define MG_HS_EVENT_SYNC 0  // 1: per-event barrier groups (HsGroup) instead of CTA barriers
-#endif
-#ifndef MG_HS_CTAS_SMALL
-#define MG_HS_CTAS_SMALL 3  // the same below 24 colour flows (smaller variant sets per event)
+#define MG_HS_CTAS 2
 #endif
 
 // current slots and contraction operands in shared memory: the ordered
@@ -46,22 +42,27 @@ namespace mg {
 template <class P, class R, int N>
 using HsSlots = std::conditional_t<P::HS_ORDERED, PlanarSlots<R, N>, Slots<R, N>>;
 
-// Many-colour processes in FP32: several 256-thread CTAs per SM (two of
-// 4 events x 64 helicities for gg -> t t~ g g, three of 8 x 32 for
-// gg -> t t~ g), so that one CTA's short barrier-bound phases overlap the
-// others' contractions (measured).  FP64 needs more registers per thread:
-// one 256-thread CTA per SM.
-template <class P, class R>
+// Lane type of a kernel: pairs of events (f2) in the mixed mode with the
+// CUDA-core colour sum; the tensor-core colour sum takes one row per thread.
+template <class P, class R, int CS>
+using HsLane = std::conditional_t<std::is_same_v<R, float> && CS == CS_SIMT && (P::NCOLOR > 1), f2, R>;
+
+// CTA shape.  A thread takes one helicity of one unit, a unit being the events
+// of a lane (a pair in the mixed mode).
+template <class P, class R, int CS = CS_SIMT>
 struct HsCfg {
-  static constexpr int NT = P::NCOLOR >= 6 ? (sizeof(R) == 4 ? MG_HS_NT : 256) : 128;
-  static constexpr int EVMIN = (NT / P::NHEL) > 0 ? (NT / P::NHEL) : 1;
-  static constexpr int EVWANT = (4 * EVMIN) < 32 ? 4 * EVMIN : 32;
-  // shared memory for the current variants and one chunk of amputated currents
-  static constexpr int CTAS =
-      P::NCOLOR >= 6 && sizeof(R) == 4 ? (P::NCOLOR >= 24 ? MG_HS_CTAS : MG_HS_CTAS_SMALL) : 1;
+  using V = HsLane<P, R, CS>;
+  static constexpr int EW = LaneOf<V>::EW;
+  static constexpr int NT = P::NCOLOR < 6 ? 128 : EW == 2 ? MG_HS_NT : 256;
+  static constexpr int EVMIN = (NT / P::NHEL) > 0 ? (NT / P::NHEL) : 1;  // units, all helicities good
+  static constexpr int MORE = P::NCOLOR >= 24 ? 1 : EW == 1 || P::NCOLOR == 1 ? 4 : (P::NCOLOR >= 6 ? 1 : 2);
+  static constexpr int EVWANT = (MORE * EVMIN) < 32 ? MORE * EVMIN : 32;
+  // shared memory for the currents and the contractions' operands
+  static constexpr int CTAS = P::NCOLOR < 6 || sizeof(R) != 4 ? 1 : EW == 2 ? (P::NCOLOR >= 24 ? 1 : MG_HS_CTAS)
+                                                             : (P::NCOLOR >= 24 ? 2 : 3);
   static constexpr size_t CUR_BUDGET = 192 * 1024 / CTAS;
   static constexpr size_t EV_BYTES =
-      (size_t)(P::HS_NSLOT + P::HS_XBUFS * P::HS_XCAP) * sizeof(W4<R>) + (size_t)P::HS_NSC * sizeof(cx<R>);
+      (size_t)(P::HS_NSLOT + P::HS_XCAP) * sizeof(W4<V>) + (size_t)P::HS_NSC * sizeof(cx<V>);
   static constexpr int FIT = (int)(CUR_BUDGET / EV_BYTES);
   static constexpr int EVCAP = FIT < EVWANT ? (FIT > EVMIN ? FIT : EVMIN) : EVWANT;
   static constexpr int KP = ((P::NCOLOR + 15) / 16) * 16;
@@ -71,7 +72,9 @@ struct HsCfg {
 
 template <class P, class R, int CS>
 struct HsLayout {
-  using H = HsCfg<P, R>;
+  using H = HsCfg<P, R, CS>;
+  using V = typename H::V;
+  static constexpr int EW = H::EW;
   static constexpr int NT = H::NT, EVCAP = H::EVCAP, KP = H::KP, NP = H::NP, MBLK = H::MBLK;
   static constexpr bool TC = CS == CS_TC;
   static constexpr size_t o_proptab = 0;  // {momentum entry, line kind} per propagator
@@ -82,38 +85,38 @@ struct HsLayout {
   static constexpr size_t o_mconst = align_up(o_misc + 32, 16);
   static constexpr size_t o_p = align_up(o_mconst + 32, 16);
   // the next group's momenta (FP64), copied asynchronously while this group runs
-  static constexpr size_t o_ps = align_up(o_p + 8 * EVCAP * P::NPAR * 4, 16);
-  static constexpr size_t o_K = align_up(o_ps + 8 * EVCAP * P::NPAR * 4, 16);
-  // momentum-table entries (R) from one event to the next: an odd number of
-  // 16-byte words, so that one entry of the CTA's events falls in different
-  // bank groups (the lanes of a warp read it for several events at once)
+  static constexpr size_t o_ps = align_up(o_p + 8 * EW * EVCAP * P::NPAR * 4, 16);
+  static constexpr size_t o_K = align_up(o_ps + 8 * EW * EVCAP * P::NPAR * 4, 16);
+  // momentum-table entries (V) from one unit to the next: an odd number of
+  // 16-byte words, so that one entry of the CTA's units falls in different
+  // bank groups (the lanes of a warp read it for several units at once)
   static constexpr int KEV =
-      4 * P::NMOM + ((4 * P::NMOM * (int)sizeof(R) / 16) % 2 == 0 ? 16 / (int)sizeof(R) : 0);
-  static constexpr size_t o_pr = align_up(o_K + sizeof(R) * EVCAP * KEV, 16);
-  static constexpr size_t o_m2 = align_up(o_pr + 2 * sizeof(R) * EVCAP * P::NPROP, 16);
-  // variant of a leg set for a helicity: vt[S * NHEL + ihel]
-  static constexpr size_t o_vt = align_up(o_m2 + 8 * NT, 16);
-  static constexpr size_t o_U = align_up(o_vt + (size_t(1) << P::NPAR) * P::NHEL, 1024);
-  // union: current variants + amputated chunk (phases 2-3), then the tensor-core
+      4 * P::NMOM + ((4 * P::NMOM * (int)sizeof(V) / 16) % 2 == 0 ? 16 / (int)sizeof(V) : 0);
+  static constexpr size_t o_pr = align_up(o_K + sizeof(V) * EVCAP * KEV, 16);
+  static constexpr size_t o_m2 = align_up(o_pr + 2 * sizeof(V) * EVCAP * P::NPROP, 16);
+  // variant of a leg set for a helicity: vt[row * NHEL + ihel]
+  static constexpr size_t o_vt = align_up(o_m2 + sizeof(R) * EW * NT, 16);
+  static constexpr size_t o_U = align_up(o_vt + (size_t)P::HS_NVT * P::NHEL, TC ? 1024 : 128);
+  // union: current variants + contraction operands (phases 2-3), then the tensor-core
   // A tiles and, after them, the colour matrix as the B operand (phase 4).
-  // Per-event strides in 16-byte words, padded so that one slot of the CTA's
-  // events falls in different bank groups: the lanes of a warp take an item
-  // for several events at once (the plane stride, a multiple of 8 words for
+  // Per-unit strides in 16-byte words, padded so that one slot of the CTA's
+  // units falls in different bank groups: the lanes of a warp take an item
+  // for several units at once (the plane stride, a multiple of 8 words for
   // the processes' slot counts, would otherwise map them to one group).
   static constexpr int EVPAD = EVCAP >= 8 ? 1 : 8 / EVCAP;
-  static constexpr int CUR_EV = P::HS_NSLOT * Slots<R, 1>::NPL + EVPAD;
+  static constexpr int CUR_EV = P::HS_NSLOT * Slots<V, 1>::NPL + EVPAD;
   static constexpr int X_EV =
-      P::HS_XCAP * Slots<R, 1>::NPL + (int)(align_up((size_t)P::HS_NSC * sizeof(cx<R>), 128) / 16) + EVPAD;
+      P::HS_XCAP * Slots<V, 1>::NPL + (int)(align_up((size_t)P::HS_NSC * sizeof(cx<V>), 128) / 16) + EVPAD;
   static constexpr size_t o_cur = o_U;
   static constexpr size_t o_x = o_U + 16 * size_t(EVCAP) * CUR_EV;
   static constexpr size_t o_A = o_U;
   static constexpr size_t tileA = 128 * KP * 2;
-  static constexpr size_t u_bytes = 16 * size_t(EVCAP) * (CUR_EV + P::HS_XBUFS * X_EV);
+  static constexpr size_t u_bytes = 16 * size_t(EVCAP) * (CUR_EV + X_EV);
   static constexpr size_t a_bytes = TC ? 3 * MBLK * tileA : 0;  // one component's three splits
   static constexpr size_t o_B = o_U + a_bytes;  // copied in for every group's colour sum
   static constexpr size_t b_bytes = TC ? size_t(NP) * KP * 2 : 0;
   static constexpr size_t bytes = o_U + (u_bytes > a_bytes + b_bytes ? u_bytes : a_bytes + b_bytes);
-  static_assert(o_B % 1024 == 0, "B operand on a 1024-byte boundary");
+  static_assert(!TC || o_B % 1024 == 0, "B operand on a 1024-byte boundary");
   static constexpr uint32_t TMEM_COLS = tc::tmem_cols(MBLK * 2 * NP);
   static_assert(!TC || NT % 128 == 0, "CTA rows must fill 128-row MMA blocks");
   static_assert(TMEM_COLS <= 512, "TMEM holds 512 columns");
@@ -278,8 +281,8 @@ __device__ __forceinline__ R colour_sum_sym(const cx<R>* J) {
     static_for<i + 1, NC>([&](auto Jc) {
       constexpr int j = decltype(Jc)::value;
       if constexpr (P::cnum(i, j) != 0) {
-        ur += R(2 * P::cnum(i, j)) * J[j].re;
-        ui += R(2 * P::cnum(i, j)) * J[j].im;
+        ur = fmac(R(2 * P::cnum(i, j)), J[j].re, ur);
+        ui = fmac(R(2 * P::cnum(i, j)), J[j].im, ui);
       }
     });
     sum = fmac(J[i].re, ur, fmac(J[i].im, ui, sum));
@@ -287,10 +290,10 @@ __device__ __forceinline__ R colour_sum_sym(const cx<R>* J) {
   return sum / R(P::CDEN);
 }
 
-// Four-point Hadamard transform of every orbit of chains, in place, times s
-// (its own inverse for s = 1/4)
-template <class P, class R>
-__device__ __forceinline__ void colour_hadamard(cx<R>* J, R s) {
+// Four-point Hadamard transform of every orbit of chains, in place; BACK: its
+// inverse (times 1/4)
+template <class P, class R, bool BACK>
+__device__ __forceinline__ void colour_hadamard(cx<R>* J) {
   static_for<0, 6>([&](auto O) {
     constexpr int o = decltype(O)::value;
     cx<R>&a = J[P::colour_orbit(o, 0)], &b = J[P::colour_orbit(o, 1)], &c = J[P::colour_orbit(o, 2)],
@@ -300,7 +303,8 @@ __device__ __forceinline__ void colour_hadamard(cx<R>* J, R s) {
     b = ab - cd;
     c = am + cm;
     d = am - cm;
-    if (s != R(1)) {
+    if constexpr (BACK) {
+      const R s(0.25);
       a = s * a; b = s * b; c = s * c; d = s * d;
     }
   });
@@ -314,7 +318,7 @@ __device__ __forceinline__ R colour_sum(cx<R>* J) {
   if constexpr (!P::COLOUR_BLOCKS) {
     return colour_sum_sym<P, R>(J);
   } else {
-    colour_hadamard<P, R>(J, R(1));
+    colour_hadamard<P, R, false>(J);
     cx<R> tot(R(0), R(0));  // re: sum of the products' real parts; im: of the imaginary parts
     static_for<0, 24>([&](auto I) {
       constexpr int x = decltype(I)::value / 6, i = decltype(I)::value % 6;
@@ -610,89 +614,36 @@ __device__ __forceinline__ void hs_convert_momenta(unsigned char* smem, int nev)
   }
 }
 
-// Barrier domain of the phases after the CTA's first barrier: the threads of
-// one event, or of the events that share one warp, synchronise only among
-// themselves, so the events of a CTA move through their phases independently.
-// With ng good helicities (thread = (event, good helicity)): ng = 64 -> one
-// event per two warps on a named barrier; ng = 32 -> one event per warp; ng a
-// divisor of 32 -> the 32 / ng events of one warp; otherwise, and for the
-// tensor-core colour sum (one MMA spans several events), the whole CTA.
-struct HsGroup {
-  int kind;      // 0 CTA barrier, 1 warp, 2 named barrier
-  int tpg;       // threads per group
-  int j;         // thread index within the group
-  int ev0, nev;  // the group's events (CTA-local)
-  int id;        // named barrier (kind 2)
-  __device__ __forceinline__ void sync() const {
-    if (kind == 0) __syncthreads();
-    else if (kind == 1) __syncwarp();
-    else named_sync();
-  }
-  // barrier ids as immediates, so only the ids in use are reserved
-  __device__ __forceinline__ void named_sync() const {
-    switch (id) {
-      case 1: asm volatile("bar.sync 1, 64;" ::: "memory"); break;
-      case 2: asm volatile("bar.sync 2, 64;" ::: "memory"); break;
-      case 3: asm volatile("bar.sync 3, 64;" ::: "memory"); break;
-      case 4: asm volatile("bar.sync 4, 64;" ::: "memory"); break;
-      case 5: asm volatile("bar.sync 5, 64;" ::: "memory"); break;
-      case 6: asm volatile("bar.sync 6, 64;" ::: "memory"); break;
-      case 7: asm volatile("bar.sync 7, 64;" ::: "memory"); break;
-      default: asm volatile("bar.sync 8, 64;" ::: "memory"); break;
-    }
-  }
-};
-
-template <int NT>
-__device__ __forceinline__ HsGroup hs_group(bool cta_only, int ng, int ev, int nev) {
-  static_assert(NT % 64 == 0 && NT / 64 <= 8, "named barriers 1..8 for the two-warp groups");
-  HsGroup g;
-  int epg;
-  if (cta_only || ng < 1 || !(ng == 64 || 32 % ng == 0)) {
-    g.kind = 0;
-    g.tpg = NT;
-    epg = ev;
-  } else if (ng == 64) {
-    g.kind = 2;
-    g.tpg = 64;
-    epg = 1;
-  } else {
-    g.kind = 1;
-    g.tpg = 32;
-    epg = 32 / ng;
-  }
-  const int grp = (int)threadIdx.x / g.tpg;
-  g.j = (int)threadIdx.x - grp * g.tpg;
-  g.ev0 = grp * epg;
-  g.nev = max(0, min(epg, nev - g.ev0));
-  g.id = 1 + grp;
-  return g;
-}
-
-// CUR_EV: 16-byte words from one event's current variants to the next's;
-// KEV: momentum-table entries (R) from one event's table to the next's
-template <class P, class R, class L, int CUR_EV = P::HS_NSLOT * Slots<R, 1>::NPL, int KEV = 4 * P::NMOM>
-__device__ __forceinline__ void hs_tables(unsigned char* smem, const PhysParams& pp, const HsGroup& grp, uint4* curs,
+// CUR_EV: 16-byte words from one unit's current variants to the next's; KEV:
+// momentum-table entries (V) from one unit's table to the next's.  Events that
+// fill up the last unit repeat the last event's momenta.
+template <class P, class R, class L, class V = R, int CUR_EV = P::HS_NSLOT * Slots<V, 1>::NPL, int KEV = 4 * P::NMOM>
+__device__ __forceinline__ void hs_tables(unsigned char* smem, const PhysParams& pp, int nev, uint4* curs,
                                           const Couplings<R>& cp) {
-  constexpr int NM = P::NMOM, NPAR = P::NPAR;
+  constexpr int NM = P::NMOM, NPAR = P::NPAR, EW = LaneOf<V>::EW;
   constexpr int NEXT = P::hs_level(1);  // external variants
   constexpr bool DF = sizeof(R) == 4;
   const int4* md = reinterpret_cast<const int4*>(smem + L::o_md);
   const int2* prop_tab = reinterpret_cast<const int2*>(smem + L::o_proptab);
-  R* K = reinterpret_cast<R*>(smem + L::o_K);                // [EV][NMOM][4]
-  cx<R>* pr = reinterpret_cast<cx<R>*>(smem + L::o_pr);      // [EV][NPROP]
-  const int nev = grp.nev;
+  R* K = reinterpret_cast<R*>(smem + L::o_K);    // V [unit][NMOM][4]
+  R* pr = reinterpret_cast<R*>(smem + L::o_pr);  // cx<V> [unit][NPROP]
+  const int nep = (nev + EW - 1) / EW * EW;
   // mixed mode: one thread per (event, leg), both helicities (consecutive items)
   static_assert(NEXT == 2 * NPAR, "level 0: two helicities per leg");
   constexpr int NE = DF ? NPAR : NEXT;
-  for (int t = grp.j; t < nev * (NM + NE); t += grp.tpg) {
-    if (t < nev * NM) {
-      const int el = t / NM, j = t - el * NM, e = grp.ev0 + el;
+  for (int t = threadIdx.x; t < nep * (NM + NE); t += L::NT) {
+    const bool mom = t < nep * NM;
+    const int t2 = mom ? t : t - nep * NM, e = t2 / (mom ? NM : NE), j = t2 - e * (mom ? NM : NE);
+    const int u = e / EW, lane = e - u * EW, es = EW == 1 ? e : min(e, nev - 1);
+    if (mom) {
       const int4 d = md[j];
+      auto put = [&](int pj, cx<R> f) {
+        pr[((u * P::NPROP + pj) * 2 + 0) * EW + lane] = f.re;
+        pr[((u * P::NPROP + pj) * 2 + 1) * EW + lane] = f.im;
+      };
       if constexpr (DF) {
-        const float2* q = reinterpret_cast<const float2*>(smem + L::o_p) + e * NPAR * 4;
+        const float2* q = reinterpret_cast<const float2*>(smem + L::o_p) + es * NPAR * 4;
         float2 kf[4];
-        float kv[4];
 #pragma unroll
         for (int mu = 0; mu < 4; ++mu) {
           DflSum k;
@@ -704,20 +655,19 @@ __device__ __forceinline__ void hs_tables(unsigned char* smem, const PhysParams&
             k.add(c * v.x, c * v.y);
           }
           kf[mu] = make_float2(k.s, k.err);
-          kv[mu] = k.value();
+          K[(u * KEV + 4 * j + mu) * EW + lane] = k.value();
         }
-        *reinterpret_cast<float4*>(K + e * KEV + 4 * j) = make_float4(kv[0], kv[1], kv[2], kv[3]);
         const float4* mc = reinterpret_cast<const float4*>(smem + L::o_mconst);
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int pj = u == 0 ? d.z : d.w;
+        for (int i = 0; i < 2; ++i) {
+          const int pj = i == 0 ? d.z : d.w;
           if (pj < 0) continue;
           const int kind = prop_tab[pj].y;
           const float4 c = mc[kind == 3 ? 1 : 0];  // {m^2 hi, m^2 lo, m w, 0} of the top / the Z
-          pr[e * P::NPROP + pj] = propagator_dfl(kf, kind, dfl{c.x, c.y}, c.z);
+          put(pj, propagator_dfl(kf, kind, dfl{c.x, c.y}, c.z));
         }
       } else {
-        const double* q = reinterpret_cast<const double*>(smem + L::o_p) + e * NPAR * 4;
+        const double* q = reinterpret_cast<const double*>(smem + L::o_p) + es * NPAR * 4;
         double k[4];
 #pragma unroll
         for (int mu = 0; mu < 4; ++mu) {
@@ -728,56 +678,66 @@ __device__ __forceinline__ void hs_tables(unsigned char* smem, const PhysParams&
             s += c * q[l * 4 + mu];
           }
           k[mu] = s;
-          K[e * KEV + j * 4 + mu] = R(s);
+          K[(u * KEV + 4 * j + mu) * EW + lane] = R(s);
         }
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int pj = u == 0 ? d.z : d.w;
+        for (int i = 0; i < 2; ++i) {
+          const int pj = i == 0 ? d.z : d.w;
           if (pj < 0) continue;
-          pr[e * P::NPROP + pj] = propagator_hs<R>(k, prop_tab[pj].y, pp);
+          put(pj, propagator_hs<R>(k, prop_tab[pj].y, pp));
         }
       }
     } else {
-      const int t2 = t - nev * NM, el = t2 / NE, e = grp.ev0 + el, j = t2 - el * NE;
-      const HsSlots<P, R, P::HS_NSLOT> cur{curs + e * CUR_EV};
+      const HsSlots<P, V, P::HS_NSLOT> cur{curs + u * CUR_EV};
       if constexpr (DF) {
         const HsItem it = P::hs_items()[2 * j];
         dfl k[4];
 #pragma unroll
         for (int mu = 0; mu < 4; ++mu) {
-          const float2 v = reinterpret_cast<const float2*>(smem + L::o_p)[(e * NPAR + it.a) * 4 + mu];
+          const float2 v = reinterpret_cast<const float2*>(smem + L::o_p)[(es * NPAR + it.a) * 4 + mu];
           k[mu] = dfl{v.x, v.y};
         }
         W4<R> o[2];
         if (it.type == 2) ext_vector_dfl(k, it.c, o);
         else ext_fermion_dfl(k, it.flag ? cp.mt : 0.0f, it.c, it.type == 1, o);
-        cur.set(it.out, o[0]);
-        cur.set(P::hs_items()[2 * j + 1].out, o[1]);
+        cur.set_lane(it.out, lane, o[0]);
+        cur.set_lane(P::hs_items()[2 * j + 1].out, lane, o[1]);
       } else {
         const HsItem it = P::hs_items()[j];
-        const double* k = reinterpret_cast<const double*>(smem + L::o_p) + (e * NPAR + it.a) * 4;
+        const double* k = reinterpret_cast<const double*>(smem + L::o_p) + (es * NPAR + it.a) * 4;
         W4<R> o;
         if (it.type == 0) o = ixxxxx<R>(k, it.flag ? cp.mt : R(0), it.b, it.c);
         else if (it.type == 1) o = oxxxxx<R>(k, it.flag ? cp.mt : R(0), it.b, it.c);
         else o = vxxxxx<R>(k, it.b, it.c);
-        cur.set(it.out, o);
+        cur.set_lane(it.out, lane, o);
       }
     }
   }
-  grp.sync();
+  __syncthreads();
 }
 
 // a shared-memory word read where it is written here (not kept in a register)
 __device__ __forceinline__ int lds_again(const int* p) { return *reinterpret_cast<const volatile int*>(p); }
 
+// Events per group (whole units of ew): the most a CTA takes at once, or fewer
+// where one round spreads the batch over all the grid's CTAs (a small batch has
+// one unit per CTA instead of a few full CTAs).  With more than one round full
+// groups are kept: their warps are full.
+__device__ __forceinline__ int hs_events_per_group(int64_t n, int most, int ew) {
+  const int g = (int)gridDim.x;
+  if (n >= (int64_t)g * most) return most;
+  return min(most, ((int)n + g * ew - 1) / (g * ew) * ew);
+}
+
 // Item of work index t when the lanes take items item-major: consecutive
-// lanes take one item for each of the group's nev events, so that a warp holds
-// 32 / nev items (of one vertex type wherever the generator's per-event type
+// lanes take one item for each of the group's units, so that a warp holds
+// 32 / units items (of one vertex type wherever the generator's per-event type
 // segments are multiples of that) and reads each descriptor once for all
-// its events.
+// its units.
 template <class L>
-__device__ __forceinline__ int hs_item_of(int t, int nev) {
-  return nev == L::EVCAP ? t / L::EVCAP : t / nev;
+__device__ __forceinline__ int hs_item_of(int t, int nu) {
+  // t / nu: t nu < 2^32, so the high word of t times ceil(2^32 / nu) is exact
+  return nu == L::EVCAP ? t / L::EVCAP : (nu == 1 ? t : (int)__umulhi((unsigned)t, 0xffffffffu / (unsigned)nu + 1u));
 }
 
 // Items of the ordered program: a two-leg current ...
@@ -788,7 +748,7 @@ __device__ __forceinline__ void ord_item(const HsItem& it, const HsSlots<P, R, P
   switch (it.type) {
     case 15: o = FFV1_2<R>(cur[it.in[0]], cur[it.in[1]], R(1), K + 4 * it.k0, cp.mt, pr[it.prop]); break;
     case 16: o = FFV1_1<R>(cur[it.in[0]], cur[it.in[1]], R(1), K + 4 * it.k0, cp.mt, pr[it.prop]); break;
-    case 17: o = w4_rscale(ord_pair(cur[it.in[0]], cur[it.in[1]]), -pr[it.prop].im); break;
+    case 17: o = w4_rscale(vector_pair(cur[it.in[0]], cur[it.in[1]]), -pr[it.prop].im); break;
     default: o = w4_rscale(ord_v3(cur[it.in[0]], cur[it.in[1]], K + 4 * it.k0, K + 4 * it.k1), pr[it.prop].im);
   }
   cur.set(it.out, o);
@@ -821,9 +781,9 @@ __device__ __forceinline__ void ord_xitem(const HsItem& it, const HsSlots<P, R, 
     xb.set(it.out + HS_WORD, o2);
   } else if (it.type == 22) {
     const W4<R> g = ord_v3(cur[it.in[2]], cur[it.in3()], K + 4 * it.k0, K + 4 * it.k1);
-    o = w4_lower(w4_sub(ord_pair(cur[it.in[0]], cur[it.in[1]]), g));
+    o = w4_lower(w4_sub(vector_pair(cur[it.in[0]], cur[it.in[1]]), g));
   } else if (it.type == 23) {
-    o = w4_lower(ord_pair(cur[it.in[0]], cur[it.in[1]]));
+    o = w4_lower(vector_pair(cur[it.in[0]], cur[it.in[1]]));
   } else {
     o = ord_v3(cur[it.in[0]], cur[it.in[1]], K + 4 * it.k0, K + 4 * it.k1);  // times -1, lower index
     o.w[0] = -o.w[0];
@@ -831,15 +791,12 @@ __device__ __forceinline__ void ord_xitem(const HsItem& it, const HsSlots<P, R, 
   xb.set(it.out, o);
 }
 
-// one current variant
+// one current variant (external wavefunctions: hs_tables)
 template <class P, class R>
 __device__ __forceinline__ void hs_item(const HsItem& it, const Slots<R, P::HS_NSLOT>& cur, const R* K,
                                         const cx<R>* pr, const Couplings<R>& cp) {
   W4<R> o;
   switch (it.type) {
-    case 0: o = ixxxxx<R>(K + 4 * it.k0, it.flag ? cp.mt : R(0), it.b, it.c); break;
-    case 1: o = oxxxxx<R>(K + 4 * it.k0, it.flag ? cp.mt : R(0), it.b, it.c); break;
-    case 2: o = vxxxxx<R>(K + 4 * it.k0, it.b, it.c); break;
     case 3: o = FFV1_2<R>(cur[it.in[0]], cur[it.in[1]], cp.gs, K + 4 * it.k0, cp.mt, pr[it.prop]); break;
     case 4: o = FFV1_1<R>(cur[it.in[0]], cur[it.in[1]], cp.gs, K + 4 * it.k0, cp.mt, pr[it.prop]); break;
     case 5: o = FFV1P0_3<R>(cur[it.in[0]], cur[it.in[1]], it.a ? cp.ee : cp.gs, pr[it.prop]); break;
@@ -906,10 +863,10 @@ __device__ __forceinline__ int warp_inverse_cdf(int n, double u, int lane, F get
 }
 
 // Per event: a good helicity with probability |M_h|^2 / sum (weights sm2 of
-// the event's threads, helicity order) and a colour flow s with probability
+// the event, helicity order) and a colour flow s with probability
 // w_s / sum, w_s = sum over the good helicities of |J_s|^2; one warp per event.
-// The |J_s|^2 of every thread are staged in the dead union region, thread-major
-// with an odd row stride (lane s of the event's warp sums row entries s over
+// The |J_s|^2 of every (event, helicity) are staged in the dead union region, one
+// row each with an odd row stride (lane s of the event's warp sums row entries s over
 // the event's helicities, in helicity order, in the working precision; the
 // running sums that decide are FP64).
 template <class P, class R>
@@ -919,16 +876,16 @@ struct HsChoice {
 
 template <class P, class R, class L>
 __device__ __forceinline__ void hs_choices(const unsigned char* smem, const SigArgs& a, int64_t e0, int nev, int ng,
-                                           const int* good, const double* sm2) {
+                                           const int* good, const R* sm2) {
   constexpr int NT = L::NT, NC = P::NCOLOR, NCP = HsChoice<P, R>::NCP;
   static_assert(NC <= 32, "one lane per colour flow");
-  static_assert(sizeof(R) * NCP * NT <= L::u_bytes, "colour weights overflow their scratch");
+  static_assert(sizeof(R) * NCP * NT * L::EW <= L::u_bytes, "colour weights overflow their scratch");
   const int tid = threadIdx.x, lane = tid & 31;
   const R* wj = reinterpret_cast<const R*>(smem + L::o_U);
   for (int e = tid >> 5; e < nev; e += NT / 32) {
     if (a.hel_out) {
       const int k = warp_inverse_cdf<(P::NHEL + 31) / 32>(ng, a.hel_rnd[e0 + e], lane,
-                                                          [&](int i) { return sm2[e * ng + i]; });
+                                                          [&](int i) { return (double)sm2[e * ng + i]; });
       if (lane == 0) a.hel_out[e0 + e] = k < 0 ? -1 : good[k];
     }
     if (a.col_out) {
@@ -942,9 +899,9 @@ __device__ __forceinline__ void hs_choices(const unsigned char* smem, const SigA
   }
 }
 
-// Record of one event's current variants and momentum table in global memory
+// Record of one unit's current variants and momentum tables in global memory
 // (the kernel-split variant: the first kernel writes them, the second reads
-// them back into shared memory): HS_NSLOT slots of 16-byte planes, then the
+// them back into shared memory; R the lane type): HS_NSLOT slots of 16-byte planes, then the
 // momentum table K[NMOM][4] in the working precision and, where operands of the
 // contractions have propagators (ordered program), the propagator factors.
 template <class P, class R>
@@ -1002,30 +959,30 @@ __device__ __forceinline__ double hs_norm(const PhysParams& pp) {
 
 // The helicity-shared program for the events [first, last) of the batch.
 // SRC == kSrcRecords: phases 1-2 (momenta, tables, current variants) are
-// replaced by a copy of the events' records from `rec` (one record per event,
-// event first - first at rec[0]).
+// replaced by a copy of the records from `rec` (one record per unit, the unit of
+// event `first` at rec[0]).
 template <class P, class R, int CS, int SRC>
 __device__ __forceinline__ void hs_sigmakin_body(const SigArgs& a, const Couplings<R>& cp, int64_t first, int64_t last,
                                                  const uint4* __restrict__ rec, const RamboArgs* ra = nullptr) {
-  using C = HsCfg<P, R>;
   using L = HsLayout<P, R, CS>;
+  using V = typename L::V;
   constexpr bool FROM_RECORDS = SRC == kSrcRecords;
   static_assert(!(FROM_RECORDS && L::TC), "the kernel-split variant sums colours on CUDA cores");
-  constexpr int NT = C::NT, NC = P::NCOLOR;
+  constexpr int NT = L::NT, NC = P::NCOLOR, EW = L::EW;
   extern __shared__ __align__(1024) unsigned char smem[];
   int* good = reinterpret_cast<int*>(smem + L::o_good);
   int* misc = reinterpret_cast<int*>(smem + L::o_misc);
-  double* sm2 = reinterpret_cast<double*>(smem + L::o_m2);
+  R* sm2 = reinterpret_cast<R*>(smem + L::o_m2);
   uint8_t* vtab = reinterpret_cast<uint8_t*>(smem + L::o_vt);
-  // per event: HS_NSLOT current slots, HS_XCAP amputated slots (16-byte planes)
+  // per unit: HS_NSLOT current slots, HS_XCAP further operands (16-byte planes)
   uint4* curs = reinterpret_cast<uint4*>(smem + L::o_cur);
   uint4* xbufs = reinterpret_cast<uint4*>(smem + L::o_x);
   constexpr int CUR_EV = L::CUR_EV, X_EV = L::X_EV;
   const int tid = threadIdx.x, lane = tid & 31;
   hs_setup_words<P, R, L>(smem, a.pp);
-  // vt[S][ihel]: variant index of leg set S for helicity ihel (generated table)
-  static_assert(((1 << P::NPAR) * P::NHEL) % 16 == 0, "variant table copied in 16-byte words");
-  for (int i = tid; i < (1 << P::NPAR) * P::NHEL / 16; i += NT)
+  // vt[row][ihel]: variant index of the row's leg set for helicity ihel (generated table)
+  static_assert((P::HS_NVT * P::NHEL) % 16 == 0, "variant table copied in 16-byte words");
+  for (int i = tid; i < P::HS_NVT * P::NHEL / 16; i += NT)
     reinterpret_cast<uint4*>(vtab)[i] = reinterpret_cast<const uint4*>(P::hs_variants())[i];
   // good helicities: every warp ballots the mask itself (32 helicities per
   // word), so the events and their momenta are known before any barrier;
@@ -1038,7 +995,7 @@ __device__ __forceinline__ void hs_sigmakin_body(const SigArgs& a, const Couplin
     if (w & bit) good[__popc(w & (bit - 1u)) + (tid >= 32 ? __popc(w0) : 0)] = tid;
   }
   const int ng = __popc(w0) + __popc(w1);
-  const int ev = ng > 0 ? min(L::EVCAP, NT / ng) : C::EVMIN;
+  const int ev = hs_events_per_group(last - first, EW * (ng > 0 ? min(L::EVCAP, NT / ng) : L::H::EVMIN), EW);
   // groups of ev events, g = blockIdx.x, blockIdx.x + gridDim.x, ...: one
   // group per CTA for a grid of all groups, several for a persistent grid
   const int ngrp = (int)((last - first + ev - 1) / ev);
@@ -1072,8 +1029,9 @@ __device__ __forceinline__ void hs_sigmakin_body(const SigArgs& a, const Couplin
     tc::fence_async_shared();
     tc::fence_before_sync();
   }
-  const R* Kall = reinterpret_cast<const R*>(smem + L::o_K);
-  const cx<R>* prall = reinterpret_cast<const cx<R>*>(smem + L::o_pr);
+  const V* Kall = reinterpret_cast<const V*>(smem + L::o_K);
+  const cx<V>* prall = reinterpret_cast<const cx<V>*>(smem + L::o_pr);
+  const Couplings<V> cv = lane_couplings<V>(cp);
   const HsItem* items = P::hs_items();
   if constexpr (SRC == kSrcMomenta) {
     // the first group's momenta; later groups' arrive by prefetch
@@ -1099,24 +1057,24 @@ __device__ __forceinline__ void hs_sigmakin_body(const SigArgs& a, const Couplin
     // e0 and nev are formed again after the contractions (fewer live registers)
     const int ev = lds_again(misc + 7);
     const int nev = (int)min((int64_t)ev, last - (first + (int64_t)g * ev));
-    const HsGroup grp = hs_group<NT>(L::TC || !MG_HS_EVENT_SYNC, ng, ev, nev);
+    const int nu = (nev + EW - 1) / EW;
     if constexpr (FROM_RECORDS) {
-      // 1-2. the events' current variants and momentum tables from their records
-      using RC = HsRecord<P, R>;
-      const uint4* in = rec + (int64_t)g * ev * RC::WORDS;
+      // 1-2. the units' current variants and momentum tables from their records
+      using RC = HsRecord<P, V>;
+      const uint4* in = rec + (int64_t)g * (ev / EW) * RC::WORDS;
       uint4* ks = reinterpret_cast<uint4*>(smem + L::o_K);
-      for (int t = tid; t < nev * RC::WORDS; t += NT) {
-        const int e = t / RC::WORDS, w = t - e * RC::WORDS;
+      for (int t = tid; t < nu * RC::WORDS; t += NT) {
+        const int u = t / RC::WORDS, w = t - u * RC::WORDS;
         const uint4 v = __ldcs(in + t);  // read once: streaming
-        if (w < RC::CUR) curs[e * CUR_EV + w] = v;
-        else if (w < RC::CUR + RC::KW) ks[e * (L::KEV * (int)sizeof(R) / 16) + (w - RC::CUR)] = v;
+        if (w < RC::CUR) curs[u * CUR_EV + w] = v;
+        else if (w < RC::CUR + RC::KW) ks[u * (L::KEV * (int)sizeof(V) / 16) + (w - RC::CUR)] = v;
         else {
-          const cx<R>* f = reinterpret_cast<const cx<R>*>(&v);
-          constexpr int PER = (int)(16 / sizeof(cx<R>));
+          const cx<V>* f = reinterpret_cast<const cx<V>*>(&v);
+          constexpr int PER = (int)(16 / sizeof(cx<V>));
 #pragma unroll
           for (int k = 0; k < PER; ++k) {
             const int j = (w - RC::CUR - RC::KW) * PER + k;
-            if (j < P::NPROP) reinterpret_cast<cx<R>*>(smem + L::o_pr)[e * P::NPROP + j] = f[k];
+            if (j < P::NPROP) reinterpret_cast<cx<V>*>(smem + L::o_pr)[u * P::NPROP + j] = f[k];
           }
         }
       }
@@ -1138,79 +1096,83 @@ __device__ __forceinline__ void hs_sigmakin_body(const SigArgs& a, const Couplin
         if (nevn > 0) hs_prefetch_momenta<P, L>(smem, a.mom, a.nevt, e0n, nevn);
       }
       // 1. per-event tables (the momenta are in p)
-      hs_tables<P, R, L, CUR_EV, L::KEV>(smem, a.pp, grp, curs, cp);
+      hs_tables<P, R, L, V, CUR_EV, L::KEV>(smem, a.pp, nev, curs, cp);
       // 2. current variants, level by level (level 0, the external wavefunctions,
       //    came with phase 1); consecutive threads take one item for each event (hs_item_of)
 #pragma unroll
       for (int l = 1; l < P::HS_NLEVEL; ++l) {
-        const int i0 = P::hs_level(l), ni = P::hs_level(l + 1) - i0, n = ni * grp.nev;
-        for (int t = grp.j; t < n; t += grp.tpg) {
-          const int ii = hs_item_of<L>(t, grp.nev), e = grp.ev0 + t - ii * grp.nev;
+        const int i0 = P::hs_level(l), n = (P::hs_level(l + 1) - i0) * nu;
+        for (int t = tid; t < n; t += NT) {
+          const int ii = hs_item_of<L>(t, nu), u = t - ii * nu;
           const HsItem it = items[i0 + ii];
-          const HsSlots<P, R, P::HS_NSLOT> cur{curs + e * CUR_EV};
-          if constexpr (P::HS_ORDERED) ord_item<P, R>(it, cur, Kall + e * L::KEV, prall + e * P::NPROP, cp);
-          else hs_item<P, R>(it, cur, Kall + e * L::KEV, prall + e * P::NPROP, cp);
+          const HsSlots<P, V, P::HS_NSLOT> cur{curs + u * CUR_EV};
+          if constexpr (P::HS_ORDERED) ord_item<P, V>(it, cur, Kall + u * L::KEV, prall + u * P::NPROP, cv);
+          else hs_item<P, V>(it, cur, Kall + u * L::KEV, prall + u * P::NPROP, cv);
         }
         if (l == P::HS_NLEVEL - 1) {
           cp_async_wait_all();
           __syncthreads();
           if (nevn > 0) hs_convert_momenta<P, R, L>(smem, nevn);
         } else {
-          grp.sync();
+          __syncthreads();
         }
       }
     }
     // 3. the operands of the contractions (amputated currents), then every
-    //    thread contracts for its (event, helicity), J in registers
+    //    thread contracts for its (unit, helicity), J in registers
+    static_assert(P::HS_NXCHUNK == 1, "the operands of every contraction at once");
     {
-      const int i0 = P::hs_xitem(0), ni = P::hs_xitem(1) - i0, n = ni * grp.nev;
-      for (int t = grp.j; t < n; t += grp.tpg) {
-        const int ii = hs_item_of<L>(t, grp.nev), ex = grp.ev0 + t - ii * grp.nev;
+      const int i0 = P::hs_xitem(0), n = (P::hs_xitem(1) - i0) * nu;
+      for (int t = tid; t < n; t += NT) {
+        const int ii = hs_item_of<L>(t, nu), ui = t - ii * nu;
         const HsItem it = items[i0 + ii];
-        const HsSlots<P, R, P::HS_NSLOT> cur{curs + ex * CUR_EV};
-        const HsSlots<P, R, P::HS_XCAP> xs{xbufs + ex * X_EV};
-        if constexpr (P::HS_ORDERED) ord_xitem<P, R>(it, cur, xs, Kall + ex * L::KEV, prall + ex * P::NPROP, cp);
-        else hs_xitem<P, R>(it, cur, xs, Kall + ex * L::KEV, cp);
+        const HsSlots<P, V, P::HS_NSLOT> cur{curs + ui * CUR_EV};
+        const HsSlots<P, V, P::HS_XCAP> xs{xbufs + ui * X_EV};
+        if constexpr (P::HS_ORDERED) ord_xitem<P, V>(it, cur, xs, Kall + ui * L::KEV, prall + ui * P::NPROP, cv);
+        else hs_xitem<P, V>(it, cur, xs, Kall + ui * L::KEV, cv);
       }
     }
-    grp.sync();
+    __syncthreads();
     const int ng = lds_again(misc + 6);
-    const bool active = tid < nev * ng;
-    const int e = active ? tid / ng : 0;
-    const int ih = good[active ? tid - e * ng : 0];
-    cx<R> J[NC];
+    const bool active = tid < nu * ng;
+    const int u = active ? tid / ng : 0, kh = active ? tid - u * ng : 0;  // unit, good helicity
+    cx<V> J[NC];
 #pragma unroll
-    for (int s = 0; s < NC; ++s) J[s] = cx<R>(R(0), R(0));
-    P::template hs_contract<R>(0, HsSlots<P, R, P::HS_NSLOT>{curs + e * CUR_EV},
-                               HsSlots<P, R, P::HS_XCAP>{xbufs + e * X_EV}, vtab + ih, J);
-    // 4. colour sum and helicity sum
-    double m2;
+    for (int s = 0; s < NC; ++s) J[s] = cx<V>(V(0), V(0));
+    P::template hs_contract<V>(0, HsSlots<P, V, P::HS_NSLOT>{curs + u * CUR_EV},
+                               HsSlots<P, V, P::HS_XCAP>{xbufs + u * X_EV}, vtab + good[kh], J);
+    // 4. colour sum and helicity sum; |M_h|^2 of (event, good helicity) k at
+    //    sm2[event * ng + k]
+    V m2;
     if constexpr (L::TC) {
       __syncthreads();  // the A tiles overwrite the current variants
-      m2 = (double)colour_sum_tc_regs<P, L>(smem, J, tmem, mbar);
+      m2 = colour_sum_tc_regs<P, L>(smem, J, tmem, mbar);
     } else {
-      m2 = (double)colour_sum<P, R>(J);
+      m2 = colour_sum<P, V>(J);
     }
-    sm2[tid] = active ? m2 : 0.0;
+    if (active) {
+#pragma unroll
+      for (int i = 0; i < EW; ++i) sm2[(u * EW + i) * ng + kh] = lane_value(m2, i);
+    }
     if constexpr (L::TC) tc::fence_before_sync();
-    grp.sync();
+    __syncthreads();
     const int64_t e0 = first + (int64_t)g * lds_again(misc + 7);
     // fixed-order FP64 helicity sum per event: eight lanes per event each add
     // every eighth helicity in order, then a butterfly over the eight lanes
     // (addition commutes, so every lane ends with the same bits); sm2 is next
     // written at the end of the next group, after several barriers
-    for (int b = 0; b < grp.nev * 8; b += grp.tpg) {
-      const int t = b + grp.j, eh = grp.ev0 + (t >> 3), q = t & 7;
+    for (int b = 0; b < nev * 8; b += NT) {
+      const int t = b + tid, eh = t >> 3, q = t & 7;
       double sum = 0.0;
-      if (t < grp.nev * 8) {
+      if (t < nev * 8) {
 #pragma unroll
         for (int i = 0; i < (P::NHEL + 7) / 8; ++i)
-          if (q + 8 * i < ng) sum += sm2[eh * ng + q + 8 * i];
+          if (q + 8 * i < ng) sum += (double)sm2[eh * ng + q + 8 * i];
       }
       sum += __shfl_xor_sync(0xffffffffu, sum, 1);
       sum += __shfl_xor_sync(0xffffffffu, sum, 2);
       sum += __shfl_xor_sync(0xffffffffu, sum, 4);
-      if (t < grp.nev * 8 && q == 0) a.me[e0 + eh] = sum * hs_norm<P>(a.pp);
+      if (t < nev * 8 && q == 0) a.me[e0 + eh] = sum * hs_norm<P>(a.pp);
     }
     // 5. helicity and colour-flow choices (batched entry point), once every
     //    group of the CTA is done with the union region; the closing barrier
@@ -1218,10 +1180,17 @@ __device__ __forceinline__ void hs_sigmakin_body(const SigArgs& a, const Couplin
     if (a.hel_out || a.col_out) {
       __syncthreads();
       if (a.col_out) {
-        if constexpr (!L::TC && P::COLOUR_BLOCKS) colour_hadamard<P, R>(J, R(0.25));  // back to the chains
-        R* wj = reinterpret_cast<R*>(smem + L::o_U) + tid * HsChoice<P, R>::NCP;  // the union is dead here
+        if constexpr (!L::TC && P::COLOUR_BLOCKS) colour_hadamard<P, V, true>(J);  // back to the chains
+        R* wj = reinterpret_cast<R*>(smem + L::o_U);  // the union is dead here; rows as sm2's
+        if (active) {
 #pragma unroll
-        for (int s = 0; s < NC; ++s) wj[s] = active ? J[s].re * J[s].re + J[s].im * J[s].im : R(0);
+          for (int i = 0; i < EW; ++i)
+#pragma unroll
+            for (int s = 0; s < NC; ++s) {
+              const R re = lane_value(J[s].re, i), im = lane_value(J[s].im, i);
+              wj[((u * EW + i) * ng + kh) * HsChoice<P, R>::NCP + s] = re * re + im * im;
+            }
+        }
         __syncthreads();
       }
       hs_choices<P, R, L>(smem, a, e0, nev, ng, good, sm2);
@@ -1237,13 +1206,13 @@ __device__ __forceinline__ void hs_sigmakin_body(const SigArgs& a, const Couplin
 }
 
 template <class P, class R, int CS>
-__global__ void __launch_bounds__(HsCfg<P, R>::NT, HsCfg<P, R>::CTAS) sigmakin_hs_kernel(SigArgs a, Couplings<R> cp) {
+__global__ void __launch_bounds__(HsCfg<P, R, CS>::NT, HsCfg<P, R, CS>::CTAS) sigmakin_hs_kernel(SigArgs a, Couplings<R> cp) {
   hs_sigmakin_body<P, R, CS, kSrcMomenta>(a, cp, 0, a.nevt, nullptr);
 }
 
 // RAMBO and SIGMAKIN in one kernel: no momentum buffer in HBM
 template <class P, class R, int CS>
-__global__ void __launch_bounds__(HsCfg<P, R>::NT, HsCfg<P, R>::CTAS)
+__global__ void __launch_bounds__(HsCfg<P, R, CS>::NT, HsCfg<P, R, CS>::CTAS)
     sigmakin_hs_rambo_kernel(SigArgs a, Couplings<R> cp, RamboArgs ra) {
   hs_sigmakin_body<P, R, CS, kSrcRambo>(a, cp, 0, a.nevt, nullptr, &ra);
 }

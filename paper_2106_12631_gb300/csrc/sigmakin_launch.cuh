@@ -19,7 +19,8 @@ cudaError_t launch_sigmakin_variant(const SigArgs& a, const Couplings<R>& cp, in
 
 // The helicity-shared kernel runs persistent: as many CTAs as are resident at
 // once (SMs x CTAs per SM, cached per device), each looping over groups of
-// events (the CTA's group count follows from the mask on the device).  CTAs
+// events (the CTA's group count follows from the mask and the grid on the device;
+// a batch that does not fill the CTAs is spread over all of them).  CTAs
 // per SM: the larger of the occupancy query and the count the kernel's shared
 // memory budget and launch bounds are built for (the query has returned 1 for
 // the tcgen05 variant, whose two CTAs per SM fit); should fewer fit, the
@@ -29,13 +30,14 @@ template <class P, class R, int CS, bool FUSED = false>
 cudaError_t launch_sigmakin_hs_variant(const SigArgs& a, const Couplings<R>& cp, int64_t grid, cudaStream_t s,
                                        const RamboArgs* ra = nullptr) {
   using L = HsLayout<P, R, CS>;
-  constexpr int NT = HsCfg<P, R>::NT;
+  using H = typename L::H;
+  constexpr int NT = L::NT;
   constexpr int kMaxDevices = 64;
   static int resident[kMaxDevices];  // CTAs resident on the whole device; 0 until known
   const void* k = FUSED ? (const void*)sigmakin_hs_rambo_kernel<P, R, CS> : (const void*)sigmakin_hs_kernel<P, R, CS>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::bytes);
   if (e != cudaSuccess) return e;
-  grid = (a.nevt + HsCfg<P, R>::EVMIN - 1) / HsCfg<P, R>::EVMIN;
+  grid = (a.nevt + H::EW - 1) / H::EW;  // one unit per CTA at least
   int dev = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   int cap = dev < kMaxDevices ? resident[dev] : 0;
@@ -43,7 +45,7 @@ cudaError_t launch_sigmakin_hs_variant(const SigArgs& a, const Couplings<R>& cp,
     int nsm = 0, per = 0;
     if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, NT, L::bytes)) != cudaSuccess) return e;
-    cap = nsm * (per > HsCfg<P, R>::CTAS ? per : HsCfg<P, R>::CTAS);
+    cap = nsm * (per > H::CTAS ? per : H::CTAS);
     if (dev < kMaxDevices) resident[dev] = cap;
   }
   if (grid > cap) grid = cap;

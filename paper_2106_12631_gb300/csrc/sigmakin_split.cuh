@@ -21,15 +21,16 @@ namespace mg {
 // the currents kernel's own smaller CTA: 4 events, 128 threads, three CTAs per SM
 template <class P, class R>
 struct HsSplitA {
-  static constexpr int NT = 128, EV = 4, CTAS = 3;
+  using V = HsLane<P, R, CS_SIMT>;
+  static constexpr int NT = 128, EV = 4, CTAS = 3, EW = LaneOf<V>::EW, EU = EV / EW;  // EU units
   static constexpr size_t o_proptab = 0;
   static constexpr size_t o_md = align_up(o_proptab + 8 * P::NPROP, 16);
   static constexpr size_t o_mconst = align_up(o_md + 16 * P::NMOM, 16);
   static constexpr size_t o_p = align_up(o_mconst + 32, 16);
   static constexpr size_t o_K = align_up(o_p + 8 * EV * P::NPAR * 4, 16);
-  static constexpr size_t o_pr = align_up(o_K + sizeof(R) * EV * P::NMOM * 4, 16);
-  static constexpr size_t o_cur = align_up(o_pr + 2 * sizeof(R) * EV * P::NPROP, 16);
-  static constexpr size_t bytes = o_cur + sizeof(W4<R>) * EV * P::HS_NSLOT;
+  static constexpr size_t o_pr = align_up(o_K + sizeof(V) * EU * P::NMOM * 4, 16);
+  static constexpr size_t o_cur = align_up(o_pr + 2 * sizeof(V) * EU * P::NPROP, 16);
+  static constexpr size_t bytes = o_cur + sizeof(W4<V>) * EU * P::HS_NSLOT;
   static_assert(bytes <= 232448, "shared memory per CTA above the 227 KB limit");
 };
 
@@ -37,7 +38,8 @@ template <class P, class R>
 __global__ void __launch_bounds__(HsSplitA<P, R>::NT, HsSplitA<P, R>::CTAS)
     sigmakin_hs_currents_kernel(SigArgs a, Couplings<R> cp, int64_t first, int64_t last, uint4* __restrict__ rec) {
   using L = HsSplitA<P, R>;
-  using RC = HsRecord<P, R>;
+  using V = typename L::V;
+  using RC = HsRecord<P, V>;
   constexpr int NT = L::NT;
   extern __shared__ __align__(1024) unsigned char smem[];
   const int tid = threadIdx.x;
@@ -48,36 +50,37 @@ __global__ void __launch_bounds__(HsSplitA<P, R>::NT, HsSplitA<P, R>::CTAS)
   hs_setup_words<P, R, L>(smem, a.pp);
   hs_load_momenta<P, R, L>(smem, a.mom, a.nevt, e0, nev);
   __syncthreads();
-  const HsGroup cta{0, NT, tid, 0, nev, 0};
-  hs_tables<P, R, L>(smem, a.pp, cta, curs, cp);
-  const R* Kall = reinterpret_cast<const R*>(smem + L::o_K);
-  const cx<R>* prall = reinterpret_cast<const cx<R>*>(smem + L::o_pr);
+  const int nu = (nev + L::EW - 1) / L::EW;
+  hs_tables<P, R, L, V>(smem, a.pp, nev, curs, cp);
+  const V* Kall = reinterpret_cast<const V*>(smem + L::o_K);
+  const cx<V>* prall = reinterpret_cast<const cx<V>*>(smem + L::o_pr);
+  const Couplings<V> cv = lane_couplings<V>(cp);
   const HsItem* items = P::hs_items();
 #pragma unroll
   for (int l = 1; l < P::HS_NLEVEL; ++l) {
-    const int i0 = P::hs_level(l), ni = P::hs_level(l + 1) - i0, n = ni * nev;
+    const int i0 = P::hs_level(l), ni = P::hs_level(l + 1) - i0, n = ni * nu;
     for (int t = tid; t < n; t += NT) {
-      const int e = t / ni;
-      const HsItem it = items[i0 + t - e * ni];
-      const HsSlots<P, R, P::HS_NSLOT> cur{curs + e * RC::CUR};
-      if constexpr (P::HS_ORDERED) ord_item<P, R>(it, cur, Kall + e * P::NMOM * 4, prall + e * P::NPROP, cp);
-      else hs_item<P, R>(it, cur, Kall + e * P::NMOM * 4, prall + e * P::NPROP, cp);
+      const int u = t / ni;
+      const HsItem it = items[i0 + t - u * ni];
+      const HsSlots<P, V, P::HS_NSLOT> cur{curs + u * RC::CUR};
+      if constexpr (P::HS_ORDERED) ord_item<P, V>(it, cur, Kall + u * P::NMOM * 4, prall + u * P::NPROP, cv);
+      else hs_item<P, V>(it, cur, Kall + u * P::NMOM * 4, prall + u * P::NPROP, cv);
     }
     __syncthreads();
   }
   const uint4* ks = reinterpret_cast<const uint4*>(smem + L::o_K);
-  uint4* out = rec + (e0 - first) * RC::WORDS;
-  for (int t = tid; t < nev * RC::WORDS; t += NT) {
-    const int e = t / RC::WORDS, w = t - e * RC::WORDS;
+  uint4* out = rec + (e0 - first) / L::EW * RC::WORDS;
+  for (int t = tid; t < nu * RC::WORDS; t += NT) {
+    const int u = t / RC::WORDS, w = t - u * RC::WORDS;
     if (w < RC::CUR + RC::KW) {
-      out[t] = w < RC::CUR ? curs[e * RC::CUR + w] : ks[e * RC::KW + (w - RC::CUR)];
+      out[t] = w < RC::CUR ? curs[u * RC::CUR + w] : ks[u * RC::KW + (w - RC::CUR)];
     } else {
-      constexpr int PER = (int)(16 / sizeof(cx<R>));
-      alignas(16) cx<R> f[PER];
+      constexpr int PER = (int)(16 / sizeof(cx<V>));
+      alignas(16) cx<V> f[PER];
 #pragma unroll
       for (int k = 0; k < PER; ++k) {
         const int j = (w - RC::CUR - RC::KW) * PER + k;
-        f[k] = prall[e * P::NPROP + min(j, P::NPROP - 1)];
+        f[k] = prall[u * P::NPROP + min(j, P::NPROP - 1)];
       }
       out[t] = *reinterpret_cast<const uint4*>(f);
     }
@@ -109,7 +112,7 @@ struct SplitLaunch {
   static cudaError_t amplitudes(const SigArgs& a, const Couplings<R>& cp, int64_t first, int64_t last,
                                 const uint4* rec, cudaStream_t s) {
     using C = HsCfg<P, R>;
-    const int64_t grid = (last - first + C::EVMIN - 1) / C::EVMIN;
+    const int64_t grid = (last - first + C::EVMIN * C::EW - 1) / (C::EVMIN * C::EW);
     sigmakin_hs_amplitudes_kernel<P, R>
         <<<(unsigned)grid, C::NT, HsLayout<P, R, CS_SIMT>::bytes, s>>>(a, cp, first, last, rec);
     return cudaGetLastError();
@@ -120,21 +123,28 @@ struct SplitLaunch {
 
 namespace mg {
 
-// One batch through the split kernels: chunk = workspace / (2 records), a
-// multiple of the currents kernel's events per CTA; the graph key holds every
+// bytes per event (a record holds the events of one lane)
+template <class P, class R>
+constexpr int64_t split_record_bytes() {
+  using A = HsSplitA<P, R>;
+  static_assert(HsRecord<P, typename A::V>::WORDS * 16 % A::EW == 0, "record in whole bytes per event");
+  return (int64_t)HsRecord<P, typename A::V>::WORDS * 16 / A::EW;
+}
+
+// One batch through the split kernels: chunk = workspace / (2 records per event),
+// a multiple of the currents kernel's events per CTA; the graph key holds every
 // launch argument, so a call with other buffers or parameters re-captures.
 template <class P, class R>
 cudaError_t launch_split_impl(int proc, const SigLaunch& l, const Couplings<R>& cp, int mode, void* ws,
                               int64_t ws_bytes, cudaStream_t s) {
-  using RC = HsRecord<P, R>;
-  constexpr int64_t rec_bytes = (int64_t)RC::WORDS * 16;
+  constexpr int64_t rec_bytes = split_record_bytes<P, R>();
   int64_t chunk = ws_bytes / (2 * rec_bytes);
   // whole waves of the amplitudes kernel (all helicities good) where the
   // workspace allows: a partial last wave per chunk idles SMs
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return cudaGetLastError();
-  const int64_t wave = (int64_t)nsm * HsCfg<P, R>::CTAS * HsCfg<P, R>::EVMIN;
+  const int64_t wave = (int64_t)nsm * HsCfg<P, R>::CTAS * HsCfg<P, R>::EVMIN * HsCfg<P, R>::EW;
   chunk -= chunk >= wave ? chunk % wave : chunk % HsSplitA<P, R>::EV;
   if (chunk < HsSplitA<P, R>::EV) return cudaErrorInvalidValue;
   if (l.nevt == 0) return cudaSuccess;
@@ -178,8 +188,8 @@ cudaError_t launch_split_impl(int proc, const SigLaunch& l, const Couplings<R>& 
                                                                   const Couplings<double>&, int, void*, \
                                                                   int64_t, cudaStream_t);               \
   int64_t split_record_bytes_p##N(int mode) {                                                           \
-    return mode == 0 ? (int64_t)HsRecord<Proc##N, double>::WORDS * 16                                    \
-                     : (int64_t)HsRecord<Proc##N, float>::WORDS * 16;                                    \
+    return mode == 0 ? split_record_bytes<Proc##N, double>()                                            \
+                     : split_record_bytes<Proc##N, float>();                                             \
   }                                                                                                      \
   cudaError_t launch_sigmakin_split_p##N(const SigLaunch& l, int mode, void* ws, int64_t ws_bytes,      \
                                          cudaStream_t s) {                                               \

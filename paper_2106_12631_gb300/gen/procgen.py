@@ -1431,8 +1431,8 @@ class SharedProgram:
             "  static constexpr int HS_NSC = 0;",
             "  static constexpr int HS_NSLOT = %d;   // current variant slots per event" % self.nslots,
             "  static constexpr int HS_XCAP = %d;    // amputated-current slots per event and chunk" % self.xcap,
+            "  static constexpr int HS_NVT = %d;" % (1 << self.n),
             "  static constexpr int HS_NXCHUNK = %d;" % len(self.chunks),
-            "  static constexpr int HS_XBUFS = %d;   // chunk buffers" % (1 if len(self.chunks) == 1 else 2),
             "  static constexpr int HS_NITEM = %d;" % t["nitems"],
             "  static constexpr int HS_NLEVEL = %d;" % (len(t["level_start"]) - 1),
             "  static constexpr int HS_NAMP = %d;" % t["namps"],
@@ -1680,6 +1680,7 @@ class OrderedProgram:
         self.nslots = self.nx = self.nsc = 0
         self.levels, self.xitems, self.ext = [[], []], [], []
         self.kinds = []
+        self.vrows = {}     # leg sets of the contractions' operands -> rows of the variant table
         self._program()
 
     # ---- storage and momenta -------------------------------------------------
@@ -1862,7 +1863,7 @@ class OrderedProgram:
         out.append("static __constant__ int kHsXItem%d[2] = {%d, %d};  // item range of the contractions' operands"
                    % (pid, xitem_start[0], xitem_start[1]))
         var = []
-        for S in range(1 << self.n):
+        for S in self.vrows:
             for ih in range(nh):
                 v = k = 0
                 for l in range(self.n):
@@ -1884,8 +1885,8 @@ class OrderedProgram:
             "  static constexpr int HS_NSLOT = %d;   // current variant slots per event" % self.nslots,
             "  static constexpr int HS_XCAP = %d;    // slots per event of the contractions' further operands" % self.xcap,
             "  static constexpr int HS_NSC = %d;     // scalar products per event" % self.nsc,
+            "  static constexpr int HS_NVT = %d;      // rows of the variant table" % len(self.vrows),
             "  static constexpr int HS_NXCHUNK = 1;",
-            "  static constexpr int HS_XBUFS = 1;",
             "  static constexpr int HS_NITEM = %d;" % t["nitems"],
             "  static constexpr int HS_NLEVEL = %d;" % (len(lv) - 1),
             "  // operations: items per event, contractions + flow sums per helicity",
@@ -1907,13 +1908,16 @@ class OrderedProgram:
         index = {tuple(gl[k] for k in p): i for i, p in enumerate(itertools.permutations(range(4)))}
         G = lambda *w: "G" + "".join("%d" % l for l in w)
         flops = 0
-        started = set()
+
+        def row(legs):
+            """Row of the variant table of a leg set, numbered in order of use."""
+            return self.vrows.setdefault(sum(1 << l for l in legs), len(self.vrows))
 
         def ref(table, nm):
             first, legs = table[nm]
             arr = {id(self.cur): "cur[%d + vt[%d]]", id(self.x): "xb[%d + vt[%d]]",
                    id(self.sc): "xb.scalar(%d + vt[%d])"}[id(table)]
-            return arr % (first, sum(1 << l for l in legs) * nh)
+            return arr % (first, row(legs) * nh)
 
         def add(word, sign, a):
             nonlocal flops
@@ -1922,7 +1926,7 @@ class OrderedProgram:
             return "flow_add<%d>(J[%d], %s);" % (0 if sign > 0 else 1, s, a)
 
         L = ["  // J_s of one helicity: operands cur[..] (currents), xb[..] and xb.scalar(..), variant of a leg",
-             "  // set S for this helicity = vt[S * NHEL]; J in the order of the colour chains",
+             "  // set for this helicity = vt[its row * NHEL]; J in the order of the colour chains",
              "  template <class R, class CUR, class XB>",
              "  static __device__ __forceinline__ void hs_contract(int, const CUR& cur, const XB& xb,"
              " const uint8_t* __restrict__ vt, cx<R>* J) {"]
