@@ -128,13 +128,13 @@ struct Proc1 {
       default: break;
     }
   }
-  static constexpr int NMOM = 5;
-  static constexpr int NPROP = 2;
   static constexpr int NFINAL = 2;
   // floating-point operations per helicity: diagram program, CUDA-core colour sum
   static constexpr long FLOPS_AMP = 604;
   static constexpr long FLOPS_CSUM = 9;
   static constexpr double NORM = 1.0 / 4.0;  // 1/(helicity avg x colour avg x symmetry)
+  static constexpr int NMOM = 5;
+  static constexpr int NPROP = 2;
   // momentum table: {0 physical / 1 all-outgoing sum, leg mask, mask of legs entering as -p}
   static __host__ __device__ constexpr int mom(int j, int k) {
     constexpr int t[NMOM][3] = {{0, 1, 0}, {0, 2, 0}, {0, 4, 0}, {0, 8, 0}, {1, 3, 3}};

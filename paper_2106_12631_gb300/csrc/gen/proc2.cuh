@@ -159,13 +159,13 @@ struct Proc2 {
       default: break;
     }
   }
-  static constexpr int NMOM = 9;
-  static constexpr int NPROP = 3;
   static constexpr int NFINAL = 2;
   // floating-point operations per helicity: diagram program, CUDA-core colour sum
   static constexpr long FLOPS_AMP = 898;
   static constexpr long FLOPS_CSUM = 25;
   static constexpr double NORM = 1.0 / 256.0;  // 1/(helicity avg x colour avg x symmetry)
+  static constexpr int NMOM = 9;
+  static constexpr int NPROP = 3;
   // momentum table: {0 physical / 1 all-outgoing sum, leg mask, mask of legs entering as -p}
   static __host__ __device__ constexpr int mom(int j, int k) {
     constexpr int t[NMOM][3] = {{0, 1, 0}, {0, 2, 0}, {0, 4, 0}, {0, 8, 0}, {1, 1, 1}, {1, 2, 2}, {1, 3, 3}, {1, 5, 1}, {1, 6, 2}};
@@ -306,5 +306,6 @@ struct Proc2 {
     }
     return m2;
   }
+  using GradProgram = struct Proc2;  // program of the helicity-shared adjoint
 };
 }  // namespace mg

@@ -501,10 +501,10 @@ template <class P>
 cudaError_t launch_grad_impl(const GradLaunch& l, int mode, cudaStream_t s) {
   GradArgs a{l.nevt, l.ecm, l.rnd, l.nrows, l.mask, l.gout, l.grad, l.me, l.pp, l.st};
   switch (mode) {
-    case 0: return launch_hs_grad_variant<P, double>(a, l.cd, s);
+    case 0: return launch_hs_grad_variant<typename P::GradProgram, double>(a, l.cd, s);
     case 1:
     case 2:
-    case 5: return launch_hs_grad_variant<P, float>(a, l.cf, s);
+    case 5: return launch_hs_grad_variant<typename P::GradProgram, float>(a, l.cf, s);
     case 3: return launch_grad_variant<P, double>(a, l.cd, s);
     case 4: return launch_grad_variant<P, float>(a, l.cf, s);
   }

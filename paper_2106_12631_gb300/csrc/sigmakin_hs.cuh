@@ -55,7 +55,11 @@ struct HsCfg {
   static constexpr int EW = LaneOf<V>::EW;
   static constexpr int NT = P::NCOLOR < 6 ? 128 : EW == 2 ? MG_HS_NT : 256;
   static constexpr int EVMIN = (NT / P::NHEL) > 0 ? (NT / P::NHEL) : 1;  // units, all helicities good
-  static constexpr int MORE = P::NCOLOR >= 24 ? 1 : EW == 1 || P::NCOLOR == 1 ? 4 : (P::NCOLOR >= 6 ? 1 : 2);
+  // room for groups of fewer helicities than all: four times the units (one
+  // flow: four of the sixteen helicities of e+e- -> mu+mu- are good), two times;
+  // none for the larger programs, whose shared memory then admits more CTAs per
+  // SM (gg -> t t~ g FP64, 50021 events: 2449 -> 2226 us)
+  static constexpr int MORE = P::NCOLOR == 1 ? 4 : P::NCOLOR >= 6 ? 1 : EW == 1 ? 4 : 2;
   static constexpr int EVWANT = (MORE * EVMIN) < 32 ? MORE * EVMIN : 32;
   // shared memory for the currents and the contractions' operands
   static constexpr int CTAS = P::NCOLOR < 6 || sizeof(R) != 4 ? 1 : EW == 2 ? (P::NCOLOR >= 24 ? 1 : MG_HS_CTAS)
@@ -765,10 +769,10 @@ __device__ __forceinline__ void ord_xitem(const HsItem& it, const HsSlots<P, R, 
   W4<R> o, o2;
   if (it.type <= 21) {  // two words
     const HsItemExt ext = P::hs_item_ext()[it.in3()];
-    if (it.type == 21) {
+    if (P::HS_FOUR && it.type == 21) {
       ord_g3(cur[it.in[0]], cur[it.in[1]], cur[it.in[2]], cur[ext.in[0]], cur[ext.in[1]], cur[ext.in[2]], K, ext.k,
              pr[it.prop].im, o, o2);
-    } else if (it.type == 19) {
+    } else if (P::HS_FOUR && it.type == 19) {
       const W4<R> c = row_slash(cur[it.in[2]], cur[ext.in[2]]);
       const cx<R> s = mul_i(pr[it.prop]);
       o = scale(row_kslash_m(w4_add(row_slash(cur[it.in[0]], cur[it.in[1]]), c), K + 4 * it.k0, cp.mt), s);
@@ -779,7 +783,7 @@ __device__ __forceinline__ void ord_xitem(const HsItem& it, const HsSlots<P, R, 
       o2 = w4_sub(slash_col(cur[ext.in[1]], cur[ext.in[0]]), c);
     }
     xb.set(it.out + HS_WORD, o2);
-  } else if (it.type == 22) {
+  } else if (P::HS_FOUR && it.type == 22) {
     const W4<R> g = ord_v3(cur[it.in[2]], cur[it.in3()], K + 4 * it.k0, K + 4 * it.k1);
     o = w4_lower(w4_sub(vector_pair(cur[it.in[0]], cur[it.in[1]]), g));
   } else if (it.type == 23) {

@@ -762,7 +762,7 @@ def bf16_colour_image(cnum) -> np.ndarray:
     return img.view(np.uint32)
 
 
-ORDERED_PROCS = (4,)  # processes evaluated by the ordered program
+ORDERED_PROCS = (3, 4)  # processes evaluated by the ordered program
 
 
 def program(proc: Process, em: "Emitter"):
@@ -770,47 +770,9 @@ def program(proc: Process, em: "Emitter"):
     return (OrderedProgram if proc.spec.pid in ORDERED_PROCS else SharedProgram)(proc, em)
 
 
-def generate(pid: int) -> str:
-    proc = Process(PROCS[pid])
-    em = Emitter(proc)
-    # physical momenta first so that external legs have fixed slots
-    for leg in range(proc.n):
-        em.momentum_phys(leg)
-    body = em.emit()
-    spec = proc.spec
-    ncol = em.coef.shape[1]
-    nflow_used = int(np.count_nonzero(np.any(em.coef != 0, axis=0)))
-    assert nflow_used == ncol
-    coefs = set(complex(z) for z in em.coef.reshape(-1) if z != 0)
-    out = []
-    out.append("// GENERATED by paper_2106_12631_gb300/gen/procgen.py -- do not edit.")
-    out.append("// Process %d: %s (%s)" % (pid, spec.name, " ".join(L.name for L in spec.legs)))
-    out.append("// %d Feynman diagrams (%d amplitude terms), %d colour flows, %d wavefunctions"
-               % (proc.ndiagrams, len(proc.amps), ncol, em.ncurrents))
-    out.append("// colour-flow coefficients used: %s" % sorted(coefs, key=lambda z: (z.real, z.imag)))
-    out.append("#pragma once")
-    out.append("namespace mg {")
-    sp = program(proc, em)
-    out.extend(sp.emit_tables(pid))
-    img = bf16_colour_image(em.cnum)
-    out.append("// colour-matrix numerators as the BF16 B operand of the tensor-core colour sum")
-    out.append("static __device__ __align__(16) const uint32_t kColourB%d[%d] = {%s};"
-               % (pid, img.size, ", ".join("0x%08x" % int(w) for w in img)))
-    out.append("struct Proc%d {" % pid)
-    out.append("  static constexpr int NPAR = %d;" % proc.n)
-    out.append("  static constexpr int NHEL = %d;" % (1 << proc.n))
-    out.append("  static constexpr int NCOLOR = %d;" % ncol)
-    out.append("  static constexpr int NDIAGRAMS = %d;" % proc.ndiagrams)
-    out.append("  static constexpr int NAMPS = %d;" % len(proc.amps))
-    out.extend(sp.struct_lines(pid))
-    out.append("  static constexpr int NMOM = %d;" % len(em.mom))
-    out.append("  static constexpr int NPROP = %d;" % len(em.props))
-    out.append("  static constexpr int NFINAL = %d;" % (proc.n - 2))
-    out.append("  // floating-point operations per helicity: diagram program, CUDA-core colour sum")
-    out.append("  static constexpr long FLOPS_AMP = %d;" % em.flops)
-    out.append("  static constexpr long FLOPS_CSUM = %d;" % colour_sum_flops(em.cnum))
-    out.append("  static constexpr double NORM = 1.0 / %d.0;  // 1/(helicity avg x colour avg x symmetry)"
-               % (spec.hel_avg * spec.col_avg * spec.sym))
+def momentum_lines(em, spec) -> list:
+    """Momentum-table and propagator constants of a process struct."""
+    out = ["  static constexpr int NMOM = %d;" % len(em.mom), "  static constexpr int NPROP = %d;" % len(em.props)]
     # momentum table: for each entry, the legs (signs: incoming legs enter as -p)
     mrows = []
     for key in em.mom:
@@ -855,6 +817,49 @@ def generate(pid: int) -> str:
     out.append("    constexpr int t[NMOM][2] = {%s};" % ", ".join("{%d, %d}" % tuple(r) for r in pof))
     out.append("    return t[j][k];")
     out.append("  }")
+    return out
+
+
+def generate(pid: int) -> str:
+    proc = Process(PROCS[pid])
+    em = Emitter(proc)
+    # physical momenta first so that external legs have fixed slots
+    for leg in range(proc.n):
+        em.momentum_phys(leg)
+    body = em.emit()
+    spec = proc.spec
+    ncol = em.coef.shape[1]
+    nflow_used = int(np.count_nonzero(np.any(em.coef != 0, axis=0)))
+    assert nflow_used == ncol
+    coefs = set(complex(z) for z in em.coef.reshape(-1) if z != 0)
+    out = []
+    out.append("// GENERATED by paper_2106_12631_gb300/gen/procgen.py -- do not edit.")
+    out.append("// Process %d: %s (%s)" % (pid, spec.name, " ".join(L.name for L in spec.legs)))
+    out.append("// %d Feynman diagrams (%d amplitude terms), %d colour flows, %d wavefunctions"
+               % (proc.ndiagrams, len(proc.amps), ncol, em.ncurrents))
+    out.append("// colour-flow coefficients used: %s" % sorted(coefs, key=lambda z: (z.real, z.imag)))
+    out.append("#pragma once")
+    out.append("namespace mg {")
+    sp = program(proc, em)
+    out.extend(sp.emit_tables(pid))
+    img = bf16_colour_image(em.cnum)
+    out.append("// colour-matrix numerators as the BF16 B operand of the tensor-core colour sum")
+    out.append("static __device__ __align__(16) const uint32_t kColourB%d[%d] = {%s};"
+               % (pid, img.size, ", ".join("0x%08x" % int(w) for w in img)))
+    out.append("struct Proc%d {" % pid)
+    out.append("  static constexpr int NPAR = %d;" % proc.n)
+    out.append("  static constexpr int NHEL = %d;" % (1 << proc.n))
+    out.append("  static constexpr int NCOLOR = %d;" % ncol)
+    out.append("  static constexpr int NDIAGRAMS = %d;" % proc.ndiagrams)
+    out.append("  static constexpr int NAMPS = %d;" % len(proc.amps))
+    out.extend(sp.struct_lines(pid))
+    out.append("  static constexpr int NFINAL = %d;" % (proc.n - 2))
+    out.append("  // floating-point operations per helicity: diagram program, CUDA-core colour sum")
+    out.append("  static constexpr long FLOPS_AMP = %d;" % em.flops)
+    out.append("  static constexpr long FLOPS_CSUM = %d;" % colour_sum_flops(em.cnum))
+    out.append("  static constexpr double NORM = 1.0 / %d.0;  // 1/(helicity avg x colour avg x symmetry)"
+               % (spec.hel_avg * spec.col_avg * spec.sym))
+    out.extend(momentum_lines(em, spec))
     out.append("  static __device__ __forceinline__ const uint32_t* colour_bf16_image() { return kColourB%d; }" % pid)
     out.append("  // colour matrix = CNUM / CDEN (real symmetric)")
     out.append("  static constexpr int CDEN = %d;" % em.cden)
@@ -896,7 +901,18 @@ def generate(pid: int) -> str:
                    " const cx<R>* __restrict__ prop, const int* hel, const Couplings<R>& cp, R* pb) {")
         out.append(GradEmitter(em).emit())
         out.append("  }")
+    own_grad = pid in GRAD_PROCS and isinstance(sp, SharedProgram)
+    if pid in GRAD_PROCS:
+        out.append("  using GradProgram = struct Proc%d%s;  // program of the helicity-shared adjoint" % (pid, "" if own_grad else "Grad"))
     out.append("};")
+    if pid in GRAD_PROCS and not own_grad:
+        gp = SharedProgram(proc, em)
+        out.extend(gp.emit_tables(pid, "Grad"))
+        out.append("// the diagram-wise helicity-shared program, whose adjoint is generated")
+        out.append("struct Proc%dGrad : Proc%d {" % (pid, pid))
+        out.extend(gp.struct_lines(pid, "Grad"))
+        out.extend(momentum_lines(em, spec))
+        out.append("};")
     out.append("}  // namespace mg")
     return "\n".join(out) + "\n"
 
@@ -1332,7 +1348,7 @@ class SharedProgram:
             raise ValueError(kind)
         return (t, a, b, c, flag, out, ins, k0, k1, prop)
 
-    def emit_tables(self, pid: int) -> list:
+    def emit_tables(self, pid: int, suffix: str = "") -> list:
         nh = 1 << self.n
         items, level_start = [], []
         cur_level = -1
@@ -1383,12 +1399,12 @@ class SharedProgram:
                    " currents in %d chunk(s) of <= %d slots, %d amplitudes; %d flops per event (all helicities)"
                    % (len(self.order), len(level_start) - 1, self.nslots, len(self.xoff), len(self.chunks),
                       self.xcap, len(amps), self.flops_items + nh * self.flops_amps_hel))
-        out.append("static __device__ const HsItem kHsItems%d[%d] = {%s};" % (
-            pid, len(items), ", ".join("{%d, {%s}, %d, %d, %d, %d, %d, %d, %d, %d}" % (
+        out.append("static __device__ const HsItem kHsItems%s[%d] = {%s};" % (
+            "%d%s" % (pid, suffix), len(items), ", ".join("{%d, {%s}, %d, %d, %d, %d, %d, %d, %d, %d}" % (
                 o, ", ".join(map(str, ins)), t, a, b, c, flag, k0, k1, pr)
                 for (t, a, b, c, flag, o, ins, k0, k1, pr) in items)))
-        out.append("static __constant__ int kHsXItem%d[%d] = {%s};  // item ranges of the amputated chunks"
-                   % (pid, len(xitem_start), ", ".join(map(str, xitem_start))))
+        out.append("static __constant__ int kHsXItem%s[%d] = {%s};  // item ranges of the amputated chunks"
+                   % ("%d%s" % (pid, suffix), len(xitem_start), ", ".join(map(str, xitem_start))))
         # variant of every leg set S for every event helicity h: the bits of the
         # legs of S in ascending order, leg l being +1 when bit n-1-l of h is set
         var = []
@@ -1400,8 +1416,8 @@ class SharedProgram:
                         v |= ((ih >> (self.n - 1 - l)) & 1) << k
                         k += 1
                 var.append(v)
-        out.append("static __device__ __align__(16) const uint8_t kHsVar%d[%d] = {%s};  // [leg set][helicity]"
-                   % (pid, len(var), ", ".join(map(str, var))))
+        out.append("static __device__ __align__(16) const uint8_t kHsVar%s[%d] = {%s};  // [leg set][helicity]"
+                   % ("%d%s" % (pid, suffix), len(var), ", ".join(map(str, var))))
         return out
 
     def _exact_flops(self, items, amps):
@@ -1416,7 +1432,7 @@ class SharedProgram:
         self.flops_amps_hel = sum(FLOPS["DOT4"] + FLOPS["jamp"] * len(g["flows"]) + FLOPS["W4ADD"] * (len(g["ys"]) - 1)
                                   for g in groups)
 
-    def struct_lines(self, pid: int) -> list:
+    def struct_lines(self, pid: int, suffix: str = "") -> list:
         t = self.tables
 
         def table_fn(name, vals):
@@ -1443,9 +1459,9 @@ class SharedProgram:
             "  static constexpr long HS_FLOPS_AMP_HEL = %d;" % self.flops_amps_hel,
             "  // item ranges of the current levels and of the amputated chunks; amplitude ranges of the chunks",
         ] + table_fn("hs_level", t["level_start"]) + [
-            "  static __device__ __forceinline__ int hs_xitem(int c) { return kHsXItem%d[c]; }" % pid,
-            "  static __device__ __forceinline__ const uint8_t* hs_variants() { return kHsVar%d; }" % pid,
-            "  static __device__ __forceinline__ const HsItem* hs_items() { return kHsItems%d; }" % pid,
+            "  static __device__ __forceinline__ int hs_xitem(int c) { return kHsXItem%d%s[c]; }" % (pid, suffix),
+            "  static __device__ __forceinline__ const uint8_t* hs_variants() { return kHsVar%d%s; }" % (pid, suffix),
+            "  static __device__ __forceinline__ const HsItem* hs_items() { return kHsItems%d%s; }" % (pid, suffix),
         ] + self._contract_code() + self._contract_adj_code()
 
     @staticmethod
@@ -1675,7 +1691,7 @@ class OrderedProgram:
         self.p, self.em, self.n = proc, emitter, proc.n
         self.q, self.Q = 2, 3
         self.gl = proc.gluon_legs()
-        assert len(self.gl) == 4 and proc.spec.root == self.Q
+        assert len(self.gl) in (3, 4) and proc.spec.root == self.Q
         self.cur, self.x, self.sc = {}, {}, {}      # name -> (first slot or scalar, legs)
         self.nslots = self.nx = self.nsc = 0
         self.levels, self.xitems, self.ext = [[], []], [], []
@@ -1759,7 +1775,71 @@ class OrderedProgram:
         for v in range(self._add(cur, "V", vq)):
             self._item(L1, self.T_PAIR, cur["V"][0] + v, [self._at(cur, "q", vq, v), self._at(cur, "Q", vq, v)],
                        prop=self._prop(vq, "g"), kind="pair")
-        # ---- what the contractions read besides the two-leg currents -----------------
+        self._operands3(pairs) if len(gl) == 3 else self._operands4(pairs)
+        self.xcap = self.nx
+        self.chunks = [list(x)]
+        self.xoff = {nm: x[nm][0] for nm in x}
+        self.order = list(cur)
+        self.flops_items = (sum({0: FLOPS["ixxxxx"], 1: FLOPS["oxxxxx"], 2: FLOPS["vxxxxx"]}[t[0]] for t in L0)
+                            + sum(self.COST[k] for k in self.kinds))
+
+    # what the contractions read besides the two-leg currents
+    def _two_words(self, pairs, ends):
+        """R(ab) and R(ba), amputated C(ab) and C(ba): one item for both words (a < b), which
+        share the term with G(ab) = -G(ba)."""
+        cur, x, q, Q = self.cur, self.x, self.q, self.Q
+        G = lambda *w: "G" + "".join("%d" % l for l in w)
+        for nm, end, t in (("R", q, self.T_ROW2), ("C", Q, self.T_COL2)):
+            if nm not in ends:
+                continue
+            for a, b in pairs:
+                legs = tuple(sorted((end, a, b)))
+                self._add(x, "%s%d%d" % (nm, a, b), legs)
+                self._add(x, "%s%d%d" % (nm, b, a), legs)
+                # row: R(a) G(b), R(b) G(a); column: C(b) G(a), C(a) G(b)
+                f, g = (a, b) if end == q else (b, a)
+                for v in range(8):
+                    at = lambda n_: self._at(cur, n_, legs, v)
+                    self._item(self.xitems, t, x["%s%d%d" % (nm, a, b)][0] + v,
+                               [at("%s%d" % (nm, f)), at(G(g)), at("q" if end == q else "Q")],
+                               ext=([at("%s%d" % (nm, g)), at(G(f)), at(G(a, b))], [0] * 6),
+                               k0=self._k(legs) if end == q else 0, prop=self._prop(legs, "t") if end == q else 0,
+                               kind="row2" if end == q else "col2")
+
+    def _dot(self, m, n, legs):
+        """Scalar products of two gluon lines (four-gluon vertices)."""
+        legs = tuple(sorted(legs))
+        nm = m + "." + n
+        for v in range(self._add(self.sc, nm, legs)):
+            self._item(self.xitems, self.T_DOT, self.sc[nm][0] + v,
+                       [self._at(self.cur, m, legs, v), self._at(self.cur, n, legs, v)], kind="dot")
+
+    def _operands3(self, pairs):
+        """A(123) = R(1) . C(23) + G(12) . A(3) - (G(12) . E(3)) + G(23) . E(1) + {V, 1, 2, 3}
+        with A(g) = u gamma C(g), E(g) = -V3(V, g), amputated."""
+        cur, x, q, Q, gl = self.cur, self.x, self.q, self.Q, self.gl
+        G = lambda *w: "G" + "".join("%d" % l for l in w)
+        self._two_words(pairs, "C")
+        kV = self._k((q, Q))
+        for nm in "AE":
+            for g in gl:
+                legs = tuple(sorted((q, Q, g)))
+                for v in range(self._add(x, "%s%d" % (nm, g), legs)):
+                    at = lambda n_: self._at(cur, n_, legs, v)
+                    out = x["%s%d" % (nm, g)][0] + v
+                    if nm == "A":
+                        self._item(self.xitems, self.T_W, out, [at("q"), at("C%d" % g)], kind="w")
+                    else:
+                        self._item(self.xitems, self.T_P, out, [at("V"), at(G(g))], kV, self._k((g,)), kind="p")
+        for g in gl:
+            self._dot("V", G(g), (q, Q, g))
+        for a, b in pairs:
+            self._dot(G(a), G(b), (a, b))
+
+    def _operands4(self, pairs):
+        cur, x, sc, q, Q, gl = self.cur, self.x, self.sc, self.q, self.Q, self.gl
+        G = lambda *w: "G" + "".join("%d" % l for l in w)
+        vq = (q, Q)
         X = self.xitems
         words = list(itertools.permutations(gl, 2))
         # three-gluon currents: words (i j k) and (i k j) of each set i < j < k
@@ -1795,22 +1875,7 @@ class OrderedProgram:
             for v in range(self._add(x, nm, four)):
                 self._item(X, self.T_P, x[nm][0] + v, [self._at(cur, G(*ab), four, v), self._at(cur, G(*cd), four, v)],
                            self._k(ab), self._k(cd), kind="p")
-        # R(ab) and R(ba), amputated C(ab) and C(ba): one item for both words (a < b), which share
-        # the term with G(ab) = -G(ba)
-        for nm, end, t in (("R", q, self.T_ROW2), ("C", Q, self.T_COL2)):
-            for a, b in pairs:
-                legs = tuple(sorted((end, a, b)))
-                self._add(x, "%s%d%d" % (nm, a, b), legs)
-                self._add(x, "%s%d%d" % (nm, b, a), legs)
-                # row: R(a) G(b), R(b) G(a); column: C(b) G(a), C(a) G(b)
-                f, g = (a, b) if end == q else (b, a)
-                for v in range(8):
-                    at = lambda n_: self._at(cur, n_, legs, v)
-                    self._item(X, t, x["%s%d%d" % (nm, a, b)][0] + v,
-                               [at("%s%d" % (nm, f)), at(G(g)), at("q" if end == q else "Q")],
-                               ext=([at("%s%d" % (nm, g)), at(G(f)), at(G(a, b))], [0] * 6),
-                               k0=self._k(legs) if end == q else 0, prop=self._prop(legs, "t") if end == q else 0,
-                               kind="row2" if end == q else "col2")
+        self._two_words(pairs, "RC")
         # R(a) gamma C(b)
         for a, b in words:
             legs = tuple(sorted((q, Q, a, b)))
@@ -1818,28 +1883,16 @@ class OrderedProgram:
             for v in range(self._add(x, nm, legs)):
                 at = lambda n_: self._at(cur, n_, legs, v)
                 self._item(X, self.T_W, x[nm][0] + v, [at("R%d" % a), at("C%d" % b)], kind="w")
-        # scalar products of gluon lines (four-gluon vertices)
-        def dot(m, n, legs):
-            nm = m + "." + n
-            for v in range(self._add(sc, nm, legs)):
-                self._item(X, self.T_DOT, sc[nm][0] + v, [self._at(cur, m, tuple(sorted(legs)), v),
-                                                         self._at(cur, n, tuple(sorted(legs)), v)], kind="dot")
         for a, b in pairs:
-            dot(G(a), G(b), (a, b))
+            self._dot(G(a), G(b), (a, b))
         for g in gl:
-            dot("V", G(g), (q, Q, g))
+            self._dot("V", G(g), (q, Q, g))
         for a, b in pairs:
-            dot("V", G(a, b), (q, Q, a, b))
+            self._dot("V", G(a, b), (q, Q, a, b))
         for a, b in pairs:
             for g in gl:
                 if g not in (a, b):
-                    dot(G(g), G(a, b), (g, a, b))
-        self.xcap = self.nx
-        self.chunks = [list(x)]
-        self.xoff = {nm: x[nm][0] for nm in x}
-        self.order = list(cur)
-        self.flops_items = (sum({0: FLOPS["ixxxxx"], 1: FLOPS["oxxxxx"], 2: FLOPS["vxxxxx"]}[t[0]] for t in L0)
-                            + sum(self.COST[k] for k in self.kinds))
+                    self._dot(G(g), G(a, b), (g, a, b))
 
     # ---- emission -----------------------------------------------------------------------
     def emit_tables(self, pid: int) -> list:
@@ -1881,6 +1934,7 @@ class OrderedProgram:
         return [
             "  // ordered program (tables above)",
             "  static constexpr bool HS_ORDERED = true;",
+            "  static constexpr bool HS_FOUR = %s;  // items of the four-gluon program" % ("true" if len(self.gl) == 4 else "false"),
             "  static constexpr int HS_GS_POWER = %d;  // |M|^2 carries g_s to this power, applied to the sum" % (2 * len(self.gl)),
             "  static constexpr int HS_NSLOT = %d;   // current variant slots per event" % self.nslots,
             "  static constexpr int HS_XCAP = %d;    // slots per event of the contractions' further operands" % self.xcap,
@@ -1905,7 +1959,7 @@ class OrderedProgram:
     def _contract_code(self) -> list:
         nh = 1 << self.n
         gl = self.gl
-        index = {tuple(gl[k] for k in p): i for i, p in enumerate(itertools.permutations(range(4)))}
+        index = {tuple(gl[k] for k in p): i for i, p in enumerate(itertools.permutations(range(len(gl))))}
         G = lambda *w: "G" + "".join("%d" % l for l in w)
         flops = 0
 
@@ -1930,6 +1984,35 @@ class OrderedProgram:
              "  template <class R, class CUR, class XB>",
              "  static __device__ __forceinline__ void hs_contract(int, const CUR& cur, const XB& xb,"
              " const uint8_t* __restrict__ vt, cx<R>* J) {"]
+        if len(gl) == 3:
+            for a, b, c in itertools.permutations(gl):
+                if b < c:
+                    L.append("    { const W4<R> X = %s;" % ref(self.cur, "R%d" % a))
+                L.append("      J[%d] = dot4p(X, %s);" % (index[(a, b, c)], ref(self.x, "C%d%d" % (b, c))))
+                flops += 30
+                if b > c:
+                    L.append("    }")
+            for b, c in itertools.combinations(gl, 2):
+                (g,) = [l for l in gl if l not in (b, c)]
+                L.append("    { const W4<R> Y = %s;" % ref(self.cur, G(b, c)))
+                L.append("      const cx<R> e = dot4p(Y, %s), a = dot4p(Y, %s) - e;"
+                         % (ref(self.x, "E%d" % g), ref(self.x, "A%d" % g)))
+                flops += 62
+                L.append("      " + " ".join([add((b, c, g), 1, "a"), add((c, b, g), -1, "a"),
+                                              add((g, b, c), 1, "e"), add((g, c, b), -1, "e")]))
+                L.append("    }")
+            x_, y_, z_ = gl
+            for g, (m, n) in ((x_, (y_, z_)), (y_, (x_, z_)), (z_, (x_, y_))):
+                L.append("    const cx<R> t%d = %s * %s;" % (g, ref(self.sc, "V." + G(g)),
+                                                            ref(self.sc, G(m) + "." + G(n))))
+            L.append("    const cx<R> w = t%d + t%d + t%d;" % tuple(gl))
+            flops += 18 + 4
+            for g, (m, n) in ((x_, (y_, z_)), (y_, (x_, z_)), (z_, (x_, y_))):
+                L.append("    { const cx<R> l = vertex4(t%d, w); %s %s }" % (g, add((m, g, n), 1, "l"), add((n, g, m), 1, "l")))
+                flops += 4
+            L.append("  }")
+            self.flops_amps_hel = flops
+            return L
         # R(ab) . C(cd): one per flow, the first term of its sum
         for ab in itertools.combinations(gl, 2):
             cd = tuple(g for g in gl if g not in ab)
