@@ -53,13 +53,18 @@ template <class P, class R, int CS = CS_SIMT>
 struct HsCfg {
   using V = HsLane<P, R, CS>;
   static constexpr int EW = LaneOf<V>::EW;
-  static constexpr int NT = P::NCOLOR < 6 ? 128 : EW == 2 ? MG_HS_NT : 256;
+  // measured: 128 threads for pairs of g g -> t t~ events (2^20 events 565 us, 256
+  // threads 632 us) and for FP64 e+e- -> mu+mu- (200003 events 1256 us, 1301 us);
+  // 256 for FP64 g g -> t t~ (100003 events 914 us, 128 threads 974 us) and mixed
+  // e+e- -> mu+mu- (200003 events 91 us, 97 us), as for the larger processes
+  static constexpr int NT =
+      (P::NCOLOR == 2 && EW == 2) || (P::NCOLOR == 1 && sizeof(R) == 8) ? 128 : EW == 2 ? MG_HS_NT : 256;
   static constexpr int EVMIN = (NT / P::NHEL) > 0 ? (NT / P::NHEL) : 1;  // units, all helicities good
-  // room for groups of fewer helicities than all: four times the units (one
-  // flow: four of the sixteen helicities of e+e- -> mu+mu- are good), two times;
-  // none for the larger programs, whose shared memory then admits more CTAs per
-  // SM (gg -> t t~ g FP64, 50021 events: 2449 -> 2226 us)
-  static constexpr int MORE = P::NCOLOR == 1 ? 4 : P::NCOLOR >= 6 ? 1 : EW == 1 ? 4 : 2;
+  // room for groups of fewer helicities than all: four times the units with one
+  // flow (four of the sixteen helicities of e+e- -> mu+mu- are good); none for the
+  // others, whose shared memory then admits more CTAs per SM (2^20 pairs of
+  // g g -> t t~ events 629 -> 565 us, 50021 FP64 gg -> t t~ g events 2449 -> 2226 us)
+  static constexpr int MORE = P::NCOLOR == 1 ? 4 : 1;
   static constexpr int EVWANT = (MORE * EVMIN) < 32 ? MORE * EVMIN : 32;
   // shared memory for the currents and the contractions' operands
   static constexpr int CTAS = P::NCOLOR < 6 || sizeof(R) != 4 ? 1 : EW == 2 ? (P::NCOLOR >= 24 ? 1 : MG_HS_CTAS)
@@ -518,6 +523,43 @@ __device__ __forceinline__ void ext_fermion_dfl(const dfl* p, float m, int nsf, 
   }
 }
 
+// The same in FP64: the arithmetic of ixxxxx, oxxxxx and vxxxxx, its square roots
+// and quotients (most of the work in FP64) formed once for both helicities.
+__device__ __forceinline__ void ext_vector_fp64(const double* k, int nsv, W4<double>* w) {
+  const double kt = sqrt(k[1] * k[1] + k[2] * k[2]);
+  const double kk = sqrt(kt * kt + k[3] * k[3]);
+  double ct, st, cp, sp;
+  if (kt == 0.0) { ct = k[3] >= 0.0 ? 1.0 : -1.0; st = 0.0; cp = 1.0; sp = 0.0; }
+  else { ct = k[3] / kk; st = kt / kk; cp = k[1] / kt; sp = k[2] / kt; }
+  const double r2 = 0.70710678118654752440, b = nsv > 0 ? -r2 : r2;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const double a = h == 0 ? r2 : -r2;
+    w[h].w[0] = cx<double>(0.0, 0.0);
+    w[h].w[1] = cx<double>(a * ct * cp, b * -sp);
+    w[h].w[2] = cx<double>(a * ct * sp, b * cp);
+    w[h].w[3] = cx<double>(-a * st, 0.0);
+  }
+}
+__device__ __forceinline__ void ext_fermion_fp64(const double* p, double m, int nsf, bool row, W4<double>* w) {
+  cx<double> p0, p1;
+  helicity_chi(p, 1, p0, p1);
+  // chi_- = (-conj(c1), c0) of chi_+ = (c0, c1), c0 real
+  const cx<double> m0(-p1.re, p1.im), m1(p0.re, 0.0);
+  double wp, wm;
+  omegas(p, m, wp, wm);
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const bool plus = h == 1, chip = nsf > 0 ? plus : !plus;
+    const cx<double> c0 = chip ? p0 : m0, c1 = chip ? p1 : m1;
+    const double lo = nsf > 0 ? (plus ? wm : wp) : (plus ? -wp : wm);
+    const double hi = nsf > 0 ? (plus ? wp : wm) : (plus ? wm : -wp);
+    const cx<double> c[4] = {lo * c0, lo * c1, hi * c0, hi * c1};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[h].w[i] = row ? conj(c[(i + 2) & 3]) : c[i];
+  }
+}
+
 // Phase 1 of the forward kernels, in three parts:
 //   hs_setup_words   per-CTA constants: {momentum entry, line kind} per
 //                    propagator, a descriptor per momentum-table entry, and in
@@ -632,9 +674,9 @@ __device__ __forceinline__ void hs_tables(unsigned char* smem, const PhysParams&
   R* K = reinterpret_cast<R*>(smem + L::o_K);    // V [unit][NMOM][4]
   R* pr = reinterpret_cast<R*>(smem + L::o_pr);  // cx<V> [unit][NPROP]
   const int nep = (nev + EW - 1) / EW * EW;
-  // mixed mode: one thread per (event, leg), both helicities (consecutive items)
+  // one thread per (event, leg), both helicities (consecutive items)
   static_assert(NEXT == 2 * NPAR, "level 0: two helicities per leg");
-  constexpr int NE = DF ? NPAR : NEXT;
+  constexpr int NE = NPAR;
   for (int t = threadIdx.x; t < nep * (NM + NE); t += L::NT) {
     const bool mom = t < nep * NM;
     const int t2 = mom ? t : t - nep * NM, e = t2 / (mom ? NM : NE), j = t2 - e * (mom ? NM : NE);
@@ -693,28 +735,24 @@ __device__ __forceinline__ void hs_tables(unsigned char* smem, const PhysParams&
       }
     } else {
       const HsSlots<P, V, P::HS_NSLOT> cur{curs + u * CUR_EV};
+      const HsItem it = P::hs_items()[2 * j];
+      W4<R> o[2];
       if constexpr (DF) {
-        const HsItem it = P::hs_items()[2 * j];
         dfl k[4];
 #pragma unroll
         for (int mu = 0; mu < 4; ++mu) {
           const float2 v = reinterpret_cast<const float2*>(smem + L::o_p)[(es * NPAR + it.a) * 4 + mu];
           k[mu] = dfl{v.x, v.y};
         }
-        W4<R> o[2];
         if (it.type == 2) ext_vector_dfl(k, it.c, o);
         else ext_fermion_dfl(k, it.flag ? cp.mt : 0.0f, it.c, it.type == 1, o);
-        cur.set_lane(it.out, lane, o[0]);
-        cur.set_lane(P::hs_items()[2 * j + 1].out, lane, o[1]);
       } else {
-        const HsItem it = P::hs_items()[j];
         const double* k = reinterpret_cast<const double*>(smem + L::o_p) + (es * NPAR + it.a) * 4;
-        W4<R> o;
-        if (it.type == 0) o = ixxxxx<R>(k, it.flag ? cp.mt : R(0), it.b, it.c);
-        else if (it.type == 1) o = oxxxxx<R>(k, it.flag ? cp.mt : R(0), it.b, it.c);
-        else o = vxxxxx<R>(k, it.b, it.c);
-        cur.set_lane(it.out, lane, o);
+        if (it.type == 2) ext_vector_fp64(k, it.c, o);
+        else ext_fermion_fp64(k, it.flag ? cp.mt : 0.0, it.c, it.type == 1, o);
       }
+      cur.set_lane(it.out, lane, o[0]);
+      cur.set_lane(P::hs_items()[2 * j + 1].out, lane, o[1]);
     }
   }
   __syncthreads();
