@@ -26,14 +26,26 @@ template <int NF>
 struct RamboState {
   double c[NF], s[NF], cp[NF], sp[NF], e[NF];
   double q[NF][4];
-  double Q[4], M, b[3], g, a, x;
+  double Q[4], rM, b[3], g, a, x;  // rM = 1 / M
   double p[NF][4];   // massless momenta
   double xi;
   double k[NF][4];   // final momenta
+  double rk[NF];     // 1 / k[f][0] (massive case)
   double w;
 };
 
 constexpr double kTwoPi = 6.283185307179586477;
+
+// FP64 throughput bounds RAMBO (two FMAs per clock and SM; a square root or a
+// quotient takes a dozen of them), so the quotients by M and by the energies are
+// products with reciprocal square roots, sincospi needs no range reduction, and
+// a Newton step divides its FP64 residual in FP32.
+// sqrt and its reciprocal: the square root from the reciprocal's, corrected by its
+// residual; then the reciprocal by its own (each to rounding)
+__device__ __forceinline__ double sqrt_of_rsqrt(double t, double rt) {
+  const double s = t * rt;
+  return fma(0.5 * rt, fma(-s, s, t), s);
+}
 
 // r: 4 NF uniforms of the event (r[4i + j])
 template <int NF>
@@ -42,7 +54,7 @@ __device__ __forceinline__ void rambo_forward(const double* r, double ecm, const
   for (int f = 0; f < NF; ++f) {
     z.c[f] = 2.0 * r[4 * f] - 1.0;
     z.s[f] = sqrt(1.0 - z.c[f] * z.c[f]);
-    sincos(kTwoPi * r[4 * f + 1], &z.sp[f], &z.cp[f]);
+    sincospi(2.0 * r[4 * f + 1], &z.sp[f], &z.cp[f]);
     z.e[f] = -log(r[4 * f + 2] * r[4 * f + 3]);
     z.q[f][0] = z.e[f];
     z.q[f][1] = z.e[f] * z.s[f] * z.cp[f];
@@ -55,11 +67,13 @@ __device__ __forceinline__ void rambo_forward(const double* r, double ecm, const
 #pragma unroll
     for (int f = 0; f < NF; ++f) z.Q[mu] += z.q[f][mu];
   }
-  z.M = sqrt(z.Q[0] * z.Q[0] - z.Q[1] * z.Q[1] - z.Q[2] * z.Q[2] - z.Q[3] * z.Q[3]);
-  z.b[0] = -z.Q[1] / z.M; z.b[1] = -z.Q[2] / z.M; z.b[2] = -z.Q[3] / z.M;
-  z.g = z.Q[0] / z.M;
+  const double M2 = z.Q[0] * z.Q[0] - z.Q[1] * z.Q[1] - z.Q[2] * z.Q[2] - z.Q[3] * z.Q[3];
+  z.rM = rsqrt(M2);
+  z.rM = fma(z.rM, fma(-sqrt_of_rsqrt(M2, z.rM), z.rM, 1.0), z.rM);
+  z.b[0] = -z.Q[1] * z.rM; z.b[1] = -z.Q[2] * z.rM; z.b[2] = -z.Q[3] * z.rM;
+  z.g = z.Q[0] * z.rM;
   z.a = 1.0 / (1.0 + z.g);
-  z.x = ecm / z.M;
+  z.x = ecm * z.rM;
 #pragma unroll
   for (int f = 0; f < NF; ++f) {
     const double bq = z.b[0] * z.q[f][1] + z.b[1] * z.q[f][2] + z.b[2] * z.q[f][3];
@@ -76,10 +90,10 @@ __device__ __forceinline__ void rambo_forward(const double* r, double ecm, const
       for (int mu = 0; mu < 4; ++mu) z.k[f][mu] = z.p[f][mu];
     return;
   }
-  // Newton for sum_f sqrt(m_f^2 + xi^2 E_f^2) = ecm: first in FP32 to ~1e-6
-  // (cheap; GB300 runs FP64 at 1/64 of the FP32 rate), then FP64 steps until
-  // the residual is below 1e-15 ecm, plus one (quadratic convergence: the
-  // same root as iterating in FP64 from the start)
+  // Newton for sum_f sqrt(m_f^2 + xi^2 E_f^2) = ecm: first in FP32 to ~1e-7
+  // (cheap; GB300 runs FP64 at 1/64 of the FP32 rate), then FP64 steps until one
+  // starts from a residual below 1e-9 ecm (the step squares the error, and its
+  // FP32 quotient leaves 1e-7 of it: the root to rounding)
   float xf = (float)st.xi0;
   for (int it = 0; it < 12; ++it) {
     float fv = -(float)ecm, df = 0.0f;
@@ -94,29 +108,29 @@ __device__ __forceinline__ void rambo_forward(const double* r, double ecm, const
     if (fabsf(fv) <= 1e-6f * (float)ecm) break;
   }
   double xi = (isfinite(xf) && xf > 0.0f && xf <= 1.0f) ? (double)xf : st.xi0;  // else from the start
-  int extra = 0;
   for (int it = 0; it < 50; ++it) {
     double fv = -ecm, df = 0.0;
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
-      const double en = sqrt(st.m2[f] + xi * xi * z.p[f][0] * z.p[f][0]);
-      fv += en;
-      df += xi * z.p[f][0] * z.p[f][0] / en;
+      const double e2 = z.p[f][0] * z.p[f][0], t = fma(xi * xi, e2, st.m2[f]), rt = rsqrt(t);
+      fv += sqrt_of_rsqrt(t, rt);
+      df = fma(xi * e2, rt, df);
     }
-    xi -= fv / df;
-    if (fabs(fv) <= 1e-15 * ecm && ++extra >= 1) break;
+    xi -= fv * (double)(1.0f / (float)df);
+    if (fabs(fv) <= 1e-9 * ecm) break;
   }
   z.xi = xi;
   double w2 = 1.0, w3 = 0.0;
 #pragma unroll
   for (int f = 0; f < NF; ++f) {
     const double kk = xi * z.p[f][0];
-    const double en = sqrt(st.m2[f] + kk * kk);
+    const double t = fma(kk, kk, st.m2[f]), rt = rsqrt(t), en = sqrt_of_rsqrt(t, rt);
+    z.rk[f] = rt;
 #pragma unroll
     for (int k = 1; k < 4; ++k) z.k[f][k] = xi * z.p[f][k];
     z.k[f][0] = en;
-    w2 *= kk / en;
-    w3 += kk * kk / en;
+    w2 *= kk * rt;
+    w3 = fma(kk * kk, rt, w3);
   }
   double pw = 1.0;
 #pragma unroll
@@ -133,18 +147,18 @@ __device__ __forceinline__ void rambo_adjoint(const double* r, double ecm, const
     double xib = 0.0, fxi = 0.0;
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
-      const double p0 = z.p[f][0], k0 = z.k[f][0];
+      const double p0 = z.p[f][0], rk = z.rk[f];
 #pragma unroll
       for (int k = 1; k < 4; ++k) {
         pb[f][k] = z.xi * kb[f][k];
         xib += kb[f][k] * z.p[f][k];
       }
-      xib += kb[f][0] * z.xi * p0 * p0 / k0;
-      pb[f][0] = kb[f][0] * z.xi * z.xi * p0 / k0;
-      fxi += z.xi * p0 * p0 / k0;
+      xib += kb[f][0] * z.xi * p0 * p0 * rk;
+      pb[f][0] = kb[f][0] * z.xi * z.xi * p0 * rk;
+      fxi += z.xi * p0 * p0 * rk;
     }
 #pragma unroll
-    for (int f = 0; f < NF; ++f) pb[f][0] += xib * (-(z.xi * z.xi * z.p[f][0] / z.k[f][0]) / fxi);
+    for (int f = 0; f < NF; ++f) pb[f][0] += -(xib / fxi) * (z.xi * z.xi * z.p[f][0] * z.rk[f]);
   } else {
 #pragma unroll
     for (int f = 0; f < NF; ++f)
@@ -178,17 +192,17 @@ __device__ __forceinline__ void rambo_adjoint(const double* r, double ecm, const
     }
   }
   gb += -ab * z.a * z.a;
-  double Mb = -xb * z.x / z.M - gb * z.g / z.M;
+  double Mb = -(xb * z.x + gb * z.g) * z.rM;
   double Qb[4];
-  Qb[0] = gb / z.M;
+  Qb[0] = gb * z.rM;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    Qb[k + 1] = -bb[k] / z.M;
-    Mb += -bb[k] * z.b[k] / z.M;
+    Qb[k + 1] = -bb[k] * z.rM;
+    Mb += -bb[k] * z.b[k] * z.rM;
   }
-  Qb[0] += Mb * z.Q[0] / z.M;
+  Qb[0] += Mb * z.g;
 #pragma unroll
-  for (int k = 1; k < 4; ++k) Qb[k] += -Mb * z.Q[k] / z.M;
+  for (int k = 1; k < 4; ++k) Qb[k] += Mb * z.b[k - 1];
 #pragma unroll
   for (int f = 0; f < NF; ++f) {
 #pragma unroll
@@ -200,8 +214,9 @@ __device__ __forceinline__ void rambo_adjoint(const double* r, double ecm, const
     const double phib = -qb[f][1] * e * s * sp + qb[f][2] * e * s * cp;
     rb[4 * f + 0] = 2.0 * cb;
     rb[4 * f + 1] = kTwoPi * phib;
-    rb[4 * f + 2] = -eb / r[4 * f + 2];
-    rb[4 * f + 3] = -eb / r[4 * f + 3];
+    const double er = -eb / (r[4 * f + 2] * r[4 * f + 3]);
+    rb[4 * f + 2] = er * r[4 * f + 3];
+    rb[4 * f + 3] = er * r[4 * f + 2];
   }
 }
 
