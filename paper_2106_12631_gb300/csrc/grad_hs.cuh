@@ -31,20 +31,20 @@
 
 namespace mg {
 
-// events per CTA: small FP32 CTAs, several per SM, overlap each other's
-// latency-bound phases; the FP64 kernel prefers larger ones (measured)
-#ifndef MG_HSG_EV
-#define MG_HSG_EV 2
+// threads per CTA, one per (event, helicity): small FP32 CTAs, several per SM,
+// overlap each other's latency-bound phases; the FP64 kernel prefers larger ones
+// (measured)
+#ifndef MG_HSG_THREADS
+#define MG_HSG_THREADS 64
 #endif
-#ifndef MG_HSG_EV64
-#define MG_HSG_EV64 8
+#ifndef MG_HSG_THREADS64
+#define MG_HSG_THREADS64 128
 #endif
 
 template <class P, class R>
 struct HsGradCfg {
-  static constexpr int EVW = sizeof(R) == 4 ? MG_HSG_EV : MG_HSG_EV64;
-  // at least one whole warp (the adjoint's warp sums shuffle across all 32 lanes)
-  static constexpr int NT = EVW * P::NHEL >= 32 ? EVW * P::NHEL : 32;
+  // whole warps (the adjoint's warp sums shuffle across all 32 lanes)
+  static constexpr int NT = sizeof(R) == 4 ? MG_HSG_THREADS : MG_HSG_THREADS64;
   static constexpr int EVMIN = NT / P::NHEL;
   static constexpr int EVCAP = EVMIN;
   static_assert(P::HS_NXCHUNK == 1, "the adjoint keeps every amputated current: one chunk");
@@ -379,49 +379,53 @@ __global__ void __launch_bounds__(HsGradCfg<P, R>::NT) sigmakin_hs_grad_kernel(G
   __syncthreads();
   // 4. amputated currents, then the current levels in reverse; the items of
   //    event ex run on warp ex % (NT / 32), so each event's adjoint slots have
-  //    one writing warp (plain adds, rounds of 32 items separated by __syncwarp)
+  //    one writing warp (plain adds, rounds of 32 items separated by __syncwarp);
+  //    a warp with several events takes their items in one sequence, so that
+  //    its rounds are full (12 items per phase and event for gg -> t t~; lanes of
+  //    several events never share an address)
   const int warp = tid >> 5, lane = tid & 31;
   constexpr int NW = NT / 32;
   R* const wstage = reinterpret_cast<R*>(smem + L::o_stage) + warp * 32 * 8;  // the warp's group-sum staging
+  // work index t of a warp: item t - k ni of its event k
+  const int nwe = (nev - warp + NW - 1) / NW;  // events of this warp
   {
-    const int i0 = P::hs_xitem(0), ni = P::hs_xitem(1) - i0;
-    for (int ex = warp; ex < nev; ex += NW) {
-      for (int r0 = 0; r0 < ni; r0 += 32) {
-        if (r0 + lane < ni) {
-          const HsItem it = items[i0 + r0 + lane];
-          hs_xitem_adj<P, R>(it, Slots<R, P::HS_NSLOT>{curs + ex * CUR_EV},
-                             Slots<R, P::HS_NSLOT>{cursb + ex * CUR_EV}, Slots<R, P::HS_XCAP>{xbufsb + ex * X_EV},
-                             Kall + ex * P::NMOM * 4, Kball + ex * P::NMOM * 4, cp, wstage);
-        }
-        __syncwarp();
+    constexpr int i0 = P::hs_level(P::HS_NLEVEL), ni = P::HS_NITEM - i0;
+    for (int r0 = 0; r0 < ni * nwe; r0 += 32) {
+      const int t = r0 + lane, k = t / ni, ex = warp + NW * k;
+      if (k < nwe) {
+        const HsItem it = items[i0 + t - k * ni];
+        hs_xitem_adj<P, R>(it, Slots<R, P::HS_NSLOT>{curs + ex * CUR_EV},
+                           Slots<R, P::HS_NSLOT>{cursb + ex * CUR_EV}, Slots<R, P::HS_XCAP>{xbufsb + ex * X_EV},
+                           Kall + ex * P::NMOM * 4, Kball + ex * P::NMOM * 4, cp, wstage);
       }
+      __syncwarp();
     }
   }
   __syncthreads();
-#pragma unroll
-  for (int l = P::HS_NLEVEL - 1; l >= 1; --l) {
-    const int i0 = P::hs_level(l), ni = P::hs_level(l + 1) - i0;
-    for (int ex = warp; ex < nev; ex += NW) {
-      for (int r0 = 0; r0 < ni; r0 += 32) {
-        if (r0 + lane < ni) {
-          const HsItem it = items[i0 + r0 + lane];
-          hs_item_adj<P, R>(it, Slots<R, P::HS_NSLOT>{curs + ex * CUR_EV}, Slots<R, P::HS_NSLOT>{cursb + ex * CUR_EV},
-                            Kall + ex * P::NMOM * 4, Kball + ex * P::NMOM * 4, prall + ex * P::NPROP,
-                            prball + ex * P::NPROP, cp, wstage);
-        }
-        __syncwarp();
+  static_for<1, P::HS_NLEVEL>([&](auto Lv) {
+    constexpr int l = P::HS_NLEVEL - decltype(Lv)::value;
+    constexpr int i0 = P::hs_level(l), ni = P::hs_level(l + 1) - i0;
+    for (int r0 = 0; r0 < ni * nwe; r0 += 32) {
+      const int t = r0 + lane, k = t / ni, ex = warp + NW * k;
+      if (k < nwe) {
+        const HsItem it = items[i0 + t - k * ni];
+        hs_item_adj<P, R>(it, Slots<R, P::HS_NSLOT>{curs + ex * CUR_EV}, Slots<R, P::HS_NSLOT>{cursb + ex * CUR_EV},
+                          Kall + ex * P::NMOM * 4, Kball + ex * P::NMOM * 4, prall + ex * P::NPROP,
+                          prball + ex * P::NPROP, cp, wstage);
       }
+      __syncwarp();
     }
     __syncthreads();
-  }
+  });
   // 5. external wavefunctions -> momenta; propagators -> momentum table
   {
-    constexpr int NEXT = P::hs_level(1);
+    // the beams (legs 0 and 1, items 0 to 3) are constant
+    constexpr int NEXT = P::hs_level(1) - 4;
     const int2* prop_tab = reinterpret_cast<const int2*>(smem + L::o_proptab);
     for (int t = tid; t < nev * (NEXT + P::NPROP); t += NT) {
       if (t < nev * NEXT) {
         const int ex = t / NEXT;
-        const HsItem it = items[t - ex * NEXT];
+        const HsItem it = items[4 + t - ex * NEXT];
         const W4<R> ob = Slots<R, P::HS_NSLOT>{cursb + ex * CUR_EV}[it.out];
         R pk[4], pbk[4] = {R(0), R(0), R(0), R(0)};
 #pragma unroll
