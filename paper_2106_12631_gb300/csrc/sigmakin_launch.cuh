@@ -1,6 +1,8 @@
 // Launchers shared by the per-process translation units (one TU per process
 // so the four diagram programs compile in parallel).
 #pragma once
+#include <atomic>
+
 #include "launch.h"
 #include "sigmakin.cuh"
 #include "sigmakin_hs.cuh"
@@ -33,25 +35,29 @@ cudaError_t launch_sigmakin_hs_variant(const SigArgs& a, const Couplings<R>& cp,
   using H = typename L::H;
   constexpr int NT = L::NT;
   constexpr int kMaxDevices = 64;
-  static int resident[kMaxDevices];  // CTAs resident on the whole device; 0 until known
+  static std::atomic<int> resident[kMaxDevices];  // CTAs resident on the whole device; 0 until known
   const void* k = FUSED ? (const void*)sigmakin_hs_rambo_kernel<P, R, CS> : (const void*)sigmakin_hs_kernel<P, R, CS>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::bytes);
-  if (e != cudaSuccess) return e;
   grid = (a.nevt + H::EW - 1) / H::EW;  // one unit per CTA at least
+  auto launch = [&](int cap) {
+    const unsigned g = (unsigned)(grid > cap ? cap : grid);
+    if constexpr (FUSED) sigmakin_hs_rambo_kernel<P, R, CS><<<g, NT, L::bytes, s>>>(a, cp, *ra);
+    else sigmakin_hs_kernel<P, R, CS><<<g, NT, L::bytes, s>>>(a, cp);
+    return cudaGetLastError();
+  };
   int dev = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  int cap = dev < kMaxDevices ? resident[dev] : 0;
-  if (cap == 0) {
-    int nsm = 0, per = 0;
-    if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, NT, L::bytes)) != cudaSuccess) return e;
-    cap = nsm * (per > H::CTAS ? per : H::CTAS);
-    if (dev < kMaxDevices) resident[dev] = cap;
-  }
-  if (grid > cap) grid = cap;
-  if constexpr (FUSED) sigmakin_hs_rambo_kernel<P, R, CS><<<(unsigned)grid, NT, L::bytes, s>>>(a, cp, *ra);
-  else sigmakin_hs_kernel<P, R, CS><<<(unsigned)grid, NT, L::bytes, s>>>(a, cp);
-  return cudaGetLastError();
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  int cap = dev < kMaxDevices ? resident[dev].load(std::memory_order_relaxed) : 0;
+  // the shared-memory attribute is set with the first launch on a device, and
+  // again if a launch is refused for want of it (the device was reset)
+  if (cap != 0 && (e = launch(cap)) != cudaErrorInvalidValue) return e;
+  if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::bytes)) != cudaSuccess) return e;
+  int nsm = 0, per = 0;
+  if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, NT, L::bytes)) != cudaSuccess) return e;
+  cap = nsm * (per > H::CTAS ? per : H::CTAS);
+  if (dev < kMaxDevices) resident[dev].store(cap, std::memory_order_relaxed);
+  return launch(cap);
 }
 
 // mode 0 FP64; 1 mixed, colour sum on CUDA cores below 48 colour flows and on

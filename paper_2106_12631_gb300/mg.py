@@ -48,6 +48,8 @@ class Params(ctypes.Structure):
 def lib():
     """Load libmg.so (building it in-tree first if it is missing or stale)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             path = _build.build()
@@ -101,6 +103,9 @@ def _stream(stream) -> int:
 
 
 def _dev(t: torch.Tensor, dtype, name: str, shape=None):
+    if (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype is dtype and t.is_contiguous()
+            and (shape is None or t.shape == shape)):
+        return t.data_ptr()
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise ValueError("%s must be a CUDA tensor" % name)
     if t.dtype != dtype:
@@ -130,6 +135,19 @@ def process_info(proc) -> dict:
             "namplitudes": info.namplitudes, "nrand": info.nrand, "mass": list(info.mass)[: info.npar]}
 
 
+_dims_of = {}
+
+
+def _dims(p: int):
+    """(npar, nhel) of a process id: constants of the library, asked for once
+    (small batches are bound by the host's work per call)."""
+    d = _dims_of.get(p)
+    if d is None:
+        info = process_info(p)
+        d = _dims_of[p] = (info["npar"], info["nhel"])
+    return d
+
+
 def get_params() -> dict:
     p = Params()
     _check(lib().mg_get_params(ctypes.byref(p)), "mg_get_params")
@@ -146,7 +164,7 @@ def rambo(proc, rnd: torch.Tensor, ecm: float, mom=None, wgt=None, stream=None):
     """rnd (nrows, nevt) float64 CUDA -> (mom (npar, 4, nevt), wgt (nevt,))."""
     p = _proc(proc)
     nrows, nevt = rnd.shape
-    npar = process_info(p)["npar"]
+    npar = _dims(p)[0]
     if mom is None:
         mom = torch.empty((npar, 4, nevt), dtype=torch.float64, device=rnd.device)
     if wgt is None:
@@ -161,7 +179,7 @@ def rambo_seeded(proc, nevt: int, ecm: float, seed: int, first_event: int = 0, m
                  stream=None):
     """RAMBO with the uniforms drawn on the device (counter-based, as inputs.uniforms)."""
     p = _proc(proc)
-    npar = process_info(p)["npar"]
+    npar = _dims(p)[0]
     dev = device if device is not None else (mom.device if mom is not None else torch.device("cuda"))
     if mom is None:
         mom = torch.empty((npar, 4, nevt), dtype=torch.float64, device=dev)
@@ -215,7 +233,7 @@ def matrix_elements_batch(proc, mom_aos: torch.Tensor, mask: torch.Tensor, mode=
     """mom_aos (nevt, npar, 4) float64 CUDA -> me (nevt,), or (me, hel, col) when hel_rnd or
     col_rnd (nevt,) uniforms are given (a choice not asked for is None)."""
     p = _proc(proc)
-    nevt, npar = mom_aos.shape[0], process_info(p)["npar"]
+    nevt, npar = mom_aos.shape[0], _dims(p)[0]
     if me is None:
         me = torch.empty((nevt,), dtype=torch.float64, device=mom_aos.device)
     if hel_rnd is not None and hel is None:
@@ -229,7 +247,7 @@ def matrix_elements_batch(proc, mom_aos: torch.Tensor, mask: torch.Tensor, mode=
     opt = lambda t, dt, name: _dev(t, dt, name, (nevt,)) if t is not None else None
     _check(lib().mg_matrix_elements_batch(
         p, nevt, _dev(mom_aos, torch.float64, "mom_aos", (nevt, npar, 4)),
-        _dev(mask, torch.int32, "mask", (process_info(p)["nhel"],)), m,
+        _dev(mask, torch.int32, "mask", (_dims(p)[1],)), m,
         opt(hel_rnd, torch.float64, "hel_rnd"), opt(col_rnd, torch.float64, "col_rnd"),
         _dev(me, torch.float64, "me", (nevt,)), opt(hel, torch.int32, "hel"), opt(col, torch.int32, "col"),
         *_ws(workspace), _stream(stream)),
@@ -255,9 +273,9 @@ def sigmakin_split(proc, mom: torch.Tensor, mask: torch.Tensor, mode="mixed_simt
     if workspace is None:
         nb = max(sigmakin_split_workspace_bytes(p, m, nevt), 16)
         workspace = torch.empty(((nb + 7) // 8,), dtype=torch.float64, device=mom.device)
-    info = process_info(p)
-    _check(lib().mg_sigmakin_split(p, nevt, _dev(mom, torch.float64, "mom", (info["npar"], 4, nevt)),
-                                   _dev(mask, torch.int32, "mask", (info["nhel"],)), m,
+    npar, nhel = _dims(p)
+    _check(lib().mg_sigmakin_split(p, nevt, _dev(mom, torch.float64, "mom", (npar, 4, nevt)),
+                                   _dev(mask, torch.int32, "mask", (nhel,)), m,
                                    _dev(me, torch.float64, "me", (nevt,)), *_ws(workspace), _stream(stream)),
            "mg_sigmakin_split")
     return me
@@ -265,25 +283,25 @@ def sigmakin_split(proc, mom: torch.Tensor, mask: torch.Tensor, mode="mixed_simt
 
 def filter_helicities(proc, mom: torch.Tensor, mask=None, stream=None) -> torch.Tensor:
     p = _proc(proc)
-    info = process_info(p)
+    npar, nhel = _dims(p)
     if mask is None:
-        mask = torch.empty((info["nhel"],), dtype=torch.int32, device=mom.device)
+        mask = torch.empty((nhel,), dtype=torch.int32, device=mom.device)
     nevt = mom.shape[2]
-    _check(lib().mg_filter_helicities(p, nevt, _dev(mom, torch.float64, "mom", (info["npar"], 4, nevt)),
-                                      _dev(mask, torch.int32, "mask", (info["nhel"],)), _stream(stream)),
+    _check(lib().mg_filter_helicities(p, nevt, _dev(mom, torch.float64, "mom", (npar, 4, nevt)),
+                                      _dev(mask, torch.int32, "mask", (nhel,)), _stream(stream)),
            "mg_filter_helicities")
     return mask
 
 
 def sigmakin(proc, mom: torch.Tensor, mask: torch.Tensor, mode="mixed", me=None, stream=None) -> torch.Tensor:
     p = _proc(proc)
-    info = process_info(p)
+    npar, nhel = _dims(p)
     nevt = mom.shape[2]
     m = MODES[mode] if isinstance(mode, str) else int(mode)
     if me is None:
         me = torch.empty((nevt,), dtype=torch.float64, device=mom.device)
-    _check(lib().mg_sigmakin(p, nevt, _dev(mom, torch.float64, "mom", (info["npar"], 4, nevt)),
-                             _dev(mask, torch.int32, "mask", (info["nhel"],)),
+    _check(lib().mg_sigmakin(p, nevt, _dev(mom, torch.float64, "mom", (npar, 4, nevt)),
+                             _dev(mask, torch.int32, "mask", (nhel,)),
                              _dev(me, torch.float64, "me", (nevt,)), m, _stream(stream)), "mg_sigmakin")
     return me
 
@@ -305,7 +323,7 @@ def sigmakin_rambo(proc, rnd: torch.Tensor, ecm: float, mask: torch.Tensor, mode
     m = MODES[mode] if isinstance(mode, str) else int(mode)
     me, wgt = _me_wgt(nevt, rnd.device, me, wgt)
     _check(lib().mg_sigmakin_rambo(p, nevt, float(ecm), _dev(rnd, torch.float64, "rnd"), nrows,
-                                   _dev(mask, torch.int32, "mask", (process_info(p)["nhel"],)), m,
+                                   _dev(mask, torch.int32, "mask", (_dims(p)[1],)), m,
                                    _dev(me, torch.float64, "me", (nevt,)), _dev(wgt, torch.float64, "wgt", (nevt,)),
                                    _stream(stream)), "mg_sigmakin_rambo")
     return me, wgt
@@ -319,7 +337,7 @@ def sigmakin_seeded(proc, nevt: int, ecm: float, seed: int, mask: torch.Tensor, 
     m = MODES[mode] if isinstance(mode, str) else int(mode)
     me, wgt = _me_wgt(nevt, mask.device, me, wgt)
     _check(lib().mg_sigmakin_seeded(p, nevt, float(ecm), seed & 0xFFFFFFFFFFFFFFFF, first_event,
-                                    _dev(mask, torch.int32, "mask", (process_info(p)["nhel"],)), m,
+                                    _dev(mask, torch.int32, "mask", (_dims(p)[1],)), m,
                                     _dev(me, torch.float64, "me", (nevt,)), _dev(wgt, torch.float64, "wgt", (nevt,)),
                                     _stream(stream)), "mg_sigmakin_seeded")
     return me, wgt
@@ -337,7 +355,7 @@ def sigmakin_grad(proc, rnd: torch.Tensor, ecm: float, mask: torch.Tensor, mode=
         me = torch.empty((nevt,), dtype=torch.float64, device=rnd.device)
     g = _dev(gout, torch.float64, "gout", (nevt,)) if gout is not None else None
     _check(lib().mg_sigmakin_grad(p, nevt, float(ecm), _dev(rnd, torch.float64, "rnd"), nrows,
-                                  _dev(mask, torch.int32, "mask", (process_info(p)["nhel"],)), g,
+                                  _dev(mask, torch.int32, "mask", (_dims(p)[1],)), g,
                                   _dev(grad, torch.float64, "grad", (nrows, nevt)),
                                   _dev(me, torch.float64, "me", (nevt,)), m, _stream(stream)), "mg_sigmakin_grad")
     return grad, me
@@ -424,7 +442,7 @@ def pipeline_host(proc, rnd_host: torch.Tensor, ecm: float, mask: torch.Tensor, 
     if workspace is None:
         workspace = torch.empty(((nb + 7) // 8,), dtype=torch.float64, device=mask.device)
     _check(lib().mg_pipeline_host(p, nevt, float(ecm), rnd_host.data_ptr(), nrows,
-                                  _dev(mask, torch.int32, "mask", (process_info(p)["nhel"],)), m,
+                                  _dev(mask, torch.int32, "mask", (_dims(p)[1],)), m,
                                   me_host.data_ptr(),
                                   wgt_host.data_ptr() if wgt_host is not None else None,
                                   sums_host.data_ptr() if sums_host is not None else None,
