@@ -91,7 +91,7 @@ struct HsLayout {
   static constexpr size_t o_good = align_up(o_md + 16 * P::NMOM, 16);
   static constexpr size_t o_misc = align_up(o_good + 4 * P::NHEL, 16);
   // mixed mode: {m^2 hi, m^2 lo, m w, 0} of the top and of the Z
-  static constexpr size_t o_mconst = align_up(o_misc + 32, 16);
+  static constexpr size_t o_mconst = align_up(o_misc + 48, 16);
   static constexpr size_t o_p = align_up(o_mconst + 32, 16);
   // the next group's momenta (FP64), copied asynchronously while this group runs
   static constexpr size_t o_ps = align_up(o_p + 8 * EW * EVCAP * P::NPAR * 4, 16);
@@ -678,8 +678,9 @@ __device__ __forceinline__ void hs_tables(unsigned char* smem, const PhysParams&
   static_assert(NEXT == 2 * NPAR, "level 0: two helicities per leg");
   constexpr int NE = NPAR;
   for (int t = threadIdx.x; t < nep * (NM + NE); t += L::NT) {
-    const bool mom = t < nep * NM;
-    const int t2 = mom ? t : t - nep * NM, e = t2 / (mom ? NM : NE), j = t2 - e * (mom ? NM : NE);
+    // the wavefunctions, the longer work, first
+    const bool mom = t >= nep * NE;
+    const int t2 = mom ? t - nep * NE : t, e = t2 / (mom ? NM : NE), j = t2 - e * (mom ? NM : NE);
     const int u = e / EW, lane = e - u * EW, es = EW == 1 ? e : min(e, nev - 1);
     if (mom) {
       const int4 d = md[j];
@@ -1048,6 +1049,7 @@ __device__ __forceinline__ void hs_sigmakin_body(const SigArgs& a, const Couplin
     misc[2] = ngrp;
     misc[6] = ng;
     misc[7] = ev;
+    *reinterpret_cast<double*>(misc + 8) = hs_norm<P>(a.pp);
   }
   if (ng == 0) {
     for (int g = blockIdx.x; g < ngrp; g += gridDim.x) {
@@ -1202,9 +1204,11 @@ __device__ __forceinline__ void hs_sigmakin_body(const SigArgs& a, const Couplin
     // fixed-order FP64 helicity sum per event: eight lanes per event each add
     // every eighth helicity in order, then a butterfly over the eight lanes
     // (addition commutes, so every lane ends with the same bits); sm2 is next
-    // written at the end of the next group, after several barriers
+    // written at the end of the next group, after several barriers; the last warps
+    // take it, the first ones begin with the next group's wavefunctions
     for (int b = 0; b < nev * 8; b += NT) {
-      const int t = b + tid, eh = t >> 3, q = t & 7;
+      const int t = b + (NT - 1 - tid), eh = t >> 3, q = t & 7;
+      if ((t & ~31) >= nev * 8) continue;  // whole warps without an event
       double sum = 0.0;
       if (t < nev * 8) {
 #pragma unroll
@@ -1214,7 +1218,7 @@ __device__ __forceinline__ void hs_sigmakin_body(const SigArgs& a, const Couplin
       sum += __shfl_xor_sync(0xffffffffu, sum, 1);
       sum += __shfl_xor_sync(0xffffffffu, sum, 2);
       sum += __shfl_xor_sync(0xffffffffu, sum, 4);
-      if (t < nev * 8 && q == 0) a.me[e0 + eh] = sum * hs_norm<P>(a.pp);
+      if (t < nev * 8 && q == 0) a.me[e0 + eh] = sum * *reinterpret_cast<const double*>(misc + 8);
     }
     // 5. helicity and colour-flow choices (batched entry point), once every
     //    group of the CTA is done with the union region; the closing barrier

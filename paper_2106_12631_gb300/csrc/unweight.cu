@@ -7,8 +7,11 @@
 // counter-based generator (seed, first_event + i, row 63); event i is kept
 // iff u_i * max x < x_i (so x_i <= 0 is never kept); the kept indices are
 // written in increasing order (stable compaction from a block scan).
-// Launches: per-block maxima, their maximum, per-block counts, an exclusive
-// scan of the counts (also the total), and the scatter of the indices.
+// Launches: per-block maxima, per-block counts, and the scatter of the indices;
+// up to kUwDirect blocks every block forms the maximum of the block maxima, and
+// in the scatter the sum of the counts before it, by itself (16384 events: 27 us
+// in five launches, of which the scan 8.5 us).  Beyond, the maximum and an
+// exclusive scan of the counts (also the total) are launches of their own.
 #include <cstdint>
 
 #include "launch.h"
@@ -20,6 +23,7 @@ constexpr int kUwThreads = 256;
 constexpr int kUwPerThread = 4;
 constexpr int kUwBlock = kUwThreads * kUwPerThread;  // events per block
 constexpr int kUwScanThreads = 1024;
+constexpr int kUwDirect = 1024;  // blocks (2^20 events)
 
 int64_t unweight_blocks(int64_t n) { return (n + kUwBlock - 1) / kUwBlock; }
 
@@ -65,6 +69,34 @@ __global__ void __launch_bounds__(kUwScanThreads) uw_max_final(int64_t nblk, con
   }
 }
 
+// max(part[0 .. n)) and sum(v[0 .. n)) over a CTA of kUwThreads threads, in every thread
+__device__ __forceinline__ double uw_max_of(const double* __restrict__ part, int n) {
+  __shared__ double red[kUwThreads / 32];
+  double m = -INFINITY;
+  for (int b = threadIdx.x; b < n; b += kUwThreads) m = fmax(m, part[b]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  m = red[0];
+#pragma unroll
+  for (int k = 1; k < kUwThreads / 32; ++k) m = fmax(m, red[k]);
+  return m;
+}
+__device__ __forceinline__ int64_t uw_sum_of(const int64_t* __restrict__ v, int n) {
+  __shared__ long long red[kUwThreads / 32];
+  long long s = 0;
+  for (int b = threadIdx.x; b < n; b += kUwThreads) s += v[b];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  s = 0;
+#pragma unroll
+  for (int k = 0; k < kUwThreads / 32; ++k) s += red[k];
+  return s;
+}
+
 // kept events among a thread's kUwPerThread consecutive events, as a bit mask
 __device__ __forceinline__ unsigned uw_keep(int64_t n, const double* __restrict__ me, const double* __restrict__ w,
                                             uint64_t key, int64_t first_event, double xmax, int64_t base) {
@@ -104,12 +136,15 @@ __device__ __forceinline__ int uw_block_scan(int v, int* tot) {
   return before;
 }
 
+// DIRECT: xmax points to the block maxima, and the offsets to the block counts
+template <bool DIRECT>
 __global__ void __launch_bounds__(kUwThreads) uw_count_blocks(int64_t n, const double* __restrict__ me,
                                                               const double* __restrict__ w, uint64_t key,
                                                               int64_t first_event, const double* xmax,
                                                               int64_t* counts) {
   const int64_t base = (int64_t)blockIdx.x * kUwBlock + (int64_t)threadIdx.x * kUwPerThread;
-  const int c = __popc(uw_keep(n, me, w, key, first_event, *xmax, base));
+  const double xm = DIRECT ? uw_max_of(xmax, (int)gridDim.x) : *xmax;
+  const int c = __popc(uw_keep(n, me, w, key, first_event, xm, base));
   int tot;
   uw_block_scan(c, &tot);
   if (threadIdx.x == 0) counts[blockIdx.x] = tot;
@@ -142,14 +177,18 @@ __global__ void __launch_bounds__(kUwScanThreads) uw_scan_counts(int64_t nblk, i
   }
 }
 
+template <bool DIRECT>
 __global__ void __launch_bounds__(kUwThreads) uw_write(int64_t n, const double* __restrict__ me,
                                                        const double* __restrict__ w, uint64_t key,
                                                        int64_t first_event, const double* xmax,
-                                                       const int64_t* offsets, int64_t* idx) {
+                                                       const int64_t* offsets, int64_t* idx, int64_t* count) {
   const int64_t base = (int64_t)blockIdx.x * kUwBlock + (int64_t)threadIdx.x * kUwPerThread;
-  const unsigned bits = uw_keep(n, me, w, key, first_event, *xmax, base);
+  const double xm = DIRECT ? uw_max_of(xmax, (int)gridDim.x) : *xmax;
+  const unsigned bits = uw_keep(n, me, w, key, first_event, xm, base);
   int tot;
-  int64_t pos = offsets[blockIdx.x] + uw_block_scan(__popc(bits), &tot);
+  const int64_t before = DIRECT ? uw_sum_of(offsets, (int)blockIdx.x) : offsets[blockIdx.x];
+  int64_t pos = before + uw_block_scan(__popc(bits), &tot);
+  if (DIRECT && threadIdx.x == 0 && blockIdx.x == gridDim.x - 1) *count = before + tot;
 #pragma unroll
   for (int j = 0; j < kUwPerThread; ++j)
     if (bits >> j & 1u) idx[pos++] = base + j;
@@ -163,10 +202,15 @@ cudaError_t launch_unweight(int64_t n, const double* me, const double* w, uint64
   int64_t* counts = reinterpret_cast<int64_t*>(scratch + 1 + nblk);
   const uint64_t key = sm64_mix(seed);
   uw_max_blocks<<<(unsigned)nblk, kUwThreads, 0, s>>>(n, me, w, part);
+  if (nblk <= kUwDirect) {
+    uw_count_blocks<true><<<(unsigned)nblk, kUwThreads, 0, s>>>(n, me, w, key, first_event, part, counts);
+    uw_write<true><<<(unsigned)nblk, kUwThreads, 0, s>>>(n, me, w, key, first_event, part, counts, idx, count);
+    return cudaGetLastError();
+  }
   uw_max_final<<<1, kUwScanThreads, 0, s>>>(nblk, part, xmax);
-  uw_count_blocks<<<(unsigned)nblk, kUwThreads, 0, s>>>(n, me, w, key, first_event, xmax, counts);
+  uw_count_blocks<false><<<(unsigned)nblk, kUwThreads, 0, s>>>(n, me, w, key, first_event, xmax, counts);
   uw_scan_counts<<<1, kUwScanThreads, 0, s>>>(nblk, counts, count);
-  uw_write<<<(unsigned)nblk, kUwThreads, 0, s>>>(n, me, w, key, first_event, xmax, counts, idx);
+  uw_write<false><<<(unsigned)nblk, kUwThreads, 0, s>>>(n, me, w, key, first_event, xmax, counts, idx, nullptr);
   return cudaGetLastError();
 }
 

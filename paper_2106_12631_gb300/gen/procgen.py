@@ -1893,6 +1893,14 @@ class OrderedProgram:
             for g in gl:
                 if g not in (a, b):
                     self._dot(G(g), G(a, b), (g, a, b))
+        # A warp takes 8 items of 4 units, a CTA of 8 warps 64 items per round: with the
+        # three-gluon items (32, five times a vector vertex) on its first four warps, the
+        # other four take items of the same length in sum (multiply-adds per item: three
+        # gluons 412, R(ab) 240, C(ab) 136, vector vertex 124, pairing 84, W 32, product 16)
+        of = lambda t: [it for it in X if it[0] == t]
+        r2, c2 = of(self.T_ROW2), of(self.T_COL2)
+        X[:] = (of(self.T_G3) + r2[:32] + c2[:32] + r2[32:] + c2[32:] + of(self.T_VB) + of(self.T_P) + of(self.T_W)
+                + of(self.T_DOT))
 
     # ---- emission -----------------------------------------------------------------------
     def emit_tables(self, pid: int) -> list:
