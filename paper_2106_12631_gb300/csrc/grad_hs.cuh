@@ -176,6 +176,20 @@ __device__ __forceinline__ void own_slot_add(const Slots<R, N>& s, int i, const 
   }
 }
 
+// Sum over the four aligned lanes of a current's consecutive variants (every
+// current has a multiple of four of them, and every phase's items and rounds
+// start at multiples of four lanes): these all add into one momentum and one
+// propagator adjoint, so the group sums that follow have a quarter of the
+// members (their leaders read them one by one).
+template <int NV, class R>
+__device__ __forceinline__ void quad_sum(R* v) {
+  const unsigned act = __activemask();
+#pragma unroll
+  for (int i = 0; i < NV; ++i) v[i] += __shfl_xor_sync(act, v[i], 1);
+#pragma unroll
+  for (int i = 0; i < NV; ++i) v[i] += __shfl_xor_sync(act, v[i], 2);
+}
+
 // adjoint of one current variant (levels >= 1)
 template <class P, class R>
 __device__ __forceinline__ void hs_item_adj(const HsItem& it, const Slots<R, P::HS_NSLOT>& cur,
@@ -214,9 +228,15 @@ __device__ __forceinline__ void hs_item_adj(const HsItem& it, const Slots<R, P::
 #pragma unroll
   for (int k = 0; k < 3; ++k)
     if (k < nin) own_slot_add(curb, it.in[k], b[k], stage);
-  if (nk >= 1) own_add4(Kb + 4 * it.k0, kb0, stage);
-  if (nk >= 2) own_add4(Kb + 4 * it.k1, kb1, stage);
-  own_addc(prb + it.prop, pb, stage);
+  quad_sum<4>(kb0);
+  quad_sum<4>(kb1);
+  quad_sum<1>(&pb.re);
+  quad_sum<1>(&pb.im);
+  if ((threadIdx.x & 3) == 0) {
+    if (nk >= 1) own_add4(Kb + 4 * it.k0, kb0, stage);
+    if (nk >= 2) own_add4(Kb + 4 * it.k1, kb1, stage);
+    own_addc(prb + it.prop, pb, stage);
+  }
 }
 
 // adjoint of one amputated-current variant
@@ -248,7 +268,9 @@ __device__ __forceinline__ void hs_xitem_adj(const HsItem& it, const Slots<R, P:
 #pragma unroll
   for (int k = 0; k < 3; ++k)
     if (k < nin) own_slot_add(curb, it.in[k], b[k], stage);
-  if (mom) {
+  quad_sum<4>(kb0);
+  quad_sum<4>(kb1);
+  if (mom && (threadIdx.x & 3) == 0) {
     own_add4(Kb + 4 * it.k0, kb0, stage);
     own_add4(Kb + 4 * it.k1, kb1, stage);
   }
@@ -390,6 +412,7 @@ __global__ void __launch_bounds__(HsGradCfg<P, R>::NT) sigmakin_hs_grad_kernel(G
   const int nwe = (nev - warp + NW - 1) / NW;  // events of this warp
   {
     constexpr int i0 = P::hs_level(P::HS_NLEVEL), ni = P::HS_NITEM - i0;
+    static_assert(ni % 4 == 0, "whole quads of variants");
     for (int r0 = 0; r0 < ni * nwe; r0 += 32) {
       const int t = r0 + lane, k = t / ni, ex = warp + NW * k;
       if (k < nwe) {
@@ -405,6 +428,7 @@ __global__ void __launch_bounds__(HsGradCfg<P, R>::NT) sigmakin_hs_grad_kernel(G
   static_for<1, P::HS_NLEVEL>([&](auto Lv) {
     constexpr int l = P::HS_NLEVEL - decltype(Lv)::value;
     constexpr int i0 = P::hs_level(l), ni = P::hs_level(l + 1) - i0;
+    static_assert(ni % 4 == 0, "whole quads of variants");
     for (int r0 = 0; r0 < ni * nwe; r0 += 32) {
       const int t = r0 + lane, k = t / ni, ex = warp + NW * k;
       if (k < nwe) {
