@@ -5,20 +5,31 @@
 //   * an off-shell current over legs S depends only on the helicities of S,
 //     so each current is computed once per event for each of its 2^|S|
 //     helicity variants (not once per event helicity), into shared memory;
-//   * every diagram's amplitude is formed at a vertex chosen by the generator,
-//     with one operand Y left out: A = sum_i X_i Y_i, where the amputated
-//     current X of the other operands is again shared across helicities;
-//   * currents and amputated currents are item tables walked by short loops
-//     (lanes take one item for each of the CTA's events); the contractions of
-//     a chunk's amplitudes are generated straight-line code.
-// CTA of NT threads = units (pairs of events in the mixed mode) x ngood helicities.  Phases:
-//   1. per-event momenta, momentum sums and FP64 propagator factors (as SIGMAKIN);
+//   * every diagram's amplitude is a contraction sum_i X_i Y_i of two such
+//     objects, so that a helicity pays only the contractions.  gg -> t t~ g and
+//     gg -> t t~ g g run the ordered program (gen/procgen.py): colour-ordered
+//     currents summed over their diagrams before they are contracted, 12 and 55
+//     contractions per helicity for 18 and 159 amplitude terms; the smaller
+//     processes contract diagram by diagram;
+//   * currents and operands are item tables walked by short loops (lanes take
+//     one item for each of the CTA's units); the contractions are generated
+//     straight-line code.
+// The mixed mode takes pairs of events: a lane value is an f2, one event per
+// half, and every FP32 operation one paired instruction (mg_types.cuh).
+// CTA of NT threads = units (pairs of events in the mixed mode) x ngood
+// helicities.  Phases:
+//   1. per-event momenta, momentum sums and propagator factors, external
+//      wavefunctions;
 //   2. current variants, level by level (a level only reads earlier levels);
-//   3. per chunk of amputated currents: their variants (all threads), then one
-//      thread per (event, helicity) contracts the chunk's amplitudes and adds
-//      each into its colour flows J (registers);
+//   3. the contractions' operands (all threads), then one thread per (unit,
+//      helicity) contracts them into its colour flows J (registers);
 //   4. colour sum (CUDA cores, or tcgen05 as in sigmakin.cuh) and the
 //      fixed-order FP64 helicity sum.
+// What bounds it (gg -> t t~ g g mixed, 2^20 events): the bytes that the
+// contractions load from shared memory into registers (128 per clock and SM; 55 %
+// of the kernel's cycles) and the latency of dependent FMAs at 8 warps per SM
+// (FMA pipe 46 % busy): 10.3 ms, against 18.0 ms for the diagram-wise program on
+// single events.  In FP64 the FP64 pipe (90 % busy for gg -> t t~ g).
 #pragma once
 #include <type_traits>
 
@@ -383,41 +394,41 @@ __device__ __forceinline__ dfl dfl_split(double x) {
   const float h = (float)x;
   return {h, (float)(x - (double)h)};
 }
-// sum of signed terms t_k = hi_k + lo_k, k = 0..n-1
+// sum of signed terms t_k = hi_k + lo_k, k = 0..n-1 (V: float, or a pair of events)
+template <class V>
 struct DflSum {
-  float s, err;
-  __device__ __forceinline__ void first(float hi, float lo) { s = hi; err = lo; }
-  __device__ __forceinline__ void add(float hi, float lo) {
-    const dfl t = two_sum(s, hi);
-    s = t.hi;
-    err += t.lo + lo;
+  V s, err;
+  __device__ __forceinline__ void first(V hi, V lo) { s = hi; err = lo; }
+  __device__ __forceinline__ void add(V hi, V lo) {
+    const V t = s + hi, b = t - s;
+    err += ((s - (t - b)) + (hi - b)) + lo;
+    s = t;
   }
-  __device__ __forceinline__ float value() const { return s + err; }
+  __device__ __forceinline__ V value() const { return s + err; }
 };
 
 // Propagator factor from a double-float momentum: k^2 - m^2 summed error-free
 // from the exact squares of the components, then the reciprocal in FP32.
 // m2 = m^2 as double-float, mw = m w.
-__device__ __forceinline__ cx<float> propagator_dfl(const float2* k, int kind, dfl m2, float mw) {
-  DflSum d;
+template <class V>
+__device__ __forceinline__ cx<V> propagator_dfl(const DflSum<V>* k, int kind, dfl m2, float mw) {
+  DflSum<V> d;
 #pragma unroll
   for (int mu = 0; mu < 4; ++mu) {
-    const float h = k[mu].x, l = k[mu].y;
-    const float p = h * h;
-    float e = fmaf(h, h, -p);
-    e = fmaf(2.0f * h, l, e);
+    const V h = k[mu].s, p = h * h;
+    const V e = fmac(V(2.0f) * h, k[mu].err, fmac(h, h, -p));
     if (mu == 0) d.first(p, e);
     else d.add(-p, -e);
   }
-  float di = 0.0f;
+  V di(0.0f);
   if (kind == 1 || kind == 3) {
-    d.add(-m2.hi, -m2.lo);
-    di = mw;
+    d.add(V(-m2.hi), V(-m2.lo));
+    di = V(mw);
   }
-  const float r = d.value();
-  const float inv = 1.0f / (r * r + di * di);
-  const float ar = r * inv, ai = -di * inv;
-  return kind == 1 ? cx<float>(-ai, ar) : cx<float>(ai, -ar);
+  const V r = d.value();
+  const V inv = V(1.0f) / fmac(r, r, di * di);
+  const V ar = r * inv, ai = -di * inv;
+  return kind == 1 ? cx<V>(-ai, ar) : cx<V>(ai, -ar);
 }
 
 // Products, sums, reciprocals and reciprocal square roots of double-floats (the
@@ -566,15 +577,15 @@ __device__ __forceinline__ void ext_fermion_fp64(const double* p, double m, int 
 //                    the mixed mode {m^2 hi, m^2 lo, m w, 0} of the top and Z;
 //   hs_load_momenta  the CTA's momenta into shared memory: FP64, or in the
 //                    mixed mode each component split into a double-float pair;
-//   hs_tables        (after a barrier) one thread per (event, momentum-table
+//   hs_tables        (after a barrier) one thread per (unit, momentum-table
 //                    entry) sums the entry's signed external momenta — in FP64
 //                    (FP64 mode) or double-float (mixed mode), every leg in leg
 //                    order with coefficient +1, -1 or 0 (adding an exact zero
 //                    changes neither an FP64 sum nor a double-float pair), rounds
 //                    it to R for the currents and forms the propagator factor
 //                    of every line with that momentum from the unrounded sum;
-//                    one thread per (event, external leg variant) builds the
-//                    external wavefunction (level 0 of the current program).
+//                    one thread per (event, external leg) builds the external
+//                    wavefunctions of both helicities (level 0 of the program).
 
 // Descriptor of momentum-table entry j: {legs added, legs subtracted, first
 // propagator on that momentum, second} (-1: none).
@@ -611,19 +622,31 @@ __device__ __forceinline__ void hs_setup_words(unsigned char* smem, const PhysPa
   }
 }
 
-// p[e][leg][mu]: double, or float2 (hi, lo) in the mixed mode (same 8 bytes)
+// p[unit][leg][mu]: double, or in the mixed mode {hi, lo} of the unit's events
+// (EW high parts, then EW low parts); a last unit that is not full repeats its event
+template <class P, class R, class L>
+__device__ __forceinline__ void hs_put_momentum(unsigned char* smem, int e, int c, int nev, double x) {
+  if constexpr (sizeof(R) == 4) {
+    constexpr int EW = L::EW;
+    const dfl q = dfl_split(x);
+    float* d = reinterpret_cast<float*>(smem + L::o_p) + ((e / EW) * P::NPAR * 4 + c) * 2 * EW + e % EW;
+    d[0] = q.hi;
+    d[EW] = q.lo;
+    if (EW == 2 && e == nev - 1 && e % EW == 0) {
+      d[1] = q.hi;
+      d[EW + 1] = q.lo;
+    }
+  } else {
+    reinterpret_cast<double*>(smem + L::o_p)[e * P::NPAR * 4 + c] = x;
+  }
+}
+
 template <class P, class R, class L>
 __device__ __forceinline__ void hs_load_momenta(unsigned char* smem, const double* __restrict__ mom, int64_t nevt,
                                                 int64_t e0, int nev) {
   for (int t = threadIdx.x; t < nev * P::NPAR * 4; t += L::NT) {
     const int e = t % nev, c = t / nev;
-    const double x = mom[(int64_t)c * nevt + e0 + e];
-    if constexpr (sizeof(R) == 4) {
-      const dfl q = dfl_split(x);
-      reinterpret_cast<float2*>(smem + L::o_p)[e * P::NPAR * 4 + c] = make_float2(q.hi, q.lo);
-    } else {
-      reinterpret_cast<double*>(smem + L::o_p)[e * P::NPAR * 4 + c] = x;
-    }
+    hs_put_momentum<P, R, L>(smem, e, c, nev, mom[(int64_t)c * nevt + e0 + e]);
   }
 }
 
@@ -650,19 +673,12 @@ template <class P, class R, class L>
 __device__ __forceinline__ void hs_convert_momenta(unsigned char* smem, int nev) {
   const double* st = reinterpret_cast<const double*>(smem + L::o_ps);
   for (int t = threadIdx.x; t < nev * P::NPAR * 4; t += L::NT) {
-    const double x = st[t];
-    if constexpr (sizeof(R) == 4) {
-      const dfl q = dfl_split(x);
-      reinterpret_cast<float2*>(smem + L::o_p)[t] = make_float2(q.hi, q.lo);
-    } else {
-      reinterpret_cast<double*>(smem + L::o_p)[t] = x;
-    }
+    hs_put_momentum<P, R, L>(smem, t / (P::NPAR * 4), t % (P::NPAR * 4), nev, st[t]);
   }
 }
 
 // CUR_EV: 16-byte words from one unit's current variants to the next's; KEV:
-// momentum-table entries (V) from one unit's table to the next's.  Events that
-// fill up the last unit repeat the last event's momenta.
+// momentum-table entries (V) from one unit's table to the next's.
 template <class P, class R, class L, class V = R, int CUR_EV = P::HS_NSLOT * Slots<V, 1>::NPL, int KEV = 4 * P::NMOM>
 __device__ __forceinline__ void hs_tables(unsigned char* smem, const PhysParams& pp, int nev, uint4* curs,
                                           const Couplings<R>& cp) {
@@ -671,39 +687,36 @@ __device__ __forceinline__ void hs_tables(unsigned char* smem, const PhysParams&
   constexpr bool DF = sizeof(R) == 4;
   const int4* md = reinterpret_cast<const int4*>(smem + L::o_md);
   const int2* prop_tab = reinterpret_cast<const int2*>(smem + L::o_proptab);
-  R* K = reinterpret_cast<R*>(smem + L::o_K);    // V [unit][NMOM][4]
-  R* pr = reinterpret_cast<R*>(smem + L::o_pr);  // cx<V> [unit][NPROP]
-  const int nep = (nev + EW - 1) / EW * EW;
-  // one thread per (event, leg), both helicities (consecutive items)
+  const int nu = (nev + EW - 1) / EW, nep = nu * EW;
+  // one thread per (event, leg), both helicities (consecutive items), and one per
+  // (unit, momentum entry); the wavefunctions, the longer work, first
   static_assert(NEXT == 2 * NPAR, "level 0: two helicities per leg");
   constexpr int NE = NPAR;
-  for (int t = threadIdx.x; t < nep * (NM + NE); t += L::NT) {
-    // the wavefunctions, the longer work, first
-    const bool mom = t >= nep * NE;
-    const int t2 = mom ? t - nep * NE : t, e = t2 / (mom ? NM : NE), j = t2 - e * (mom ? NM : NE);
-    const int u = e / EW, lane = e - u * EW, es = EW == 1 ? e : min(e, nev - 1);
-    if (mom) {
+  for (int t = threadIdx.x; t < nep * NE + nu * NM; t += L::NT) {
+    if (t >= nep * NE) {
+      const int t2 = t - nep * NE, u = t2 / NM, j = t2 - u * NM;
       const int4 d = md[j];
-      auto put = [&](int pj, cx<R> f) {
-        pr[((u * P::NPROP + pj) * 2 + 0) * EW + lane] = f.re;
-        pr[((u * P::NPROP + pj) * 2 + 1) * EW + lane] = f.im;
-      };
+      V* const Kj = reinterpret_cast<V*>(smem + L::o_K) + u * KEV + 4 * j;
+      cx<V>* const pru = reinterpret_cast<cx<V>*>(smem + L::o_pr) + u * P::NPROP;
       if constexpr (DF) {
-        const float2* q = reinterpret_cast<const float2*>(smem + L::o_p) + es * NPAR * 4;
-        float2 kf[4];
+        struct alignas(sizeof(V) * 2) HiLo { V hi, lo; };
+        const HiLo* q = reinterpret_cast<const HiLo*>(smem + L::o_p) + u * NPAR * 4;
+        DflSum<V> k[4];
+        alignas(16) V kv[4];
 #pragma unroll
         for (int mu = 0; mu < 4; ++mu) {
-          DflSum k;
-          k.first(0.0f, 0.0f);
+          k[mu].first(V(0.0f), V(0.0f));
 #pragma unroll
           for (int l = 0; l < NPAR; ++l) {
-            const float2 v = q[l * 4 + mu];
-            const float c = (d.x >> l & 1) ? 1.0f : ((d.y >> l & 1) ? -1.0f : 0.0f);
-            k.add(c * v.x, c * v.y);
+            const HiLo v = q[l * 4 + mu];
+            const V c((d.x >> l & 1) ? 1.0f : ((d.y >> l & 1) ? -1.0f : 0.0f));
+            k[mu].add(c * v.hi, c * v.lo);
           }
-          kf[mu] = make_float2(k.s, k.err);
-          K[(u * KEV + 4 * j + mu) * EW + lane] = k.value();
+          kv[mu] = k[mu].value();
         }
+#pragma unroll
+        for (int i = 0; i < (int)(4 * sizeof(V) / 16); ++i)
+          reinterpret_cast<uint4*>(Kj)[i] = reinterpret_cast<const uint4*>(kv)[i];
         const float4* mc = reinterpret_cast<const float4*>(smem + L::o_mconst);
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
@@ -711,10 +724,10 @@ __device__ __forceinline__ void hs_tables(unsigned char* smem, const PhysParams&
           if (pj < 0) continue;
           const int kind = prop_tab[pj].y;
           const float4 c = mc[kind == 3 ? 1 : 0];  // {m^2 hi, m^2 lo, m w, 0} of the top / the Z
-          put(pj, propagator_dfl(kf, kind, dfl{c.x, c.y}, c.z));
+          pru[pj] = propagator_dfl<V>(k, kind, dfl{c.x, c.y}, c.z);
         }
       } else {
-        const double* q = reinterpret_cast<const double*>(smem + L::o_p) + es * NPAR * 4;
+        const double* q = reinterpret_cast<const double*>(smem + L::o_p) + u * NPAR * 4;
         double k[4];
 #pragma unroll
         for (int mu = 0; mu < 4; ++mu) {
@@ -725,16 +738,17 @@ __device__ __forceinline__ void hs_tables(unsigned char* smem, const PhysParams&
             s += c * q[l * 4 + mu];
           }
           k[mu] = s;
-          K[(u * KEV + 4 * j + mu) * EW + lane] = R(s);
+          Kj[mu] = R(s);
         }
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
           const int pj = i == 0 ? d.z : d.w;
           if (pj < 0) continue;
-          put(pj, propagator_hs<R>(k, prop_tab[pj].y, pp));
+          pru[pj] = propagator_hs<R>(k, prop_tab[pj].y, pp);
         }
       }
     } else {
+      const int e = t / NE, j = t - e * NE, u = e / EW, lane = e - u * EW;
       const HsSlots<P, V, P::HS_NSLOT> cur{curs + u * CUR_EV};
       const HsItem it = P::hs_items()[2 * j];
       W4<R> o[2];
@@ -742,13 +756,14 @@ __device__ __forceinline__ void hs_tables(unsigned char* smem, const PhysParams&
         dfl k[4];
 #pragma unroll
         for (int mu = 0; mu < 4; ++mu) {
-          const float2 v = reinterpret_cast<const float2*>(smem + L::o_p)[(es * NPAR + it.a) * 4 + mu];
-          k[mu] = dfl{v.x, v.y};
+          const float* v =
+              reinterpret_cast<const float*>(smem + L::o_p) + ((u * NPAR + it.a) * 4 + mu) * 2 * EW + lane;
+          k[mu] = dfl{v[0], v[EW]};
         }
         if (it.type == 2) ext_vector_dfl(k, it.c, o);
         else ext_fermion_dfl(k, it.flag ? cp.mt : 0.0f, it.c, it.type == 1, o);
       } else {
-        const double* k = reinterpret_cast<const double*>(smem + L::o_p) + (es * NPAR + it.a) * 4;
+        const double* k = reinterpret_cast<const double*>(smem + L::o_p) + (e * NPAR + it.a) * 4;
         if (it.type == 2) ext_vector_fp64(k, it.c, o);
         else ext_fermion_fp64(k, it.flag ? cp.mt : 0.0, it.c, it.type == 1, o);
       }

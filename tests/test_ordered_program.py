@@ -90,3 +90,42 @@ def test_helicity_subsets(orc, ng, nevt, mode):
         assert np.all(err <= fp64_tol(d_rot) * me_o)
     else:
         assert np.all(err <= MIXED_MAX_REL * me_o) and np.median(err / me_o) <= MIXED_MEDIAN_REL
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("proc,mode", [(p, m) for p in (1, 2, 3, 4) for m in ("fp64", "mixed")])
+def test_batch_size_does_not_change_an_event(proc, mode):
+    """How a batch is split into groups and pairs of events (one unit per CTA for
+    the smallest, full groups over several rounds, an odd last event) changes no
+    event's result: each batch equals the start of the largest one, bit for bit."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2106_12631_gb300 import mg
+    ecm = 500.0 if proc == 1 else 1500.0
+    most = 20011 if proc < 3 else 2611
+    mom, _ = mg.rambo_seeded(proc, most, ecm, seed=61 + proc)
+    mask = mg.filter_helicities(proc, mom[:, :, :16].contiguous())
+    want = mg.sigmakin(proc, mom, mask, mode=mode)
+    for n in (1, 2, 3, 151, 152, 153, 303, 305, 607, 609, 1215, 1217, 2433, most - 1):
+        got = mg.sigmakin(proc, mom[:, :, :n].contiguous(), mask, mode=mode)
+        torch.cuda.synchronize()
+        assert torch.equal(got, want[:n]), n
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [1, 1023, 1024, 1025, 5000, 1 << 20, (1 << 20) + 1])
+def test_unweight_block_counts(orc, n):
+    """Unweighting with one block, a ragged last block, the most blocks that find
+    maximum and offsets by themselves, and one more: the oracle's indices."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2106_12631_gb300 import mg
+    rng = np.random.default_rng(n)
+    me, wgt = rng.exponential(size=n), rng.uniform(0.5, 1.5, n)
+    u = I.uniforms(n + 7, 64, n)[63]
+    idx, count = mg.unweight(torch.from_numpy(me).cuda(), torch.from_numpy(wgt).cuda(), seed=n + 7)
+    torch.cuda.synchronize()
+    want = np.asarray(orc.unweight(me, wgt, u))
+    k = int(count.item())
+    assert k == len(want)
+    np.testing.assert_array_equal(idx[:k].cpu().numpy(), want)
