@@ -14,14 +14,6 @@
     constexpr int lock_every_ = MG_HS_LOCK_EVERY > 0 ? MG_HS_LOCK_EVERY : 1 << 30;    \
     if constexpr ((m) / lock_every_ != (n) / lock_every_) __syncthreads();            \
   } while (0)
-// A point of the straight-line contraction code that loads are not moved
-// across (a warp barrier): without it the g g -> t t~ g g kernel, at its 128
-// registers, loads operands early and spills
-#ifdef __CUDA_ARCH__
-#define HS_FENCE() __syncwarp()
-#else
-#define HS_FENCE()
-#endif
 #include "gen/proc1.cuh"
 #include "gen/proc2.cuh"
 #include "gen/proc3.cuh"

@@ -2049,7 +2049,6 @@ class OrderedProgram:
                                               add(wd(k, j, l), -1, "c"), add(wd(l, j, k), -1, "c")]))
                 L.append("    }")
         # V parts and the four-gluon vertices with V; then G(bc) . W(x, y)
-        L.append("    HS_FENCE();")
         L.append("    {")
         for ab, cd in self.pairings:
             nm = "P" + G(*ab)
@@ -2082,7 +2081,6 @@ class OrderedProgram:
                 L.append("          " + add((yy, b, c, xx), 1, "a") + " " + add((yy, c, b, xx), -1, "a") + " }")
                 flops += 64
                 L.append("      }")
-                L.append("      HS_FENCE();")
         L += ["    }", "  }"]
         self.flops_amps_hel = flops
         return L
