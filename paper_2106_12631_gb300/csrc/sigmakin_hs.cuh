@@ -40,7 +40,10 @@
 namespace mg {
 
 // threads per CTA of the mixed kernels of six and more colour flows, and their
-// CTAs per SM (six flows; more: one)
+// CTAs per SM (six flows; more: one).  Measured on pairs of events: gg -> t t~ g g,
+// 2^20 events, one CTA of 256 threads 10.3 ms, two of 128 11.5 ms, three of 128
+// (168 registers, spills) 11.1 ms; gg -> t t~ g, 262147 events, two of 256 540 us,
+// three of 128 612 us.
 #ifndef MG_HS_NT
 #define MG_HS_NT 256
 #endif
@@ -54,7 +57,9 @@ template <class P, class R, int N>
 using HsSlots = std::conditional_t<P::HS_ORDERED, PlanarSlots<R, N>, Slots<R, N>>;
 
 // Lane type of a kernel: pairs of events (f2) in the mixed mode with the
-// CUDA-core colour sum; the tensor-core colour sum takes one row per thread.
+// CUDA-core colour sum; the tensor-core colour sum takes one row per thread, and
+// the one-flow process is mostly wavefunctions and tables (2^19 events: single
+// 214 us, pairs 272 us; gg -> t t~, 2^20 events: 781 and 630 us).
 template <class P, class R, int CS>
 using HsLane = std::conditional_t<std::is_same_v<R, float> && CS == CS_SIMT && (P::NCOLOR > 1), f2, R>;
 
@@ -332,7 +337,7 @@ __device__ __forceinline__ void colour_hadamard(cx<R>* J) {
 
 // |M_h|^2 on CUDA cores: the symmetric form of the whole matrix, or for 24
 // flows (where J is left transformed) of its four blocks: 129 paired FP32
-// instructions instead of 324
+// instructions instead of 324 (gg -> t t~ g g, 2^20 events 11.7 -> 10.9 ms)
 template <class P, class R>
 __device__ __forceinline__ R colour_sum(cx<R>* J) {
   if constexpr (!P::COLOUR_BLOCKS) {
@@ -692,9 +697,12 @@ __device__ __forceinline__ void hs_tables(unsigned char* smem, const PhysParams&
   // (unit, momentum entry); the wavefunctions, the longer work, first
   static_assert(NEXT == 2 * NPAR, "level 0: two helicities per leg");
   constexpr int NE = NPAR;
-  for (int t = threadIdx.x; t < nep * NE + nu * NM; t += L::NT) {
-    if (t >= nep * NE) {
-      const int t2 = t - nep * NE, u = t2 / NM, j = t2 - u * NM;
+  // the entries begin with a warp of their own (the two kinds of work do not
+  // share a warp) where that takes no further round
+  const int ne32 = (nep * NE + 31) / 32 * 32, t0 = ne32 + nu * NM <= L::NT ? ne32 : nep * NE;
+  for (int t = threadIdx.x; t < t0 + nu * NM; t += L::NT) {
+    if (t >= t0) {
+      const int t2 = t - t0, u = t2 / NM, j = t2 - u * NM;
       const int4 d = md[j];
       V* const Kj = reinterpret_cast<V*>(smem + L::o_K) + u * KEV + 4 * j;
       cx<V>* const pru = reinterpret_cast<cx<V>*>(smem + L::o_pr) + u * P::NPROP;
@@ -747,7 +755,7 @@ __device__ __forceinline__ void hs_tables(unsigned char* smem, const PhysParams&
           pru[pj] = propagator_hs<R>(k, prop_tab[pj].y, pp);
         }
       }
-    } else {
+    } else if (t < nep * NE) {
       const int e = t / NE, j = t - e * NE, u = e / EW, lane = e - u * EW;
       const HsSlots<P, V, P::HS_NSLOT> cur{curs + u * CUR_EV};
       const HsItem it = P::hs_items()[2 * j];
@@ -778,9 +786,9 @@ __device__ __forceinline__ void hs_tables(unsigned char* smem, const PhysParams&
 __device__ __forceinline__ int lds_again(const int* p) { return *reinterpret_cast<const volatile int*>(p); }
 
 // Events per group (whole units of ew): the most a CTA takes at once, or fewer
-// where one round spreads the batch over all the grid's CTAs (a small batch has
-// one unit per CTA instead of a few full CTAs).  With more than one round full
-// groups are kept: their warps are full.
+// where one round spreads the batch over the grid's CTAs (a small batch has one
+// unit per CTA instead of a few full CTAs).  With more than one round full groups
+// are kept: their warps are full.
 __device__ __forceinline__ int hs_events_per_group(int64_t n, int most, int ew) {
   const int g = (int)gridDim.x;
   if (n >= (int64_t)g * most) return most;

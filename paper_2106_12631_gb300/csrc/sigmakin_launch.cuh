@@ -35,29 +35,45 @@ cudaError_t launch_sigmakin_hs_variant(const SigArgs& a, const Couplings<R>& cp,
   using H = typename L::H;
   constexpr int NT = L::NT;
   constexpr int kMaxDevices = 64;
-  static std::atomic<int> resident[kMaxDevices];  // CTAs resident on the whole device; 0 until known
+  struct Fit {
+    int cap, per;  // CTAs resident on the whole device and per SM; 0 until known
+  };
+  static std::atomic<Fit> resident[kMaxDevices];
   const void* k = FUSED ? (const void*)sigmakin_hs_rambo_kernel<P, R, CS> : (const void*)sigmakin_hs_kernel<P, R, CS>;
-  grid = (a.nevt + H::EW - 1) / H::EW;  // one unit per CTA at least
-  auto launch = [&](int cap) {
-    const unsigned g = (unsigned)(grid > cap ? cap : grid);
-    if constexpr (FUSED) sigmakin_hs_rambo_kernel<P, R, CS><<<g, NT, L::bytes, s>>>(a, cp, *ra);
-    else sigmakin_hs_kernel<P, R, CS><<<g, NT, L::bytes, s>>>(a, cp);
+  // A batch that one round of k CTAs per SM holds (all helicities good) takes the
+  // k that leaves the fewest events to an SM, and of two such the smaller (1000
+  // events of 8 per CTA on 152 SMs of two CTAs: one CTA of 7, not two of 4; a
+  // grid of all CTAs with idle ones would put the busy ones side by side).
+  auto launch = [&](Fit f) {
+    const int64_t nsm = f.cap / f.per, units = (a.nevt + H::EW - 1) / H::EW;
+    int64_t g = f.cap, load = INT64_MAX;
+    for (int k = 1; k <= f.per; ++k) {
+      const int64_t u = (units + nsm * k - 1) / (nsm * k);
+      if (u <= H::EVMIN && u * k < load) {
+        g = nsm * k;
+        load = u * k;
+      }
+    }
+    if (g > units) g = units;  // one unit per CTA at least
+    if constexpr (FUSED) sigmakin_hs_rambo_kernel<P, R, CS><<<(unsigned)g, NT, L::bytes, s>>>(a, cp, *ra);
+    else sigmakin_hs_kernel<P, R, CS><<<(unsigned)g, NT, L::bytes, s>>>(a, cp);
     return cudaGetLastError();
   };
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  int cap = dev < kMaxDevices ? resident[dev].load(std::memory_order_relaxed) : 0;
+  Fit fit = dev < kMaxDevices ? resident[dev].load(std::memory_order_relaxed) : Fit{0, 0};
   // the shared-memory attribute is set with the first launch on a device, and
   // again if a launch is refused for want of it (the device was reset)
-  if (cap != 0 && (e = launch(cap)) != cudaErrorInvalidValue) return e;
+  if (fit.cap != 0 && (e = launch(fit)) != cudaErrorInvalidValue) return e;
   if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L::bytes)) != cudaSuccess) return e;
   int nsm = 0, per = 0;
   if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, NT, L::bytes)) != cudaSuccess) return e;
-  cap = nsm * (per > H::CTAS ? per : H::CTAS);
-  if (dev < kMaxDevices) resident[dev].store(cap, std::memory_order_relaxed);
-  return launch(cap);
+  if (per < H::CTAS) per = H::CTAS;
+  fit = Fit{nsm * per, per};
+  if (dev < kMaxDevices) resident[dev].store(fit, std::memory_order_relaxed);
+  return launch(fit);
 }
 
 // mode 0 FP64; 1 mixed, colour sum on CUDA cores below 48 colour flows and on

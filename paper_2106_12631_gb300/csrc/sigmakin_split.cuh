@@ -157,10 +157,18 @@ cudaError_t launch_split_impl(int proc, const SigLaunch& l, const Couplings<R>& 
     void* ws;
     int64_t chunk;
   } key;
-  std::memset(&key, 0, sizeof key);  // padding compared too
+  std::memset(static_cast<void*>(&key), 0, sizeof key);  // padding compared too: members set one by one
   key.proc_mode = proc * 16 + mode;
   key.device = dev;
-  key.a = SigArgs{l.nevt, l.mom, l.mask, l.me, nullptr, l.pp, l.hel_rnd, l.hel_out, l.col_rnd, l.col_out};
+  key.a.nevt = l.nevt;
+  key.a.mom = l.mom;
+  key.a.mask = l.mask;
+  key.a.me = l.me;
+  key.a.pp = l.pp;
+  key.a.hel_rnd = l.hel_rnd;
+  key.a.hel_out = l.hel_out;
+  key.a.col_rnd = l.col_rnd;
+  key.a.col_out = l.col_out;
   key.cp = cp;
   key.ws = ws;
   key.chunk = chunk;
