@@ -179,7 +179,7 @@ int mg_event_sum_noalloc(int64_t nevt, const double* me, const double* wgt, doub
  * mg_rambo_seeded) followed by mg_sigmakin with the same mask and mode.  On
  * GB300 it saves memory, not time: RAMBO's FP64 work on one lane per event
  * takes longer than a group's matrix elements, so the kernel waits for it
- * (gg -> t t~ g g, 2^20 events, mixed: 44.5 ms against 22.2 ms for the two
+ * (gg -> t t~ g g, 2^20 events, mixed: 30.2 ms against 11.1 ms for the two
  * kernels).
  * mg_sigmakin_rambo: uniforms rnd [nrows][nevt] (device), as mg_rambo.
  * mg_sigmakin_seeded: uniforms drawn on the device, as mg_rambo_seeded
