@@ -26,10 +26,10 @@
 //   4. colour sum (CUDA cores, or tcgen05 as in sigmakin.cuh) and the
 //      fixed-order FP64 helicity sum.
 // What bounds it (gg -> t t~ g g mixed, 2^20 events): the bytes that the
-// contractions load from shared memory into registers (128 per clock and SM; 55 %
-// of the kernel's cycles) and the latency of dependent FMAs at 8 warps per SM
-// (FMA pipe 46 % busy): 10.3 ms, against 18.0 ms for the diagram-wise program on
-// single events.  In FP64 the FP64 pipe (90 % busy for gg -> t t~ g).
+// contractions load from shared memory into registers (128 per clock and SM; with
+// the items' loads 59 % of the kernel's cycles) and the latency of dependent FMAs
+// at 8 warps per SM (FMA pipe 49 % busy): 9.9 ms, against 18.0 ms for the
+// diagram-wise program on single events.  In FP64 the FP64 pipe (90 % busy for gg -> t t~ g).
 #pragma once
 #include <type_traits>
 
