@@ -98,29 +98,28 @@ __device__ __forceinline__ void atomic_addc(cx<R>* d, cx<R> v) {
 // values pass through the warp's staging area in shared memory (32 lanes x NV,
 // at most 8 values of R per lane): every lane stores its values and each
 // leader reads its members' (a group of n lanes costs its leader n - 1 reads,
-// not n - 1 rounds of warp-wide shuffles).  The lanes taking part are the ones
-// executing together (__activemask), and every collective below runs on all
-// of them.
-template <int NV, class R>
-__device__ __forceinline__ bool warp_group_sum(unsigned key, R* v, R* stage) {
+// not n - 1 rounds of warp-wide shuffles).  act: the lanes taking part, a mask
+// that the caller formed with a ballot (lanes that happen to run together after
+// a branch are no such set: a group split in two would have two leaders).
+// add(v): the leader's plain read-modify-write, done before the closing
+// barrier, so that the next call's leaders find it whichever lanes they are.
+template <int NV, class R, class F>
+__device__ __forceinline__ void warp_group_add(unsigned act, unsigned key, R* v, R* stage, F add) {
   static_assert(NV <= 8, "staging holds 8 values per lane");
-  const unsigned act = __activemask();
   const int lane = threadIdx.x & 31;
   const unsigned g = __match_any_sync(act, key);
-  if (!__any_sync(act, g != (1u << lane))) return true;  // every lane alone: no sums
-  R* mine = stage + 8 * lane;
-  if constexpr ((NV * sizeof(R)) % 16 == 0) {
+  if (__any_sync(act, g != (1u << lane))) {  // else every lane alone: no sums
+    R* mine = stage + 8 * lane;
+    if constexpr ((NV * sizeof(R)) % 16 == 0) {
 #pragma unroll
-    for (int i = 0; i < (int)(NV * sizeof(R) / 16); ++i)
-      reinterpret_cast<uint4*>(mine)[i] = reinterpret_cast<const uint4*>(v)[i];
-  } else {
+      for (int i = 0; i < (int)(NV * sizeof(R) / 16); ++i)
+        reinterpret_cast<uint4*>(mine)[i] = reinterpret_cast<const uint4*>(v)[i];
+    } else {
 #pragma unroll
-    for (int i = 0; i < NV; ++i) mine[i] = v[i];
-  }
-  __syncwarp(act);
-  const bool leader = lane == __ffs(g) - 1;
-  if (leader) {
-    unsigned others = g & ~(1u << lane);
+      for (int i = 0; i < NV; ++i) mine[i] = v[i];
+    }
+    __syncwarp(act);
+    unsigned others = lane == __ffs(g) - 1 ? g & ~(1u << lane) : 0u;
     while (others) {
       const int src = __ffs(others) - 1;
       others &= others - 1;
@@ -138,8 +137,8 @@ __device__ __forceinline__ bool warp_group_sum(unsigned key, R* v, R* stage) {
       }
     }
   }
+  if (lane == __ffs(g) - 1) add(v);
   __syncwarp(act);
-  return leader;
 }
 __device__ __forceinline__ unsigned smem_key(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 
@@ -148,42 +147,42 @@ __device__ __forceinline__ unsigned smem_key(const void* p) { return (unsigned)_
 // the group sum with a plain read-modify-write; the caller separates rounds of
 // items with __syncwarp.
 template <class R>
-__device__ __forceinline__ void own_add4(R* d, const R* v, R* stage) {
+__device__ __forceinline__ void own_add4(unsigned act, R* d, const R* v, R* stage) {
   alignas(16) R t[4] = {v[0], v[1], v[2], v[3]};
-  if (warp_group_sum<4>(smem_key(d), t, stage)) {
+  warp_group_add<4>(act, smem_key(d), t, stage, [d](const R* x) {
 #pragma unroll
-    for (int mu = 0; mu < 4; ++mu) d[mu] += t[mu];
-  }
+    for (int mu = 0; mu < 4; ++mu) d[mu] += x[mu];
+  });
 }
 template <class R>
-__device__ __forceinline__ void own_addc(cx<R>* d, cx<R> v, R* stage) {
+__device__ __forceinline__ void own_addc(unsigned act, cx<R>* d, cx<R> v, R* stage) {
   alignas(16) R t[2] = {v.re, v.im};
-  if (warp_group_sum<2>(smem_key(d), t, stage)) *d = cx<R>(d->re + t[0], d->im + t[1]);
+  warp_group_add<2>(act, smem_key(d), t, stage, [d](const R* x) { *d = cx<R>(d->re + x[0], d->im + x[1]); });
 }
 template <class R, int N>
-__device__ __forceinline__ void own_slot_add(const Slots<R, N>& s, int i, const W4<R>& w, R* stage) {
+__device__ __forceinline__ void own_slot_add(unsigned act, const Slots<R, N>& s, int i, const W4<R>& w, R* stage) {
   alignas(16) R t[8];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     t[2 * k] = w.w[k].re;
     t[2 * k + 1] = w.w[k].im;
   }
-  if (warp_group_sum<8>(smem_key(s.p + i), t, stage)) {
+  warp_group_add<8>(act, smem_key(s.p + i), t, stage, [&s, i](const R* x) {
     W4<R> o = s[i];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) o.w[k] = cx<R>(o.w[k].re + t[2 * k], o.w[k].im + t[2 * k + 1]);
+    for (int k = 0; k < 4; ++k) o.w[k] = cx<R>(o.w[k].re + x[2 * k], o.w[k].im + x[2 * k + 1]);
     s.set(i, o);
-  }
+  });
 }
 
 // Sum over the four aligned lanes of a current's consecutive variants (every
-// current has a multiple of four of them, and every phase's items and rounds
-// start at multiples of four lanes): these all add into one momentum and one
-// propagator adjoint, so the group sums that follow have a quarter of the
-// members (their leaders read them one by one).
+// current has a multiple of four of them, which the generator checks item by
+// item, and every phase's items and rounds start at multiples of four lanes):
+// these all add into one momentum and one propagator adjoint, so the group sums
+// that follow have a quarter of the members (their leaders read them one by
+// one).  act holds whole quads.
 template <int NV, class R>
-__device__ __forceinline__ void quad_sum(R* v) {
-  const unsigned act = __activemask();
+__device__ __forceinline__ void quad_sum(unsigned act, R* v) {
 #pragma unroll
   for (int i = 0; i < NV; ++i) v[i] += __shfl_xor_sync(act, v[i], 1);
 #pragma unroll
@@ -194,7 +193,7 @@ __device__ __forceinline__ void quad_sum(R* v) {
 template <class P, class R>
 __device__ __forceinline__ void hs_item_adj(const HsItem& it, const Slots<R, P::HS_NSLOT>& cur,
                                             const Slots<R, P::HS_NSLOT>& curb, const R* K, R* Kb, const cx<R>* pr,
-                                            cx<R>* prb, const Couplings<R>& cp, R* stage) {
+                                            cx<R>* prb, const Couplings<R>& cp, R* stage, unsigned act) {
   const W4<R> ob = curb[it.out];
   W4<R> b[3];
 #pragma unroll
@@ -225,17 +224,21 @@ __device__ __forceinline__ void hs_item_adj(const HsItem& it, const Slots<R, P::
       nin = 3;
     }
   }
-#pragma unroll
-  for (int k = 0; k < 3; ++k)
-    if (k < nin) own_slot_add(curb, it.in[k], b[k], stage);
-  quad_sum<4>(kb0);
-  quad_sum<4>(kb1);
-  quad_sum<1>(&pb.re);
-  quad_sum<1>(&pb.im);
-  if ((threadIdx.x & 3) == 0) {
-    if (nk >= 1) own_add4(Kb + 4 * it.k0, kb0, stage);
-    if (nk >= 2) own_add4(Kb + 4 * it.k1, kb1, stage);
-    own_addc(prb + it.prop, pb, stage);
+  own_slot_add(act, curb, it.in[0], b[0], stage);
+  own_slot_add(act, curb, it.in[1], b[1], stage);
+  const unsigned a3 = __ballot_sync(act, nin == 3);
+  if (nin == 3) own_slot_add(a3, curb, it.in[2], b[2], stage);
+  quad_sum<4>(act, kb0);
+  quad_sum<4>(act, kb1);
+  quad_sum<1>(act, &pb.re);
+  quad_sum<1>(act, &pb.im);
+  const bool first = (threadIdx.x & 3) == 0;
+  const unsigned q0 = act & 0x11111111u, q1 = __ballot_sync(act, first && nk >= 1),
+                 q2 = __ballot_sync(act, first && nk >= 2);
+  if (first) {
+    if (nk >= 1) own_add4(q1, Kb + 4 * it.k0, kb0, stage);
+    if (nk >= 2) own_add4(q2, Kb + 4 * it.k1, kb1, stage);
+    own_addc(q0, prb + it.prop, pb, stage);
   }
 }
 
@@ -243,7 +246,7 @@ __device__ __forceinline__ void hs_item_adj(const HsItem& it, const Slots<R, P::
 template <class P, class R>
 __device__ __forceinline__ void hs_xitem_adj(const HsItem& it, const Slots<R, P::HS_NSLOT>& cur,
                                              const Slots<R, P::HS_NSLOT>& curb, const Slots<R, P::HS_XCAP>& xbb,
-                                             const R* K, R* Kb, const Couplings<R>& cp, R* stage) {
+                                             const R* K, R* Kb, const Couplings<R>& cp, R* stage, unsigned act) {
   const W4<R> ob = xbb[it.out];
   W4<R> b[3];
 #pragma unroll
@@ -265,14 +268,17 @@ __device__ __forceinline__ void hs_xitem_adj(const HsItem& it, const Slots<R, P:
       nin = 3;
     }
   }
-#pragma unroll
-  for (int k = 0; k < 3; ++k)
-    if (k < nin) own_slot_add(curb, it.in[k], b[k], stage);
-  quad_sum<4>(kb0);
-  quad_sum<4>(kb1);
-  if (mom && (threadIdx.x & 3) == 0) {
-    own_add4(Kb + 4 * it.k0, kb0, stage);
-    own_add4(Kb + 4 * it.k1, kb1, stage);
+  own_slot_add(act, curb, it.in[0], b[0], stage);
+  own_slot_add(act, curb, it.in[1], b[1], stage);
+  const unsigned a3 = __ballot_sync(act, nin == 3);
+  if (nin == 3) own_slot_add(a3, curb, it.in[2], b[2], stage);
+  quad_sum<4>(act, kb0);
+  quad_sum<4>(act, kb1);
+  mom = mom && (threadIdx.x & 3) == 0;
+  const unsigned q = __ballot_sync(act, mom);
+  if (mom) {
+    own_add4(q, Kb + 4 * it.k0, kb0, stage);
+    own_add4(q, Kb + 4 * it.k1, kb1, stage);
   }
 }
 
@@ -415,11 +421,12 @@ __global__ void __launch_bounds__(HsGradCfg<P, R>::NT) sigmakin_hs_grad_kernel(G
     static_assert(ni % 4 == 0, "whole quads of variants");
     for (int r0 = 0; r0 < ni * nwe; r0 += 32) {
       const int t = r0 + lane, k = t / ni, ex = warp + NW * k;
+      const unsigned act = __ballot_sync(0xffffffffu, k < nwe);
       if (k < nwe) {
         const HsItem it = items[i0 + t - k * ni];
         hs_xitem_adj<P, R>(it, Slots<R, P::HS_NSLOT>{curs + ex * CUR_EV},
                            Slots<R, P::HS_NSLOT>{cursb + ex * CUR_EV}, Slots<R, P::HS_XCAP>{xbufsb + ex * X_EV},
-                           Kall + ex * P::NMOM * 4, Kball + ex * P::NMOM * 4, cp, wstage);
+                           Kall + ex * P::NMOM * 4, Kball + ex * P::NMOM * 4, cp, wstage, act);
       }
       __syncwarp();
     }
@@ -431,11 +438,12 @@ __global__ void __launch_bounds__(HsGradCfg<P, R>::NT) sigmakin_hs_grad_kernel(G
     static_assert(ni % 4 == 0, "whole quads of variants");
     for (int r0 = 0; r0 < ni * nwe; r0 += 32) {
       const int t = r0 + lane, k = t / ni, ex = warp + NW * k;
+      const unsigned act = __ballot_sync(0xffffffffu, k < nwe);
       if (k < nwe) {
         const HsItem it = items[i0 + t - k * ni];
         hs_item_adj<P, R>(it, Slots<R, P::HS_NSLOT>{curs + ex * CUR_EV}, Slots<R, P::HS_NSLOT>{cursb + ex * CUR_EV},
                           Kall + ex * P::NMOM * 4, Kball + ex * P::NMOM * 4, prall + ex * P::NPROP,
-                          prball + ex * P::NPROP, cp, wstage);
+                          prball + ex * P::NPROP, cp, wstage, act);
       }
       __syncwarp();
     }

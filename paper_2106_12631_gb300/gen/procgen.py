@@ -978,6 +978,19 @@ VVVV_PAIRS = {0: (((0, 2), (1, 3)), ((0, 3), (1, 2))),
               2: (((0, 1), (2, 3)), ((0, 2), (1, 3)))}
 
 
+def check_adjoint_quads(items, starts):
+    """The helicity-shared adjoint sums the momentum and propagator adjoints of four
+    consecutive items before it adds them: within each phase (starts: first item of
+    every phase, then the end) the items come in whole quads that agree in type,
+    momentum entries and propagator."""
+    for i0, i1 in zip(starts, starts[1:]):
+        if (i1 - i0) % 4:
+            raise ValueError("items %d to %d: not whole quads of variants" % (i0, i1))
+        for q in range(i0, i1, 4):
+            if len({(it[0],) + tuple(it[7:]) for it in items[q:q + 4]}) != 1:
+                raise ValueError("items %d to %d: variants of different currents in a quad" % (q, q + 3))
+
+
 class SharedProgram:
     SLOT_BUDGET = 768  # current + amputated-chunk variant slots per event (FP32: 8 events in 192 KB)
     # amputated-chunk slots per event are rounded up to a multiple of this: a
@@ -1366,6 +1379,8 @@ class SharedProgram:
                 for v in range(self.nvar(X)):
                     items.append(self._item(X, v))
         xitem_start.append(len(items))
+        if self.p.spec.pid in GRAD_PROCS:
+            check_adjoint_quads(items, level_start[1:] + xitem_start[1:])
         # amplitudes by chunk, then by amputated current (loaded once per run) and operand
         patterns = {}
         amps = []
