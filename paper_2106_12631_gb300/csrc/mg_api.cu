@@ -151,6 +151,7 @@ int rambo_setup(int proc, double ecm, mg::RamboSetup& st) {
   }
   if (!(msum < ecm)) return MG_ERR_ARG;
   st.xi0 = std::sqrt(1.0 - (msum / ecm) * (msum / ecm));
+  st.stop = std::fmax(1e-9 * (ecm - msum), 1e-15 * ecm);
   return MG_OK;
 }
 

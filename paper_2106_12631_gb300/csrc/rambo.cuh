@@ -18,7 +18,7 @@ namespace mg {
 struct RamboSetup {
   double w0;       // flat massless volume (pi/2)^(n-1) s^(n-2) / ((n-1)! (n-2)!)
   int massive;     // any final-state mass != 0
-  double xi0;      // Newton start sqrt(1 - (sum m / ecm)^2)
+  double xi0, stop;      // Newton start sqrt(1 - (sum m / ecm)^2)
   double m2[4];    // final-state masses squared
 };
 
@@ -92,8 +92,10 @@ __device__ __forceinline__ void rambo_forward(const double* r, double ecm, const
   }
   // Newton for sum_f sqrt(m_f^2 + xi^2 E_f^2) = ecm: first in FP32 to ~1e-7
   // (cheap; GB300 runs FP64 at 1/64 of the FP32 rate), then FP64 steps until one
-  // starts from a residual below 1e-9 ecm (the step squares the error, and its
-  // FP32 quotient leaves 1e-7 of it: the root to rounding)
+  // starts from a residual r below st.stop.  A step leaves r^2 / (4 T) at most, T =
+  // ecm - sum m the energy above threshold, and 1e-7 r of its FP32 quotient: from
+  // r = 1e-9 T nothing above rounding.  Near threshold 1e-9 T is below the
+  // rounding of r itself (about 1e-16 ecm): the bound is 1e-15 ecm there.
   float xf = (float)st.xi0;
   for (int it = 0; it < 12; ++it) {
     float fv = -(float)ecm, df = 0.0f;
@@ -117,7 +119,7 @@ __device__ __forceinline__ void rambo_forward(const double* r, double ecm, const
       df = fma(xi * e2, rt, df);
     }
     xi -= fv * (double)(1.0f / (float)df);
-    if (fabs(fv) <= 1e-9 * ecm) break;
+    if (fabs(fv) <= st.stop) break;
   }
   z.xi = xi;
   double w2 = 1.0, w3 = 0.0;
