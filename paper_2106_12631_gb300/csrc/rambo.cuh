@@ -118,7 +118,8 @@ __device__ __forceinline__ void rambo_forward(const double* r, double ecm, const
       fv += sqrt_of_rsqrt(t, rt);
       df = fma(xi * e2, rt, df);
     }
-    xi -= fv * (double)(1.0f / (float)df);
+    const float q = 1.0f / (float)df;
+    xi -= fv * (q > 1e-30f && q < 1e30f ? (double)q : 1.0 / df);  // energies outside FP32's range: FP64
     if (fabs(fv) <= st.stop) break;
   }
   z.xi = xi;

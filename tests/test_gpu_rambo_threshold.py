@@ -48,3 +48,21 @@ def test_energy_to_rounding(proc, above):
     err = energy_defect(mom.cpu().numpy(), ecm, mt) / bar(rnd, NF[proc], above, ecm)
     assert err.max() <= 1, err.max()
     assert bool(torch.isfinite(wgt).all())
+
+
+@pytest.mark.parametrize("scale", [1e-42, 1e42])
+def test_energies_outside_fp32(scale):
+    """The same process in units in which its energies leave FP32's range."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2106_12631_gb300 import mg
+    p = mg.get_params()
+    rnd = torch.from_numpy(I.uniforms(600, 12, 1001)).cuda()
+    try:
+        mg.set_params(**dict(p, mt=p["mt"] * scale))
+        mom, _ = mg.rambo(3, rnd, 1500.0 * scale)
+    finally:
+        mg.set_params(**p)
+    torch.cuda.synchronize()
+    err = energy_defect(mom.cpu().numpy() / scale, 1500.0, p["mt"]) / bar(rnd.cpu().numpy(), 3, 1154.0, 1500.0)
+    assert err.max() <= 1, err.max()
