@@ -63,6 +63,9 @@ __device__ __forceinline__ f2& operator+=(f2& a, f2 b) { a = a + b; return a; }
 __device__ __forceinline__ f2& operator-=(f2& a, f2 b) { a = a - b; return a; }
 __device__ __forceinline__ f2 operator/(f2 a, f2 b) { return f2(a.x / b.x, a.y / b.y); }
 __device__ __forceinline__ f2 fmac(f2 a, f2 b, f2 c) { return f2_of(__ffma2_rn(f2_raw(a), f2_raw(b), f2_raw(c))); }
+// a product and a sum that are rounded by themselves (dfl.cuh); the paired ones always are
+__device__ __forceinline__ f2 mul_rn(f2 a, f2 b) { return a * b; }
+__device__ __forceinline__ f2 add_rn(f2 a, f2 b) { return a + b; }
 __device__ __forceinline__ cx<f2> operator*(cx<f2> a, cx<f2> b) {
   return cx<f2>(fmac(-a.im, b.im, a.re * b.re), fmac(a.im, b.re, a.re * b.im));
 }

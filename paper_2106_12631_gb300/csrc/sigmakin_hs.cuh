@@ -33,6 +33,7 @@
 #pragma once
 #include <type_traits>
 
+#include "dfl.cuh"
 #include "rambo.cuh"
 #include "rng.cuh"
 #include "sigmakin.cuh"
@@ -379,52 +380,12 @@ __device__ __forceinline__ cx<R> propagator_hs(const double* k, int kind, const 
   return kind == 1 ? cx<R>(-ai, ar) : cx<R>(ai, -ar);
 }
 
-// ---- double-float arithmetic for the mixed mode ---------------------------------
-// A value as an unevaluated sum hi + lo of two FP32 numbers.  Sums use Knuth's
-// error-free TwoSum (the rounding error of a + b is exactly representable and
-// recovered with six additions) accumulated as in the cascaded summation of
-// Ogita, Rump and Oishi (SIAM J. Sci. Comput. 26, 2005); squares use the
-// FMA-based exact product.  The result is as accurate as a sum evaluated in
-// twice the FP32 precision and then rounded — ample for momentum sums rounded
-// to FP32 and for k^2 - m^2 near a pole — while GB300 runs FP32 at 64 times its
-// FP64 rate.
-struct dfl {
-  float hi, lo;
-};
-__device__ __forceinline__ dfl two_sum(float a, float b) {
-  const float s = a + b, bb = s - a;
-  return {s, (a - (s - bb)) + (b - bb)};
-}
-__device__ __forceinline__ dfl dfl_split(double x) {
-  const float h = (float)x;
-  return {h, (float)(x - (double)h)};
-}
-// sum of signed terms t_k = hi_k + lo_k, k = 0..n-1 (V: float, or a pair of events)
-template <class V>
-struct DflSum {
-  V s, err;
-  __device__ __forceinline__ void first(V hi, V lo) { s = hi; err = lo; }
-  __device__ __forceinline__ void add(V hi, V lo) {
-    const V t = s + hi, b = t - s;
-    err += ((s - (t - b)) + (hi - b)) + lo;
-    s = t;
-  }
-  __device__ __forceinline__ V value() const { return s + err; }
-};
-
-// Propagator factor from a double-float momentum: k^2 - m^2 summed error-free
-// from the exact squares of the components, then the reciprocal in FP32.
+// Propagator factor from a double-float momentum: k^2 - m^2 in double-float, then
+// the reciprocal in FP32.
 // m2 = m^2 as double-float, mw = m w.
 template <class V>
 __device__ __forceinline__ cx<V> propagator_dfl(const DflSum<V>* k, int kind, dfl m2, float mw) {
-  DflSum<V> d;
-#pragma unroll
-  for (int mu = 0; mu < 4; ++mu) {
-    const V h = k[mu].s, p = h * h;
-    const V e = fmac(V(2.0f) * h, k[mu].err, fmac(h, h, -p));
-    if (mu == 0) d.first(p, e);
-    else d.add(-p, -e);
-  }
+  DflSum<V> d = dfl_invariant(k);
   V di(0.0f);
   if (kind == 1 || kind == 3) {
     d.add(V(-m2.hi), V(-m2.lo));
@@ -434,30 +395,6 @@ __device__ __forceinline__ cx<V> propagator_dfl(const DflSum<V>* k, int kind, df
   const V inv = V(1.0f) / fmac(r, r, di * di);
   const V ar = r * inv, ai = -di * inv;
   return kind == 1 ? cx<V>(-ai, ar) : cx<V>(ai, -ar);
-}
-
-// Products, sums, reciprocals and reciprocal square roots of double-floats (the
-// low parts not normalised), accurate to a few 2^-46.
-__device__ __forceinline__ dfl dfl_mul(dfl a, dfl b) {
-  const float p = a.hi * b.hi;
-  return {p, fmaf(a.lo, b.hi, fmaf(a.hi, b.lo, fmaf(a.hi, b.hi, -p)))};
-}
-__device__ __forceinline__ dfl dfl_add(dfl a, dfl b) {
-  const dfl s = two_sum(a.hi, b.hi);
-  return {s.hi, s.lo + (a.lo + b.lo)};
-}
-__device__ __forceinline__ float dfl_value(dfl a) { return a.hi + a.lo; }
-// one Newton step in FP32 on the FP32 value, its residual formed with FMAs; a
-// residual that is not small (the square of the value overflows) is dropped
-__device__ __forceinline__ float small_or_zero(float r) { return fabsf(r) < 1e-3f ? r : 0.0f; }
-__device__ __forceinline__ dfl dfl_rsqrt(dfl s) {
-  const float y = rsqrtf(s.hi), t = y * y, tl = fmaf(y, y, -t);
-  const float r = fmaf(s.hi, t, -1.0f) + fmaf(s.hi, tl, s.lo * t);
-  return {y, -0.5f * y * small_or_zero(r)};
-}
-__device__ __forceinline__ dfl dfl_rcp(dfl b) {
-  const float y = 1.0f / b.hi;
-  return {y, y * small_or_zero(-fmaf(b.hi, y, -1.0f) - b.lo * y)};
 }
 
 // External wavefunctions of the mixed mode, both helicities of a leg from its
