@@ -55,9 +55,12 @@ cudaError_t launch_sigmakin_hs_variant(const SigArgs& a, const Couplings<R>& cp,
       }
     }
     if (g > units) g = units;  // one unit per CTA at least
-    if constexpr (FUSED) sigmakin_hs_rambo_kernel<P, R, CS><<<(unsigned)g, NT, L::bytes, s>>>(a, cp, *ra);
-    else sigmakin_hs_kernel<P, R, CS><<<(unsigned)g, NT, L::bytes, s>>>(a, cp);
-    return cudaGetLastError();
+    // the launch's own status, not the thread's last error: that may be an
+    // earlier call's, which is not ours to answer with a second launch
+    void* args[] = {const_cast<SigArgs*>(&a), const_cast<Couplings<R>*>(&cp), const_cast<RamboArgs*>(ra)};
+    const cudaError_t e = cudaLaunchKernel(k, dim3((unsigned)g), dim3(NT), args, L::bytes, s);
+    if (e != cudaSuccess) cudaGetLastError();  // reported by the return value
+    return e;
   };
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
