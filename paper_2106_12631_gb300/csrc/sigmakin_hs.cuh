@@ -316,9 +316,8 @@ __device__ __forceinline__ R colour_sum_sym(const cx<R>* J) {
   return sum / R(P::CDEN);
 }
 
-// Four-point Hadamard transform of every orbit of chains, in place; BACK: its
-// inverse (times 1/4)
-template <class P, class R, bool BACK>
+// Four-point Hadamard transform of every orbit of chains, in place
+template <class P, class R>
 __device__ __forceinline__ void colour_hadamard(cx<R>* J) {
   static_for<0, 6>([&](auto O) {
     constexpr int o = decltype(O)::value;
@@ -329,10 +328,6 @@ __device__ __forceinline__ void colour_hadamard(cx<R>* J) {
     b = ab - cd;
     c = am + cm;
     d = am - cm;
-    if constexpr (BACK) {
-      const R s(0.25);
-      a = s * a; b = s * b; c = s * c; d = s * d;
-    }
   });
 }
 
@@ -344,7 +339,7 @@ __device__ __forceinline__ R colour_sum(cx<R>* J) {
   if constexpr (!P::COLOUR_BLOCKS) {
     return colour_sum_sym<P, R>(J);
   } else {
-    colour_hadamard<P, R, false>(J);
+    colour_hadamard<P, R>(J);
     cx<R> tot(R(0), R(0));  // re: sum of the products' real parts; im: of the imaginary parts
     static_for<0, 24>([&](auto I) {
       constexpr int x = decltype(I)::value / 6, i = decltype(I)::value % 6;
@@ -1145,6 +1140,29 @@ __device__ __forceinline__ void hs_sigmakin_body(const SigArgs& a, const Couplin
     for (int s = 0; s < NC; ++s) J[s] = cx<V>(V(0), V(0));
     P::template hs_contract<V>(0, HsSlots<P, V, P::HS_NSLOT>{curs + u * CUR_EV},
                                HsSlots<P, V, P::HS_XCAP>{xbufs + u * X_EV}, vtab + good[kh], J);
+    // the flows' |J_s|^2 for the choice of one (batched entry point), into the union
+    // once every thread of the CTA is done with it: from the J of the chains,
+    // before the colour sum transforms them (back and forth a small flow would
+    // carry the rounding of the largest of its orbit)
+    [[maybe_unused]] auto stage_flows = [&] {
+      __syncthreads();
+      R* wj = reinterpret_cast<R*>(smem + L::o_U);  // rows as sm2's
+      if (active) {
+#pragma unroll
+        for (int i = 0; i < EW; ++i)
+#pragma unroll
+          for (int s = 0; s < NC; ++s) {
+            const R re = lane_value(J[s].re, i), im = lane_value(J[s].im, i);
+            wj[((u * EW + i) * ng + kh) * HsChoice<P, R>::NCP + s] = re * re + im * im;
+          }
+      }
+    };
+    // (compiled in for every source of momenta, though only mg_matrix_elements_batch
+    // asks for choices: the branch also keeps the loads of the contractions where
+    // they are.  Without it the kernel with RAMBO inside takes 255 registers and
+    // spills, 30011 gg -> t t~ g g events 965 us instead of 871)
+    if constexpr (!L::TC)
+      if (a.col_out) stage_flows();
     // 4. colour sum and helicity sum; |M_h|^2 of (event, good helicity) k at
     //    sm2[event * ng + k]
     V m2;
@@ -1180,24 +1198,15 @@ __device__ __forceinline__ void hs_sigmakin_body(const SigArgs& a, const Couplin
       sum += __shfl_xor_sync(0xffffffffu, sum, 4);
       if (t < nev * 8 && q == 0) a.me[e0 + eh] = sum * *reinterpret_cast<const double*>(misc + 8);
     }
-    // 5. helicity and colour-flow choices (batched entry point), once every
-    //    group of the CTA is done with the union region; the closing barrier
-    //    keeps the next group's currents out of it until the choices are made
-    if (a.hel_out || a.col_out) {
-      __syncthreads();
-      if (a.col_out) {
-        if constexpr (!L::TC && P::COLOUR_BLOCKS) colour_hadamard<P, V, true>(J);  // back to the chains
-        R* wj = reinterpret_cast<R*>(smem + L::o_U);  // the union is dead here; rows as sm2's
-        if (active) {
-#pragma unroll
-          for (int i = 0; i < EW; ++i)
-#pragma unroll
-            for (int s = 0; s < NC; ++s) {
-              const R re = lane_value(J[s].re, i), im = lane_value(J[s].im, i);
-              wj[((u * EW + i) * ng + kh) * HsChoice<P, R>::NCP + s] = re * re + im * im;
-            }
+    // 5. helicity and colour-flow choices (batched entry point); the closing
+    //    barrier keeps the next group's currents out of the union, and its sm2
+    //    unwritten, until the choices are made
+    if (SRC == kSrcMomenta && (a.hel_out || a.col_out)) {
+      if constexpr (L::TC) {  // the tensor cores have read their tiles
+        if (a.col_out) {
+          stage_flows();
+          __syncthreads();
         }
-        __syncthreads();
       }
       hs_choices<P, R, L>(smem, a, e0, nev, ng, good, sm2);
       __syncthreads();
