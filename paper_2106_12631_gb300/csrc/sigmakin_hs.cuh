@@ -65,17 +65,20 @@ template <class P, class R, int CS>
 using HsLane = std::conditional_t<std::is_same_v<R, float> && CS == CS_SIMT && (P::NCOLOR > 1), f2, R>;
 
 // CTA shape.  A thread takes one helicity of one unit, a unit being the events
-// of a lane (a pair in the mixed mode).
-template <class P, class R, int CS = CS_SIMT>
+// of a lane (a pair in the mixed mode).  FUSED: the kernel with RAMBO inside.
+template <class P, class R, int CS = CS_SIMT, bool FUSED = false>
 struct HsCfg {
   using V = HsLane<P, R, CS>;
   static constexpr int EW = LaneOf<V>::EW;
   // measured: 128 threads for pairs of g g -> t t~ events (2^20 events 565 us, 256
   // threads 632 us) and for FP64 e+e- -> mu+mu- (200003 events 1256 us, 1301 us);
   // 256 for FP64 g g -> t t~ (100003 events 914 us, 128 threads 974 us) and mixed
-  // e+e- -> mu+mu- (200003 events 91 us, 97 us), as for the larger processes
-  static constexpr int NT =
-      (P::NCOLOR == 2 && EW == 2) || (P::NCOLOR == 1 && sizeof(R) == 8) ? 128 : EW == 2 ? MG_HS_NT : 256;
+  // e+e- -> mu+mu- (200003 events 91 us, 97 us), as for the larger processes.  With
+  // RAMBO inside, e+e- -> mu+mu- waits for one lane per event: CTAs of half the
+  // threads, four per SM instead of two, are the faster ones (131072 events mixed
+  // 115 us, 256 threads 167 us; not with the tensor-core colour sum, 346 and 320 us).
+  static constexpr bool HALF = P::NCOLOR == 1 ? sizeof(R) == 8 || (FUSED && CS == CS_SIMT) : P::NCOLOR == 2 && EW == 2;
+  static constexpr int NT = HALF ? 128 : EW == 2 ? MG_HS_NT : 256;
   static constexpr int EVMIN = (NT / P::NHEL) > 0 ? (NT / P::NHEL) : 1;  // units, all helicities good
   // room for groups of fewer helicities than all: four times the units with one
   // flow (four of the sixteen helicities of e+e- -> mu+mu- are good); none for the
@@ -96,9 +99,9 @@ struct HsCfg {
   static constexpr int MBLK = NT / 128;
 };
 
-template <class P, class R, int CS>
+template <class P, class R, int CS, bool FUSED = false>
 struct HsLayout {
-  using H = HsCfg<P, R, CS>;
+  using H = HsCfg<P, R, CS, FUSED>;
   using V = typename H::V;
   static constexpr int EW = H::EW;
   static constexpr int NT = H::NT, EVCAP = H::EVCAP, KP = H::KP, NP = H::NP, MBLK = H::MBLK;
@@ -962,7 +965,7 @@ __device__ __forceinline__ double hs_norm(const PhysParams& pp) {
 template <class P, class R, int CS, int SRC>
 __device__ __forceinline__ void hs_sigmakin_body(const SigArgs& a, const Couplings<R>& cp, int64_t first, int64_t last,
                                                  const uint4* __restrict__ rec, const RamboArgs* ra = nullptr) {
-  using L = HsLayout<P, R, CS>;
+  using L = HsLayout<P, R, CS, SRC == kSrcRambo>;
   using V = typename L::V;
   constexpr bool FROM_RECORDS = SRC == kSrcRecords;
   static_assert(!(FROM_RECORDS && L::TC), "the kernel-split variant sums colours on CUDA cores");
@@ -1227,7 +1230,7 @@ __global__ void __launch_bounds__(HsCfg<P, R, CS>::NT, HsCfg<P, R, CS>::CTAS) si
 
 // RAMBO and SIGMAKIN in one kernel: no momentum buffer in HBM
 template <class P, class R, int CS>
-__global__ void __launch_bounds__(HsCfg<P, R, CS>::NT, HsCfg<P, R, CS>::CTAS)
+__global__ void __launch_bounds__(HsCfg<P, R, CS, true>::NT, HsCfg<P, R, CS, true>::CTAS)
     sigmakin_hs_rambo_kernel(SigArgs a, Couplings<R> cp, RamboArgs ra) {
   hs_sigmakin_body<P, R, CS, kSrcRambo>(a, cp, 0, a.nevt, nullptr, &ra);
 }

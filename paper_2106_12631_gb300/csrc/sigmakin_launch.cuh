@@ -31,7 +31,7 @@ cudaError_t launch_sigmakin_variant(const SigArgs& a, const Couplings<R>& cp, in
 template <class P, class R, int CS, bool FUSED = false>
 cudaError_t launch_sigmakin_hs_variant(const SigArgs& a, const Couplings<R>& cp, int64_t grid, cudaStream_t s,
                                        const RamboArgs* ra = nullptr) {
-  using L = HsLayout<P, R, CS>;
+  using L = HsLayout<P, R, CS, FUSED>;
   using H = typename L::H;
   constexpr int NT = L::NT;
   constexpr int kMaxDevices = 64;
