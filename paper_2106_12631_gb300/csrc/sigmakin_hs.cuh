@@ -741,6 +741,26 @@ __device__ __forceinline__ int hs_item_of(int t, int nu) {
   return nu == L::EVCAP ? t / L::EVCAP : (nu == 1 ? t : (int)__umulhi((unsigned)t, 0xffffffffu / (unsigned)nu + 1u));
 }
 
+// Lanes per item of a phase: one per unit.  Where a process has so few items that
+// one round holds eight lanes of each, no fewer than eight: a warp then has four
+// variants of one current, where a warp of 32 items would go through every vertex
+// type one after the other (64 gg -> t t~ events FP64, one per CTA, 22.1 -> 17.6 us;
+// with sixteen lanes 20.0 us, twice the warps in the FP64 pipe.  64 e+e- -> mu+mu-
+// events FP64 18.5 -> 14.1 us).
+template <class P, class L>
+__host__ __device__ constexpr bool hs_few_items() {
+  int most = P::HS_NITEM - P::hs_level(P::HS_NLEVEL);
+  for (int l = 1; l < P::HS_NLEVEL; ++l) {
+    const int n = P::hs_level(l + 1) - P::hs_level(l);
+    if (n > most) most = n;
+  }
+  return L::EVCAP >= 8 && 8 * most <= L::NT;
+}
+template <class P, class L>
+__host__ __device__ constexpr int hs_lanes(int nu) {
+  return hs_few_items<P, L>() && nu < 8 ? 8 : nu;
+}
+
 // Items of the ordered program: a two-leg current ...
 template <class P, class R>
 __device__ __forceinline__ void ord_item(const HsItem& it, const HsSlots<P, R, P::HS_NSLOT>& cur, const R* K,
@@ -1060,6 +1080,8 @@ __device__ __forceinline__ void hs_sigmakin_body(const SigArgs& a, const Couplin
     const int ev = lds_again(misc + 7);
     const int nev = (int)min((int64_t)ev, last - (first + (int64_t)g * ev));
     const int nu = (nev + EW - 1) / EW;
+    constexpr bool FEW = hs_few_items<P, L>();
+    const int nl = hs_lanes<P, L>(nu);  // lanes per item
     if constexpr (FROM_RECORDS) {
       // 1-2. the units' current variants and momentum tables from their records
       using RC = HsRecord<P, V>;
@@ -1103,9 +1125,10 @@ __device__ __forceinline__ void hs_sigmakin_body(const SigArgs& a, const Couplin
       //    came with phase 1); consecutive threads take one item for each event (hs_item_of)
 #pragma unroll
       for (int l = 1; l < P::HS_NLEVEL; ++l) {
-        const int i0 = P::hs_level(l), n = (P::hs_level(l + 1) - i0) * nu;
+        const int i0 = P::hs_level(l), n = (P::hs_level(l + 1) - i0) * nl;
         for (int t = tid; t < n; t += NT) {
-          const int ii = hs_item_of<L>(t, nu), u = t - ii * nu;
+          const int ii = hs_item_of<L>(t, nl), u = t - ii * nl;
+          if (FEW && u >= nu) continue;
           const HsItem it = items[i0 + ii];
           const HsSlots<P, V, P::HS_NSLOT> cur{curs + u * CUR_EV};
           if constexpr (P::HS_ORDERED) ord_item<P, V>(it, cur, Kall + u * L::KEV, prall + u * P::NPROP, cv);
@@ -1124,9 +1147,10 @@ __device__ __forceinline__ void hs_sigmakin_body(const SigArgs& a, const Couplin
     //    thread contracts for its (unit, helicity), J in registers
     static_assert(P::HS_NXCHUNK == 1, "the operands of every contraction at once");
     {
-      const int i0 = P::hs_xitem(0), n = (P::hs_xitem(1) - i0) * nu;
+      const int i0 = P::hs_xitem(0), n = (P::hs_xitem(1) - i0) * nl;
       for (int t = tid; t < n; t += NT) {
-        const int ii = hs_item_of<L>(t, nu), ui = t - ii * nu;
+        const int ii = hs_item_of<L>(t, nl), ui = t - ii * nl;
+        if (FEW && ui >= nu) continue;
         const HsItem it = items[i0 + ii];
         const HsSlots<P, V, P::HS_NSLOT> cur{curs + ui * CUR_EV};
         const HsSlots<P, V, P::HS_XCAP> xs{xbufs + ui * X_EV};

@@ -23,7 +23,18 @@ template <class P, class R, int CS, bool FUSED> void show(const char* name) {
   using L = mg::HsLayout<P, R, CS, FUSED>;
   std::printf("%s %zu %d %d %d\n", name, (size_t)L::bytes, L::NT, L::EVCAP * L::EW, L::H::CTAS);
 }
+template <class P, class R, int CS> void lanes(const char* name) {
+  using L = mg::HsLayout<P, R, CS>;
+  std::printf("%s", name);
+  for (int nu = 1; nu <= L::EVCAP; ++nu) std::printf(" %d", mg::hs_lanes<P, L>(nu));
+  std::printf("\n");
+}
 int main() {
+  lanes<mg::Proc1, double, mg::CS_SIMT>("lanes_1_fp64");
+  lanes<mg::Proc1, float, mg::CS_SIMT>("lanes_1_mixed");
+  lanes<mg::Proc2, double, mg::CS_SIMT>("lanes_2_fp64");
+  lanes<mg::Proc2, float, mg::CS_SIMT>("lanes_2_mixed");
+  lanes<mg::Proc2, float, mg::CS_TC>("lanes_2_tc");
   show<mg::Proc1, float, mg::CS_SIMT, true>("p1_fused");
   return 0;
 }
@@ -57,3 +68,25 @@ def test_fused_rambo_lanes(tmp_path):
     regs = registers(tmp_path, "sigmakin_p1.cu", "sigmakin_hs_rambo_kernelINS_5Proc1EfLi0E")
     ctas = min(SM_REGISTERS // ((regs + 7) // 8 * 8 * nt), SM_BYTES // (nbytes + CTA_RESERVED))
     assert ctas * min(events, nt // 4) >= 128, (ctas, events, nt, regs)
+
+
+def test_warps_of_small_groups_hold_one_vertex_type(tmp_path):
+    """e+e- -> mu+mu- and gg -> t t~ have a dozen items per phase: a group of one
+    event would put all of them on one warp, every vertex type after the other."""
+    checked = 0
+    for name, lanes in layouts(tmp_path).items():
+        if not name.startswith("lanes_"):
+            continue
+        pid = int(name.split("_")[1])
+        text = open(os.path.join(B.CSRC, "gen", "proc%d.cuh" % pid)).read()
+        table = re.search(r"kHsItems%d\[\d+\] = \{(.*?)\};" % pid, text).group(1)
+        types = [int(m.group(1)) for m in re.finditer(r"\{\d+, \{[^}]*\}, (\d+),", table)]
+        levels = [int(x) for x in re.search(r"hs_level\(int i\) \{\s*constexpr int t\[\d+\] = \{([^}]*)\}", text).group(1).split(",")]
+        for i0, i1 in zip(levels[1:], levels[2:] + [len(types)]):
+            for nu, nl in zip(range(1, len(lanes) + 1), lanes):
+                assert nl >= nu
+                for w in range(0, (i1 - i0) * nl, 32):
+                    held = {types[i0 + t // nl] for t in range(w, min(w + 32, (i1 - i0) * nl)) if t % nl < nu}
+                    assert len(held) <= (1 if nl == 8 else 2), (name, nu, nl, held)
+                    checked += 1
+    assert checked
