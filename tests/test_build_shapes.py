@@ -87,6 +87,6 @@ def test_warps_of_small_groups_hold_one_vertex_type(tmp_path):
                 assert nl >= nu
                 for w in range(0, (i1 - i0) * nl, 32):
                     held = {types[i0 + t // nl] for t in range(w, min(w + 32, (i1 - i0) * nl)) if t % nl < nu}
-                    assert len(held) <= (1 if nl == 8 else 2), (name, nu, nl, held)
+                    assert len(held) <= (1 if nu <= 8 else 2), (name, nu, nl, held)
                     checked += 1
     assert checked
