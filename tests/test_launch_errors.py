@@ -1,4 +1,4 @@
-"""Launch errors of the helicity-shared kernels, on a fake CUDA runtime (no GPU needed).
+"""Launches of the helicity-shared kernels, on a fake CUDA runtime (no GPU needed).
 
 The launcher is compiled and linked against a runtime whose calls are counted
 and whose answers the test chooses.
@@ -10,6 +10,8 @@ and whose answers the test chooses.
   gone with a device reset) sets the attribute and is made again, once.
 * Any other refusal is returned as it is, and no refusal is left behind in the
   last-error state for the next call to find.
+* A batch whose choices of helicities and flows one round of CTAs holds is
+  spread so that the CTAs' warps, one per event, take the fewest rounds.
 """
 import os
 import shutil
@@ -24,9 +26,10 @@ RUNTIME = r'''
 // the runtime's entry points by name: every handle and enumeration is a word here
 extern "C" {
 struct dim3_ { unsigned x, y, z; };
-int launches, attributes, refuse, answer, last;
-int cudaLaunchKernel(const void*, dim3_, dim3_, void**, size_t, void*) {
+int launches, attributes, refuse, answer, last, ctas, fit = 1;
+int cudaLaunchKernel(const void*, dim3_ g, dim3_, void**, size_t, void*) {
   ++launches;
+  ctas = g.x;
   if (refuse == 0) return 0;
   --refuse;
   return last = answer;
@@ -36,8 +39,8 @@ int cudaGetLastError() { const int e = last; last = 0; return e; }
 int cudaGetDevice(int* d) { *d = 0; return 0; }
 int cudaFuncSetAttribute(const void*, int, int) { ++attributes; return 0; }
 int cudaDeviceGetAttribute(int* v, int, int) { *v = 152; return 0; }
-int cudaOccupancyMaxActiveBlocksPerMultiprocessor(int* n, const void*, int, size_t) { *n = 1; return 0; }
-int cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void*, int, size_t, unsigned) { *n = 1; return 0; }
+int cudaOccupancyMaxActiveBlocksPerMultiprocessor(int* n, const void*, int, size_t) { *n = fit; return 0; }
+int cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void*, int, size_t, unsigned) { *n = fit; return 0; }
 int __cudaGetKernel(void** k, const void* f) { *k = (void*)f; return 0; }
 int cudaGetKernel(void** k, const void* f) { *k = (void*)f; return 0; }
 static dim3_ grid, block;
@@ -81,17 +84,43 @@ int main() {
 '''
 
 
-@pytest.mark.skipif(shutil.which("nvcc") is None and not os.path.exists("/usr/local/cuda/bin/nvcc"),
-                    reason="nvcc not available")
-def test_launch_errors(tmp_path):
+SPREAD = r'''
+#include "process.cuh"
+#include "sigmakin_launch.cuh"
+#include <cstdio>
+extern "C" int ctas, fit;
+int main() {
+  fit = 5;
+  using H = mg::HsCfg<mg::Proc2, float>;
+  mg::Couplings<float> cp{};
+  int32_t hel;
+  for (int n : {64, 700, 1000, 1301, 2001}) {
+    mg::SigArgs a{};
+    a.nevt = n;
+    a.hel_out = &hel;
+    mg::launch_sigmakin_hs_variant<mg::Proc2, float, mg::CS_SIMT>(a, cp, 0, nullptr);
+    std::printf("%d %d %d %d\n", n, ctas, H::NT / 32, H::EW);
+  }
+  return 0;
+}
+'''
+
+
+def run(tmp_path, source):
     src, fake, exe = tmp_path / "probe.cu", tmp_path / "runtime.cpp", tmp_path / "probe"
-    src.write_text(SRC)
+    src.write_text(source)
     fake.write_text(RUNTIME)
     r = subprocess.run([B.nvcc(), *B.ARCH, *B.FLAGS, "-Xptxas", "-O0", "-cudart", "none", str(src), str(fake),
                         "-o", str(exe)], capture_output=True, text=True)
     assert r.returncode == 0, r.stderr[-3000:]
     out = subprocess.run([str(exe)], capture_output=True, text=True, check=True).stdout.split("\n")
-    rows = [tuple(int(x) for x in ln.split()) for ln in out if ln.strip()]
+    return [tuple(int(x) for x in ln.split()) for ln in out if ln.strip()]
+
+
+@pytest.mark.skipif(shutil.which("nvcc") is None and not os.path.exists("/usr/local/cuda/bin/nvcc"),
+                    reason="nvcc not available")
+def test_launch_errors(tmp_path):
+    rows = run(tmp_path, SRC)
     invalid_value, invalid_device, out_of_resources = 1, 101, 701
     #        status            launches attributes last error left
     assert rows == [(0, 1, 1, 0),
@@ -101,3 +130,13 @@ def test_launch_errors(tmp_path):
                     (0, 2, 1, 0),
                     (invalid_value, 2, 1, 0),
                     (out_of_resources, 1, 0, 0)]
+
+
+@pytest.mark.skipif(shutil.which("nvcc") is None and not os.path.exists("/usr/local/cuda/bin/nvcc"),
+                    reason="nvcc not available")
+def test_choices_take_the_fewest_rounds(tmp_path):
+    for n, ctas, warps, per_unit in run(tmp_path, SPREAD):
+        units = -(-n // per_unit)
+        rounds = lambda g: -(-(-(-units // g)) * per_unit // warps)
+        assert ctas <= units
+        assert rounds(ctas) == min(rounds(152 * k) for k in range(1, 6)), (n, ctas)
