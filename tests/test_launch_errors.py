@@ -12,6 +12,7 @@ and whose answers the test chooses.
   last-error state for the next call to find.
 * A batch whose choices of helicities and flows one round of CTAs holds is
   spread so that the CTAs' warps, one per event, take the fewest rounds.
+* The kernel-split variant's second kernel spreads a small chunk over the SMs.
 """
 import os
 import shutil
@@ -140,3 +141,30 @@ def test_choices_take_the_fewest_rounds(tmp_path):
         rounds = lambda g: -(-(-(-units // g)) * per_unit // warps)
         assert ctas <= units
         assert rounds(ctas) == min(rounds(152 * k) for k in range(1, 6)), (n, ctas)
+
+
+SPLIT = r'''
+#include "process.cuh"
+#include "sigmakin_split.cuh"
+#include <cstdio>
+extern "C" int ctas;
+int main() {
+  using H = mg::HsCfg<mg::Proc3, float>;
+  mg::SigArgs a{};
+  a.nevt = 1 << 20;
+  mg::Couplings<float> cp{};
+  for (int n : {1, 3, 64, 257, 1000, 2433, 100003}) {
+    mg::SplitLaunch<mg::Proc3, float>::amplitudes(a, cp, 0, n, nullptr, nullptr);
+    std::printf("%d %d %d %d\n", n, ctas, H::EVMIN, H::EW);
+  }
+  return 0;
+}
+'''
+
+
+@pytest.mark.skipif(shutil.which("nvcc") is None and not os.path.exists("/usr/local/cuda/bin/nvcc"),
+                    reason="nvcc not available")
+def test_split_chunks_fill_the_sms(tmp_path):
+    for n, ctas, group, per_unit in run(tmp_path, SPLIT):
+        units = -(-n // per_unit)
+        assert ctas == max(-(-units // group), min(units, 152)), (n, ctas)
