@@ -36,6 +36,10 @@ int main() {
   lanes<mg::Proc2, float, mg::CS_SIMT>("lanes_2_mixed");
   lanes<mg::Proc2, float, mg::CS_TC>("lanes_2_tc");
   show<mg::Proc1, float, mg::CS_SIMT, true>("p1_fused");
+  show<mg::Proc4, float, mg::CS_SIMT, false>("p4_simt");
+  show<mg::Proc4, float, mg::CS_TC, false>("p4_tc");
+  show<mg::Proc3, float, mg::CS_SIMT, false>("p3_simt");
+  show<mg::Proc3, float, mg::CS_TC, false>("p3_tc");
   return 0;
 }
 '''
@@ -90,3 +94,13 @@ def test_warps_of_small_groups_hold_one_vertex_type(tmp_path):
                     assert len(held) <= (1 if nu <= 8 else 2), (name, nu, nl, held)
                     checked += 1
     assert checked
+
+
+@pytest.mark.parametrize("name,ctas", [("p4_simt", 1), ("p4_tc", 2), ("p3_simt", 2), ("p3_tc", 3)])
+def test_layouts_fit_the_ctas_they_are_built_for(tmp_path, name, ctas):
+    """Pairs of events in one CTA of 256 threads per SM for gg -> t t~ g g and two for
+    gg -> t t~ g; single events with the tensor-core colour sum in two and three: each
+    layout's own count, not that of the process's other kernel."""
+    nbytes, _, _, built_for = layouts(tmp_path)[name]
+    assert built_for == ctas
+    assert (nbytes + CTA_RESERVED) * ctas <= SM_BYTES, nbytes
