@@ -511,7 +511,7 @@ __device__ __forceinline__ void dot4_acc(cx<R>& J, const W4<R>& x, const W4<R>& 
   else { J.im = -tr; J.re = ti; }
 }
 
-// ---- ordered program (g g -> t t~ g g) ------------------------------------------
+// ---- ordered program (g g -> t t~ g, g g -> t t~ g g) ----------------------------
 // Colour-ordered off-shell currents with the couplings and the factors i taken
 // out: G = -(V3 + V4) / K^2, R = -(sum R G/)(K/ + m) / D, V = (u gamma v) / K^2
 // with prop = i / D (top) or -i / K^2 (gluon), whose imaginary part is -1 / K^2.
@@ -540,15 +540,7 @@ __device__ __forceinline__ W4<R> w4_rscale(const W4<R>& a, R s) {
   for (int k = 0; k < 4; ++k) o.w[k] = s * a.w[k];
   return o;
 }
-// s x + o
-template <class R>
-__device__ __forceinline__ W4<R> w4_axpy(cx<R> s, const W4<R>& x, const W4<R>& o) {
-  W4<R> r;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) r.w[k] = cfma(s, x.w[k], o.w[k]);
-  return r;
-}
-// lower index, sign s
+// lower index
 template <class R>
 __device__ __forceinline__ W4<R> w4_lower(const W4<R>& a) {
   W4<R> o = a;

@@ -82,8 +82,8 @@ struct HsCfg {
   static constexpr int EVMIN = (NT / P::NHEL) > 0 ? (NT / P::NHEL) : 1;  // units, all helicities good
   // room for groups of fewer helicities than all: four times the units with one
   // flow (four of the sixteen helicities of e+e- -> mu+mu- are good); none for the
-  // others, whose shared memory then admits more CTAs per SM (2^20 pairs of
-  // g g -> t t~ events 629 -> 565 us, 50021 FP64 gg -> t t~ g events 2449 -> 2226 us)
+  // others, whose shared memory then admits more CTAs per SM (2^20 g g -> t t~ events
+  // in pairs 629 -> 565 us, 50021 FP64 gg -> t t~ g events 2449 -> 2226 us)
   static constexpr int MORE = P::NCOLOR == 1 ? 4 : 1;
   static constexpr int EVWANT = (MORE * EVMIN) < 32 ? MORE * EVMIN : 32;
   // shared memory for the currents and the contractions' operands
@@ -831,7 +831,7 @@ __device__ __forceinline__ void hs_item(const HsItem& it, const Slots<R, P::HS_N
   cur.set(it.out, o);
 }
 
-// one amputated-current variant (reads the currents, writes the chunk buffer)
+// one amputated-current variant (reads the currents, writes an operand slot)
 template <class P, class R>
 __device__ __forceinline__ void hs_xitem(const HsItem& it, const Slots<R, P::HS_NSLOT>& cur,
                                          const Slots<R, P::HS_XCAP>& xb, const R* K, const Couplings<R>& cp) {

@@ -1668,7 +1668,7 @@ class SharedProgram:
 
 
 # ---------------------------------------------------------------------------
-# Ordered program (g g -> t t~ g g): the colour-flow amplitudes J_s from off-shell
+# Ordered program (g g -> t t~ g, g g -> t t~ g g): the colour-flow amplitudes J_s from off-shell
 # currents that are summed before they are contracted.
 # ---------------------------------------------------------------------------
 # J_s of the chain (T^{a_1} T^{a_2} T^{a_3} T^{a_4})_{top, antitop} is the colour-
