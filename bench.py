@@ -41,11 +41,11 @@ SM_MAX_MHZ = 2070.0
 # (dram__bytes_read.sum + dram__bytes_write.sum of one launch over 2^18 events,
 # scaled by events; it reads the momenta once and writes |M|^2), valid only
 # while the kernel sources are the ones captured.
-SIGMAKIN_TRAFFIC = {"bytes_per_event": 192.5, "sources_sha1": "559d8b2def30a5f38822c7f81b850c585724e5bb"}
+SIGMAKIN_TRAFFIC = {"bytes_per_event": 192.5, "sources_sha1": "4f56e48e9959055c543f5b72a6873acc69b15c12"}
 # Tensor-pipe activity of the tcgen05 colour-sum variant from the same kind of
 # capture (sm__pipe_tensor_cycles_active, fraction of its peak), valid while
 # the kernel sources are the ones captured.
-TC_TENSOR_PIPE = {"frac": 0.0248, "sources_sha1": "559d8b2def30a5f38822c7f81b850c585724e5bb"}
+TC_TENSOR_PIPE = {"frac": 0.0248, "sources_sha1": "4f56e48e9959055c543f5b72a6873acc69b15c12"}
 SIGMAKIN_SOURCES = ["paper_2106_12631_gb300/csrc/" + f for f in
                     ("sigmakin_hs.cuh", "dfl.cuh", "sigmakin_launch.cuh", "sigmakin.cuh", "helas.cuh", "colour_tc.cuh",
                      "mg_types.cuh", "process.cuh", "gen/proc4.cuh")]

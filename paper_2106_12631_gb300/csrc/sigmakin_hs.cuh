@@ -27,8 +27,8 @@
 //      fixed-order FP64 helicity sum.
 // What bounds it (gg -> t t~ g g mixed, 2^20 events): the bytes that the
 // contractions load from shared memory into registers (128 per clock and SM; with
-// the items' loads 59 % of the kernel's cycles) and the latency of dependent FMAs
-// at 8 warps per SM (FMA pipe 49 % busy): 9.9 ms, against 18.0 ms for the
+// the items' loads 60 % of the kernel's cycles) and the latency of dependent FMAs
+// at 8 warps per SM (FMA pipe 49 % busy): 9.8 ms, against 18.0 ms for the
 // diagram-wise program on single events.  In FP64 the FP64 pipe (90 % busy for gg -> t t~ g).
 #pragma once
 #include <type_traits>
@@ -83,7 +83,10 @@ struct HsCfg {
   // room for groups of fewer helicities than all: four times the units with one
   // flow (four of the sixteen helicities of e+e- -> mu+mu- are good); none for the
   // others, whose shared memory then admits more CTAs per SM (2^20 g g -> t t~ events
-  // in pairs 629 -> 565 us, 50021 FP64 gg -> t t~ g events 2449 -> 2226 us)
+  // in pairs 629 -> 565 us, 50021 FP64 gg -> t t~ g events 2449 -> 2226 us).  Masks of
+  // few helicities leave threads idle in the contractions, a small part of these
+  // processes (262144 g g -> t t~ events with 1, 4 and 16 of 16 helicities 131, 134 and
+  // 133 us; with room and single events 141, 146 and 217 us)
   static constexpr int MORE = P::NCOLOR == 1 ? 4 : 1;
   static constexpr int EVWANT = (MORE * EVMIN) < 32 ? MORE * EVMIN : 32;
   // shared memory for the currents and the contractions' operands
